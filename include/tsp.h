@@ -30,7 +30,9 @@
  *  - Error paths can be exercised without a device fault: the environment
  *    variable TSP_SIM_FAULT = oom (device allocations fail: TSP_ENOMEM),
  *    launch (kernel launches fail before anything is enqueued: TSP_ECUDA),
- *    nan_event (each uploaded chunk gets a NaN z_u: TSP_EINVAL) or timeout
+ *    nan_event (each uploaded chunk gets a NaN z_u: TSP_EINVAL), records (the
+ *    window records' buffer cannot be had: no error, the passes then set each
+ *    window's rows up themselves) or timeout
  *    (tsp_wait gives up at once: TSP_ETIMEOUT) simulates that
  *    failure at every site it reaches while it is set.  A context whose call
  *    failed this way can still be destroyed, and new contexts work once the

@@ -121,7 +121,7 @@ int plan(tsp_ctx* c)
     tl.RS = RS;
     tl.RW = RS;
     tl.TZ = RS - 2 * tl.HZ;
-    const size_t budget = 216 * 1024;
+    const size_t budget = 224 * 1024;
     auto fits = [&](int ty) {
         return tiles_region_fits(ty + 2 * tl.HY, RS) &&
                tiles_smem_floats(ty + 2 * tl.HY, RS) * sizeof(float) <= budget;
@@ -217,6 +217,12 @@ int refresh_rhop(tsp_ctx* c, cudaStream_t st)
     return TSP_OK;
 }
 
+double grad_unit(const tsp_ctx* c)
+{
+    const double w = (double)c->counters_h[3];     // in-window pixels of the list
+    return (double)c->n * std::max(1.0, w > 0.0 ? 64.0 * c->npix / w : 1.0);
+}
+
 PassArgs pass_args(tsp_ctx* c)
 {
     PassArgs a;
@@ -225,6 +231,8 @@ PassArgs pass_args(tsp_ctx* c)
     a.evs.geo = c->geo;
     a.evs.geo64 = c->geo64;
     a.evs.rows = c->rows;
+    a.evs.recs = c->rec ? c->recs : nullptr;
+    a.evs.evc = c->rec ? c->evc : nullptr;
     a.items = c->items;
     a.n_items = c->n_items;
     a.outlier_first = (int)c->outlier_first;
@@ -232,6 +240,7 @@ PassArgs pass_args(tsp_ctx* c)
     a.rhop = c->rhop;
     a.A = c->A;
     a.accum = c->accum;
+    a.grad_unit = grad_unit(c);
     a.G = c->G;
     a.nseg = c->nseg;
     a.gld = c->gld;
@@ -267,6 +276,51 @@ int prep_chunk(tsp_ctx* c, long long first, long long n, cudaStream_t st)
                              c->geo_u + first, c->geo64_u + first, c->rows_u + first,
                              c->key + first, c->counters, c->bin_count, c->nbins, st));
     c->launches += 1;
+    return TSP_OK;
+}
+
+// Window records of the placed events.  They are kept when they take at most a
+// quarter of the memory that is free when their buffer has to grow (6e7 events
+// at 1 mm on an empty 280 GB); otherwise, or when the allocation fails, the
+// passes set the rows up themselves.
+int build_records(tsp_ctx* c, cudaStream_t st)
+{
+    c->rec = false;
+    const long long placed = c->outlier_first;
+    if (c->gld || c->n_items == 0 || placed == 0) return TSP_OK;
+    const size_t per = record_bytes(c->G);
+    const size_t need = (per + kEvcBytes) * (size_t)placed;
+    if (sim_fault() == kSimRecords) return TSP_OK;
+    if (need > c->rec_cap) {
+        dfree(c->recbuf);
+        c->rec_cap = 0;
+        size_t avail = 0, total = 0;
+        if (cudaMemGetInfo(&avail, &total) != cudaSuccess || need > avail / 4 ||
+            dmalloc(&c->recbuf, need) != cudaSuccess) {
+            cudaGetLastError();
+            c->recbuf = nullptr;
+            return TSP_OK;
+        }
+        c->rec_cap = need;
+    }
+    c->recs = reinterpret_cast<uint2*>(c->recbuf);
+    c->evc = reinterpret_cast<float4*>(c->recbuf + per * (size_t)placed);
+    RecArgs a;
+    a.g = c->g;
+    a.tl = c->tl;
+    a.evs = EventsView{c->geo, c->geo64, c->rows, nullptr, nullptr};
+    a.accum = c->accum;
+    a.items = c->items;
+    a.n_items = c->n_items;
+    a.G = c->G;
+    a.nseg = c->nseg;
+    a.sms = c->num_sms;
+    a.recs = c->recs;
+    a.evc = c->evc;
+    TSP_CUDA(c, cudaMemsetAsync(&c->accum->rec_qclip, 0, 2 * sizeof(unsigned long long), st));
+    TSP_CUDA(c, launch_records(c->lmax, a, st));
+    c->launches += 1;
+    c->rec = true;
     return TSP_OK;
 }
 
@@ -314,6 +368,7 @@ int prep_finish(tsp_ctx* c, cudaStream_t st)
                                c->cursor, c->geo, c->geo64, c->rows, st));
     c->launches += n > 0 ? 1 : 0;
     clear_graphs(c);
+    if (int rc = build_records(c, st)) return rc;
     c->uploaded = true;
     return TSP_OK;
 }
@@ -514,6 +569,7 @@ void tsp_destroy(tsp_ctx* c)
     dfree(c->zu); dfree(c->zd); dfree(c->dl);
     dfree(c->geo_u); dfree(c->geo); dfree(c->geo64_u); dfree(c->geo64);
     dfree(c->rows_u); dfree(c->rows); dfree(c->key);
+    dfree(c->recbuf);
     dfree(c->items); dfree(c->bin_count); dfree(c->offsets); dfree(c->cursor);
     delete c;
 }

@@ -26,6 +26,7 @@ using namespace tsp_host;
 struct BatchClass {
     int lmax = 0, nseg = 1;
     bool kz = false;           // some member has a z-dependent sigma_z
+    bool rec = false;          // the members have window records
     size_t smem = 0;
     double work = 0.0;         // estimated pass work (events x window pixels)
     int4* items = nullptr;
@@ -33,7 +34,8 @@ struct BatchClass {
     int n_items = 0, n_oitems = 0, items_cap = 0, oitems_cap = 0;
 };
 
-constexpr int kMaxClasses = 2 * kLmaxCount;
+// (with and without window records)
+constexpr int kMaxClasses = 4 * kLmaxCount;
 
 struct tsp_batch {
     std::vector<tsp_ctx*> inst;
@@ -138,14 +140,19 @@ int rebuild(tsp_batch* b, cudaStream_t st)
     // kernel class of every reconstruction: its own lane capacity and row split
     int n_cls = 0;
     int cls_lmax[kMaxClasses], cls_nseg[kMaxClasses];
+    bool cls_rec[kMaxClasses];
     std::vector<int> cls_of(k);
     for (int i = 0; i < k; ++i) {
         tsp_ctx* c = b->inst[i];
         int q = 0;
-        while (q < n_cls && !(cls_lmax[q] == c->lmax && cls_nseg[q] == c->nseg)) ++q;
+        // (a member without tile items joins either form of its class)
+        while (q < n_cls && !(cls_lmax[q] == c->lmax && cls_nseg[q] == c->nseg &&
+                              (cls_rec[q] == c->rec || c->gld || c->n_items == 0)))
+            ++q;
         if (q == n_cls) {
             cls_lmax[q] = c->lmax;
             cls_nseg[q] = c->nseg;
+            cls_rec[q] = c->rec;
             ++n_cls;
         }
         cls_of[i] = q;
@@ -156,10 +163,13 @@ int rebuild(tsp_batch* b, cudaStream_t st)
         t.evs.geo = c->geo;
         t.evs.geo64 = c->geo64;
         t.evs.rows = c->rows;
+        t.evs.recs = c->recs;
+        t.evs.evc = c->evc;
         t.rhop = c->rhop;
         t.A = c->A;
         t.accum = c->accum;
         t.G = c->G;
+        t.grad_unit = grad_unit(c);
         BatchImg& m = imgs[i];
         m.rho = c->rho;
         m.rhop = c->rhop;
@@ -180,6 +190,7 @@ int rebuild(tsp_batch* b, cudaStream_t st)
         BatchClass& bc = b->cls[q];
         bc.lmax = cls_lmax[q];
         bc.nseg = cls_nseg[q];
+        bc.rec = cls_rec[q];
         bc.kz = false;
         bc.smem = 0;
         bc.work = 0.0;
@@ -288,6 +299,7 @@ BatchArgs batch_args(const tsp_batch* b, int q)
     a.queue = b->queue + q;
     a.nseg = bc.nseg;
     a.kz = bc.kz ? 1 : 0;
+    a.rec = bc.rec ? 1 : 0;
     a.grid = b->num_sms;
     a.smem = bc.smem;
     return a;

@@ -59,6 +59,13 @@ struct tsp_ctx {
     tsp::Ev64 *geo64_u = nullptr, *geo64 = nullptr;
     int2 *rows_u = nullptr, *rows = nullptr;
     int* key = nullptr;
+    // window records of the binned events (tsp_rec.cuh); rec: those of the
+    // current upload are there
+    unsigned char* recbuf = nullptr;
+    size_t rec_cap = 0;               // bytes of recbuf
+    uint2* recs = nullptr;
+    float4* evc = nullptr;
+    bool rec = false;
     int4* items = nullptr;
     int n_items = 0, items_cap = 0;
     std::vector<int> bin_cnt;          // events per bin (host copy; last = outliers)
@@ -143,6 +150,8 @@ std::vector<int4> tile_items(const tsp_ctx* c, long long E, int w);
 long long item_events(long long placed, int items_per_sm, int sms);
 int ensure_sensitivity(tsp_ctx* c, cudaStream_t st);
 int refresh_rhop(tsp_ctx* c, cudaStream_t st);
+// The gradient pass's fixed-point unit times sum rho' (Inst::grad_unit).
+double grad_unit(const tsp_ctx* c);
 void clear_graphs(tsp_ctx* c);
 
 }  // namespace tsp_host

@@ -183,12 +183,18 @@ constexpr int kAccWords = 18432;
 // Shared-memory layout of the tile kernel, in 32-bit words: kPadFloats slack,
 // the rho' region (RH*RS), 2*kPadFloats slack, the accumulator's H region
 // (RH*RS; the float accumulator of the other passes), its L region at
-// kAccWords words from the H region, kPadFloats slack, then the groups'
-// reduction slots (warps/G groups x 2 parities x 3G floats <= 6*kMaxWarps).
+// kAccWords words from the H region, kPadFloats slack, and kPartFloats for the
+// groups' reduction slots (first in the passes over window records, which read
+// them as float4; last in the others, which use half of them: warps/G groups x
+// 2 parities x 3G floats).
+constexpr int kPartFloats = 12 * kMaxWarps;
+// Shared staging of a warp's next window records (256 bytes) and of its event's
+// coefficients (64), in floats (tsp_rec.cuh).
+constexpr int kRecSlotFloats = 80;
 __host__ __device__ constexpr size_t tiles_smem_floats(int RH, int RS)
 {
     return (size_t)kPadFloats + (size_t)RH * RS + 2 * kPadFloats + (size_t)kAccWords +
-           (size_t)RH * RS + kPadFloats + 6 * kMaxWarps;
+           (size_t)RH * RS + kPadFloats + kPartFloats + kMaxWarps * kRecSlotFloats;
 }
 
 // A staged region fits the two-word accumulator layout.
@@ -218,6 +224,9 @@ struct Accum {
     double sum_rhop;             // sum_i s_i rho_i
     int queue;                   // persistent-kernel work counter
     int pad1[3];
+    // pixels that the window records leave out (k_records, once per upload;
+    // kept between passes): as n_qclip and n_lclip
+    unsigned long long rec_qclip, rec_lclip;
 };
 
 // Bounds checks of a TSP_DEBUG_CHECKS build (a substitute for a memory checker):
@@ -265,6 +274,10 @@ struct EventsView {
     const float4* __restrict__ geo;    // (yt, zt, t, c2i) per event, rounded from geo64
     const Ev64* __restrict__ geo64; // (yt, zt, t, c2i) in double precision
     const int2* __restrict__ rows;     // (first row, row count) of the non-empty chords
+    // window records of the binned events and the events' coefficients
+    // (tsp_rec.cuh), or null: the passes then set each row up themselves
+    const uint2* __restrict__ recs;
+    const float4* __restrict__ evc;
 };
 
 // One reconstruction as the tile kernel reads it: its constants, tiling,
@@ -279,6 +292,7 @@ struct Inst {
     const float* rhop;
     float* A;
     Accum* accum;
+    double grad_unit;   // N max(1, 64 npix / W): the gradient pass's unit times sum rho'
     int G;
     int pad;
 };

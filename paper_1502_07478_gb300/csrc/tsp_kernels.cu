@@ -431,6 +431,7 @@ int sim_fault()
     if (!std::strcmp(v, "launch")) return kSimLaunch;
     if (!std::strcmp(v, "nan_event")) return kSimNan;
     if (!std::strcmp(v, "timeout")) return kSimTimeout;
+    if (!std::strcmp(v, "records")) return kSimRecords;
     return kSimNone;
 }
 
@@ -579,6 +580,18 @@ cudaError_t launch_pass(int lmax, int mode, const PassArgs& a, cudaStream_t st)
     case 24: return launch_pass_l<24>(mode, a, st);
     case 48: return launch_pass_l<48>(mode, a, st);
     case 64: return launch_pass_l<64>(mode, a, st);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t launch_records(int lmax, const RecArgs& a, cudaStream_t st)
+{
+    if (cudaError_t f = sim_launch()) return f;
+    switch (lmax) {
+    case 12: return launch_records_l<12>(a, st);
+    case 24: return launch_records_l<24>(a, st);
+    case 48: return launch_records_l<48>(a, st);
+    case 64: return launch_records_l<64>(a, st);
     default: return cudaErrorInvalidValue;
     }
 }

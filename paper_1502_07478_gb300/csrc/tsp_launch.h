@@ -25,10 +25,12 @@ bool cinv_valid(const tsp_params& p);
 //              cudaErrorLaunchOutOfResources (TSP_ECUDA)
 //   nan_event  every uploaded chunk gets a NaN in its first z_u after the copy
 //              (the event preparation rejects the upload: TSP_EINVAL)
+//   records    the window records' buffer cannot be had (no error: the passes
+//              set the rows up themselves)
 //   timeout    the bounded wait (tsp_wait) gives up at once, as when the
 //              enqueued work outlasts the limit (TSP_ETIMEOUT)
 // Unset or any other value: no fault.
-enum SimFault : int { kSimNone = 0, kSimOom = 1, kSimLaunch = 2, kSimNan = 3, kSimTimeout = 4 };
+enum SimFault : int { kSimNone = 0, kSimOom = 1, kSimLaunch = 2, kSimNan = 3, kSimTimeout = 4, kSimRecords = 5 };
 int sim_fault();
 
 // The error a launch helper returns under TSP_SIM_FAULT=launch, else success.
@@ -106,11 +108,30 @@ struct PassArgs {
     const float* rhop;
     float* A;
     Accum* accum;
+    double grad_unit;  // see Inst
     int G, nseg;
     int gld;           // tiles stage only A; rho' read from global (nseg = 2)
     int grid;          // persistent blocks
     size_t smem;       // dynamic shared memory of the tile kernel
 };
+
+// Window records of a list's binned events (tsp_rec.cuh): written once per
+// upload by launch_records, over the plain tile items.
+struct RecArgs {
+    Geo g;
+    Tiling tl;
+    EventsView evs;      // recs / evc not used
+    Accum* accum;        // rec_qclip, rec_lclip are added to
+    const int4* items;
+    int n_items;
+    int G, nseg;
+    int sms;
+    uint2* recs;
+    float4* evc;
+};
+// Bytes of one event's records: 8 a lane, and its coefficients.
+constexpr size_t kEvcBytes = 4 * sizeof(float4);
+inline size_t record_bytes(int G) { return (size_t)G * 32 * sizeof(uint2); }
 
 // A batched pass: the tile items (bin, first, count, reconstruction) of every
 // reconstruction in `table`, in one persistent launch, and the outlier items
@@ -124,6 +145,7 @@ struct BatchArgs {
     int* queue;        // work counter, zeroed before the launch
     int nseg;
     int kz;            // some reconstruction has a z-dependent sigma_z
+    int rec;           // every reconstruction has window records
     int grid;
     size_t smem;
 };
@@ -159,6 +181,10 @@ template <int LMAX>
 cudaError_t launch_batch_pass_l(int mode, const BatchArgs& a, cudaStream_t st);
 template <int LMAX>
 cudaError_t prepare_batch_pass_l(size_t smem);
+template <int LMAX>
+cudaError_t launch_records_l(const RecArgs& a, cudaStream_t st);
+// Write the window records of a list.
+cudaError_t launch_records(int lmax, const RecArgs& a, cudaStream_t st);
 
 // Auxiliary kernels (tsp_kernels.cu).
 cudaError_t launch_sensitivity(double R, double L, int ny, int nz, double dy, double dz, float* s,

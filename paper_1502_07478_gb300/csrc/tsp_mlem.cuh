@@ -110,40 +110,52 @@ __device__ __forceinline__ void row_idle(RowK<SMEM>& r, RowG& rg)
     }
 }
 
-// Row constants of lane row iy (valid_row = false for a lane without a row)
-// for the traversal TRAV.  All 32 lanes of the warp must call it together: the
+// A lane's share of an event's window: the chord of its row inside the frame
+// and the traversal of it.  With has = false the lane has no pixels.  o is the
+// image column the traversal starts at, sidx the stored index of that pixel
+// (an in-bounds index in any case), gidx the flat image index of an idle lane.
+struct RowSpan {
+    Chord c;
+    float Qc, gam2;        // Q(u) = Qc + gam2 u along the chord
+    bool has;
+    int o, lim_odd, lim_even;
+    long long sidx, gidx;
+};
+
+// Span of lane row iy (valid_row = false for a lane without a row) for the
+// traversal TRAV.  All 32 lanes of the warp must call it together: the
 // lanes agree on one stored column (the middle of their chord centres) as
 // their common traversal origin, so that at every step neighbouring lanes
 // (neighbouring rows, row stride = 1 mod 32 words) address distinct banks.  A
 // lane whose chord does not contain that column starts at its own centre.
 // The event preparation guarantees that every chord lies inside the frame;
 // the clamp keeps every access in bounds regardless (clipped pixels are
-// counted).
-template <int TRAV, int LMAX, bool GRAD, bool SMEM, bool GLD>
-__device__ __forceinline__ void make_row(const Geo& g, const EvSig& es, const float4& ev,
-                                         const Ev64* ev64, int iy, bool valid_row, int evflags,
-                                         const Frame* fp,
-                                         const float* base, const float* gimg, RowK<SMEM>& r,
-                                         RowG& rg, BlockSums* bs)
+// counted in lclip, pixels with Q <= 0 in qclip).
+template <int TRAV, int LMAX, bool SMEM>
+__device__ __forceinline__ RowSpan row_span(const Geo& g, const EvSig& es, const float4& ev,
+                                            const Ev64* ev64, int iy, bool valid_row, int evflags,
+                                            const Frame& f, unsigned long long* qclip,
+                                            unsigned long long* lclip)
 {
-    row_idle<GRAD, SMEM>(r, rg);
-    Chord c;
+    RowSpan r;
+    Chord& c = r.c;
     c.y = c.Dy = c.B0 = c.zc = 0.0f;
+    r.o = r.lim_odd = r.lim_even = 0;
+    r.gidx = 0;
     int lo = 0, hi = -1, z0row = 0;
-    const Frame f = *fp;
     float Qc = 0.0f, gam2 = 0.0f;
     if (valid_row) {
         c = row_chord(g, es, ev, ev64, iy, !(evflags & kEvExact));
         lo = c.lo;
         hi = c.lo + c.count - 1;
         if (c.count > 0 && (iy < f.oy || iy >= f.oy + f.rh)) {
-            atomicAdd(&bs->lclip, (unsigned long long)c.count);
+            atomicAdd(lclip, (unsigned long long)c.count);
             hi = lo - 1;
         }
         z0row = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0)));
         if (hi >= lo && (lo < z0row || hi >= z0row + f.rw)) {
             const int lo2 = max(lo, z0row), hi2 = min(hi, z0row + f.rw - 1);
-            atomicAdd(&bs->lclip, (unsigned long long)(c.count - max(hi2 - lo2 + 1, 0)));
+            atomicAdd(lclip, (unsigned long long)(c.count - max(hi2 - lo2 + 1, 0)));
             lo = lo2;
             hi = hi2;
         }
@@ -169,17 +181,19 @@ __device__ __forceinline__ void make_row(const Geo& g, const EvSig& es, const fl
                 mlo = max(mlo, 0);
                 mhi = min(mhi, n0 - 1);
                 const int keep = max(mhi - mlo + 1, 0);
-                atomicAdd(&bs->qclip, (unsigned long long)(n0 - keep));
+                atomicAdd(qclip, (unsigned long long)(n0 - keep));
                 hi = lo + mhi;
                 lo = lo + mlo;
             }
         }
     }
-    const bool has = hi >= lo;
+    r.Qc = Qc;
+    r.gam2 = gam2;
+    r.has = hi >= lo;
     const int sc = ((lo + hi) >> 1) - z0row;               // stored column of the centre
-    const int smin = __reduce_min_sync(0xffffffffu, has ? sc : 0x7fffffff);
-    const int smax = __reduce_max_sync(0xffffffffu, has ? sc : (int)0x80000000);
-    if (!has) {
+    const int smin = __reduce_min_sync(0xffffffffu, r.has ? sc : 0x7fffffff);
+    const int smax = __reduce_max_sync(0xffffffffu, r.has ? sc : (int)0x80000000);
+    if (!r.has) {
         // A lane without pixels still gets an in-bounds address, in its own
         // (virtual) row at the warp's common column: the packed passes run it
         // through their unpredicated pairs with P = 0, and its own row keeps
@@ -192,21 +206,12 @@ __device__ __forceinline__ void make_row(const Geo& g, const EvSig& es, const fl
                             f.rw - 1);
         const long long lo_i = LMAX / 2;
         const long long hi_i = (long long)g.ny * g.nz + kPadFloats - LMAX / 2 - 1;
-        long long sidx = (long long)vr * f.stride + col;
-        if constexpr (SMEM) {
-            r.base = (unsigned)__cvta_generic_to_shared(base) + 4u * (unsigned)sidx;
-        } else {
-            sidx = min(max(sidx, lo_i), hi_i);
-            r.base = (unsigned long long)(base + sidx);
-        }
-        if constexpr (GLD) {
-            const int iyv = min(max(f.oy + vr, 0), g.ny - 1);
-            const int zv = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(f.oy + vr - f.Y0)));
-            const long long gi = min(max((long long)iyv * g.nz + min(max(zv + col, 0), g.nz - 1),
-                                         lo_i), hi_i);
-            r.gbase = (unsigned long long)(gimg + gi);
-        }
-        return;
+        r.sidx = (long long)vr * f.stride + col;
+        if constexpr (!SMEM) r.sidx = min(max(r.sidx, lo_i), hi_i);
+        const int iyv = min(max(f.oy + vr, 0), g.ny - 1);
+        const int zv = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(f.oy + vr - f.Y0)));
+        r.gidx = min(max((long long)iyv * g.nz + min(max(zv + col, 0), g.nz - 1), lo_i), hi_i);
+        return r;
     }
     // The common origin is used only when it lies within 2 columns of the
     // lane's own chord centre cc and keeps the lane's walk within LMAX steps;
@@ -228,16 +233,42 @@ __device__ __forceinline__ void make_row(const Geo& g, const EvSig& es, const fl
     } else {
         r.lim_odd = r.lim_even = L;
     }
+    r.o = o;
+    r.sidx = (iy - f.oy) * f.stride + (o - z0row);
+    return r;
+}
+
+// Row constants of lane row iy for the traversal TRAV (all lanes of the warp
+// together; see row_span).
+template <int TRAV, int LMAX, bool GRAD, bool SMEM, bool GLD>
+__device__ __forceinline__ void make_row(const Geo& g, const EvSig& es, const float4& ev,
+                                         const Ev64* ev64, int iy, bool valid_row, int evflags,
+                                         const Frame* fp,
+                                         const float* base, const float* gimg, RowK<SMEM>& r,
+                                         RowG& rg, BlockSums* bs)
+{
+    row_idle<GRAD, SMEM>(r, rg);
+    const Frame f = *fp;
+    const RowSpan sp = row_span<TRAV, LMAX, SMEM>(g, es, ev, ev64, iy, valid_row, evflags, f,
+                                                  &bs->qclip, &bs->lclip);
+    const Chord& c = sp.c;
+    if constexpr (SMEM)
+        r.base = (unsigned)__cvta_generic_to_shared(base) + 4u * (unsigned)sp.sidx;
+    else
+        r.base = (unsigned long long)(base + sp.sidx);
+    if (!sp.has) {
+        if constexpr (GLD) r.gbase = (unsigned long long)(gimg + sp.gidx);
+        return;
+    }
+    const int o = sp.o;
+    const float Qc = sp.Qc, gam2 = sp.gam2;
+    if constexpr (GLD) r.gbase = (unsigned long long)(gimg + (size_t)iy * g.nz + o);
+    r.lim_odd = sp.lim_odd;
+    r.lim_even = sp.lim_even;
     const float t = ev.z, c2i = ev.w, y = c.y, Dy = c.Dy;
     float alpha, beta;
     row_acb(g, es, ev, c, alpha, beta);
     const float u0 = fmaf((float)o, g.dz, g.z0) - c.zc;
-    const int sidx = (iy - f.oy) * f.stride + (o - z0row);
-    if constexpr (SMEM)
-        r.base = (unsigned)__cvta_generic_to_shared(base) + 4u * (unsigned)sidx;
-    else
-        r.base = (unsigned long long)(base + sidx);
-    if constexpr (GLD) r.gbase = (unsigned long long)(gimg + (size_t)iy * g.nz + o);
     r.Q0 = fmaf(gam2, u0, Qc);
     r.dQ = gam2 * g.dz;
     r.A0 = g.kA * fmaf(alpha, u0, beta);

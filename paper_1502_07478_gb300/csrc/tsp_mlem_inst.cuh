@@ -3,6 +3,7 @@
 // row (nseg = 1) and for two lanes per row (nseg = 2).
 #include "tsp_launch.h"
 #include "tsp_mlem.cuh"
+#include "tsp_rec.cuh"
 
 #ifndef TSP_LMAX
 #error "define TSP_LMAX before including this file"
@@ -24,8 +25,19 @@ cudaError_t run_pass(const PassArgs& a, cudaStream_t st)
         p.A = a.A;
         p.accum = a.accum;
         p.G = a.G;
+        p.grad_unit = a.grad_unit;
         p.pad = 0;
-        if (a.g.kz != 0.0f)
+        bool done = false;
+        if constexpr (!GLD) {
+            if (a.evs.recs) {
+                k_tiles_rec<LMAX, MODE, NSEG, false>
+                    <<<a.grid, pass_threads(LMAX, MODE, NSEG, false), a.smem, st>>>(
+                    p, nullptr, a.items, a.n_items, &a.accum->queue);
+                done = true;
+            }
+        }
+        if (done) {
+        } else if (a.g.kz != 0.0f)
             k_tiles<LMAX, MODE, NSEG, false, GLD, true>
                 <<<a.grid, pass_threads(LMAX, MODE, NSEG, false), a.smem, st>>>(
                 p, nullptr, a.items, a.n_items, &a.accum->queue);
@@ -55,6 +67,9 @@ template <int LMAX, int MODE, int NSEG>
 cudaError_t set_smem(size_t smem)
 {
     cudaError_t e = set_smem_one<LMAX, MODE, NSEG, false, false>(smem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_tiles_rec<LMAX, MODE, NSEG, false>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = set_smem_one<LMAX, MODE, NSEG, false, true>(smem);
     if constexpr (NSEG == 2) {
         if (e == cudaSuccess) e = set_smem_one<LMAX, MODE, NSEG, true, false>(smem);
@@ -70,7 +85,11 @@ cudaError_t run_batch(const BatchArgs& a, cudaStream_t st)
 {
     Inst none{};
     if (a.n_items > 0) {
-        if (a.kz)
+        if (a.rec)
+            k_tiles_rec<LMAX, MODE, NSEG, true>
+                <<<a.grid, pass_threads(LMAX, MODE, NSEG, true), a.smem, st>>>(
+                    none, a.table, a.items, a.n_items, a.queue);
+        else if (a.kz)
             k_tiles<LMAX, MODE, NSEG, true, false, true>
                 <<<a.grid, pass_threads(LMAX, MODE, NSEG, true), a.smem, st>>>(
                     none, a.table, a.items, a.n_items, a.queue);
@@ -105,6 +124,10 @@ cudaError_t batch_smem(size_t smem)
     cudaError_t e = cudaFuncSetAttribute(k_tiles<LMAX, kMlem, NSEG, true, false, false>, at, v);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_tiles<LMAX, kMlem, NSEG, true, false, true>, at, v);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_tiles_rec<LMAX, kMlem, NSEG, true>, at, v);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_tiles_rec<LMAX, kGrad, NSEG, true>, at, v);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_tiles<LMAX, kGrad, NSEG, true, false, false>, at, v);
     if (e == cudaSuccess)
@@ -163,6 +186,27 @@ cudaError_t launch_batch_pass_l<TSP_LMAX>(int mode, const BatchArgs& a, cudaStre
 {
     return a.nseg == 1 ? run_batch_mode<TSP_LMAX, 1>(mode, a, st)
                        : run_batch_mode<TSP_LMAX, 2>(mode, a, st);
+}
+
+template <>
+cudaError_t launch_records_l<TSP_LMAX>(const RecArgs& a, cudaStream_t st)
+{
+    if (a.n_items <= 0) return cudaSuccess;
+    Inst p{};
+    p.g = a.g;
+    p.tl = a.tl;
+    p.evs = a.evs;
+    p.accum = a.accum;
+    p.G = a.G;
+    // some eight blocks an SM: several per item when the list is short
+    const int want = 8 * a.sms;
+    const dim3 grid(a.n_items < 4 * want ? a.n_items : 4 * want,
+                    a.n_items < want ? (want + a.n_items - 1) / a.n_items : 1);
+    if (a.nseg == 1)
+        k_records<TSP_LMAX, 1><<<grid, 256, 0, st>>>(p, a.items, a.n_items, a.recs, a.evc);
+    else
+        k_records<TSP_LMAX, 2><<<grid, 256, 0, st>>>(p, a.items, a.n_items, a.recs, a.evc);
+    return cudaGetLastError();
 }
 
 template <>

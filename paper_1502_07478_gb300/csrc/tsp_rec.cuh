@@ -1,0 +1,767 @@
+// The tile passes over window records.
+//
+// What a lane needs to know of its row of an event's window -- which pixels,
+// from which stored column, at which offset u from the chord centre -- depends
+// on the event, the grid and the tiling only, not on the image.  k_records
+// works it out once per upload (row_span, the same decision as the passes of
+// tsp_mlem.cuh take) and stores it: 8 bytes a lane,
+//   x = u at the lane's traversal origin (float bits),
+//   y = stored index of that pixel in the tile region (16 bits),
+//       pairs on the chord of the first / second pixel stream (8 bits each),
+// and 64 bytes an event of polynomial coefficients (EvC), so that the passes
+// form a row's constants in about twenty multiply-adds.
+//
+// Why: with the row setup in the pass, 2.5e9 of the 4.3e9 warp instructions of
+// a 1e6-event 1 mm pass (58%) were outside the pixel loops' arithmetic and
+// memory operations, and issue slots bound the pass.  The records are read once
+// per pass at 32 G lanes x 8 bytes an event (1 KB at 1 mm, 512 B at 2 mm, 256 B
+// at 4 mm), 10 GB a pass for 1e7 events at 1 mm, copied to shared memory an
+// event ahead.  MLEM passes: 1e7 events at 1 mm 42.9 -> 34.4 ms, 1e7 at 4 mm
+// 6.22 -> 3.53 ms, 1e6 at 2 mm 2.28 -> 1.66 ms.  Writing them costs an upload
+// about as much as one pass's row setup did (1.3 ms per 1e6 events at 1 mm).
+#pragma once
+
+#include "tsp_mlem.cuh"
+
+namespace tsp {
+
+// Coefficients of an event's row constants as polynomials in y and Dy = y - y~:
+//   Q(u) = q0 + y (q1 + q2 y) + g1 y u,    aCb = a1 y u + Dy (b1 y + b2),
+//   C0 = log2K - hB Dy^2,   ksu = sqrt(log2(e) iz) of the event,
+// stored as float4 (y~, mid, q0, q1), (q2, g1, a1, b1), (b2, hB, log2K, ksu) and
+// the event's geometry (y~, z~, t, c2i), which the gradient pass needs;
+// mid is the middle row of the window (lane rows count outward from it).
+constexpr int kEvcFloat4 = 4;
+
+__device__ __forceinline__ void make_evc(const Geo& g, const EvSig& es, const float4& ev, int mid,
+                                         float4* __restrict__ out)
+{
+    const float yt = ev.x, t = ev.z, c2i = ev.w;
+    const float il4 = 4.0f * g.il * c2i, iz2 = 2.0f * es.iz * c2i;
+    const float cross = il4 * fmaf(2.0f * t, t, 1.0f);
+    float q0 = iz2 * c2i * g.R * g.R;
+    float q1 = -cross * yt;
+    const float q2 = iz2 * c2i + il4 * t * t + cross;
+    float b2 = 0.0f;
+    if (g.gR8 != 0.0f) {
+        const float sec = sqrtf(c2i), r = g.gR8 * t * c2i * sec;
+        q0 = fmaf(r, yt, q0);
+        q1 -= 2.0f * r;
+        b2 = -g.gR4 * c2i * sec;
+    }
+    out[0] = make_float4(yt, (float)mid, q0, q1);
+    out[1] = make_float4(q2, -2.0f * iz2 * t, -iz2, il4 * t);
+    out[2] = make_float4(b2, g.half_log2e * il4, es.log2K, es.ksu);
+    out[3] = ev;
+}
+
+// Lane rows count outward from the middle of the window (see event_rows).
+__device__ __forceinline__ int lane_row(int rowi)
+{
+    return (rowi & 1) ? (rowi >> 1) + 1 : -(rowi >> 1);
+}
+
+// Records of the events of the plain items.  One warp per (event, 32-lane
+// block); item blocks of one warp count each so that short lists still spread.
+template <int LMAX, int NSEG>
+__global__ void __launch_bounds__(256)
+k_records(Inst p, const int4* __restrict__ items, int n_items, uint2* __restrict__ recs,
+          float4* __restrict__ evc)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const Geo& g = p.g;
+    const int G = p.G;
+    for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
+        const int4 item = items[it];
+        const Frame f = tile_frame(g, p.tl, item.x);
+        const int tasks = item.z * G;
+        for (int k = warp + 8 * blockIdx.y; k < tasks; k += 8 * gridDim.y) {
+            const int j = k / G, blk = k - j * G, e = item.y + j;
+            const float4 ev = p.evs.geo[e];
+            int2 rws = p.evs.rows[e];
+            const int evflags = rws.y & ~kEvRowsMask;
+            rws.y &= kEvRowsMask;
+            const EvSig es = ev_sig(g, ev);
+            const int mid = (rws.y - 1) >> 1;
+            const int rowi = (NSEG == 1 ? blk : blk >> 1) * 32 + lane;
+            const int ri = mid + lane_row(rowi);
+            const bool valid = ri >= 0 && ri < rws.y;
+            unsigned long long* qc = &p.accum->rec_qclip;
+            unsigned long long* lc = &p.accum->rec_lclip;
+            RowSpan sp;
+            if constexpr (NSEG == 1)
+                sp = row_span<kAlt, LMAX, true>(g, es, ev, p.evs.geo64 + e, rws.x + ri, valid,
+                                                evflags, f, qc, lc);
+            else if ((blk & 1) == 0)
+                sp = row_span<kPos, LMAX, true>(g, es, ev, p.evs.geo64 + e, rws.x + ri, valid,
+                                                evflags, f, qc, lc);
+            else
+                sp = row_span<kNeg, LMAX, true>(g, es, ev, p.evs.geo64 + e, rws.x + ri, valid,
+                                                evflags, f, qc, lc);
+            int la, lb;
+            if constexpr (NSEG == 1) {
+                la = sp.lim_odd >> 1;
+                lb = (sp.lim_even + 1) >> 1;
+            } else {
+                la = (sp.lim_odd + 1) >> 1;
+                lb = sp.lim_odd >> 1;
+            }
+            const float u0 = sp.has ? fmaf((float)sp.o, g.dz, g.z0) - sp.c.zc : 0.0f;
+            recs[((size_t)e * G + blk) * 32 + lane] =
+                make_uint2(__float_as_uint(u0), (unsigned)sp.sidx | (unsigned)la << 16 |
+                                                    (unsigned)lb << 24);
+            if (blk == 0 && lane == 0) make_evc(g, es, ev, rws.x + mid, evc + (size_t)e * kEvcFloat4);
+        }
+    }
+}
+
+// A warp's staging slot in shared memory: its lanes' records, then the event's
+// coefficients.  The next event's are copied (cp.async) while this one is
+// evaluated, so that their latency stays behind a whole event without holding
+// registers (fourteen, which the pixel loops of the 64-register kernels would
+// spill).
+__device__ __forceinline__ void rec_fetch(unsigned slot, const uint2* rp, const float4* ep, int lane)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(slot + 8u * lane), "l"(rp)
+                 : "memory");
+    if (lane < kEvcFloat4)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(slot + 256u + 16u * lane),
+                     "l"(ep + lane)
+                     : "memory");
+}
+
+__device__ __forceinline__ void rec_wait()
+{
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+}
+
+__device__ __forceinline__ float4 lds128(unsigned a)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+    return v;
+}
+
+// An event's coefficients and a lane's record.
+struct RecIn {
+    uint2 r;
+    float4 a, b, c;
+};
+
+__device__ __forceinline__ void rec_take(RecIn& x, unsigned slot, int lane)
+{
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];"
+                 : "=r"(x.r.x), "=r"(x.r.y) : "r"(slot + 8u * lane) : "memory");
+    x.a = lds128(slot + 256u);
+    x.b = lds128(slot + 272u);
+    x.c = lds128(slot + 288u);
+}
+
+// aCb along a row, for the gradient pass: B0 + d dB.
+struct GradC {
+    float2 B0, dB;
+};
+
+// The row's constants, as pairs, from the event's coefficients (rowoff: lane
+// row, counted from the window's middle).  GRAD: e0, e1, e2 hold C0, s at the
+// origin and its step, so that the exponent is formed as C0 - s^2 (see p1g_pair).
+template <int TRAV, bool GRAD>
+__device__ __forceinline__ PairC rec_row(const Geo& g, const RecIn& x, float rowoff, float& y,
+                                         float& Dy, float& u0, GradC* gc)
+{
+    u0 = __uint_as_float(x.r.x);
+    y = fmaf(x.a.y + rowoff, g.dy, g.y0);
+    Dy = y - x.a.x;
+    const float Qc = fmaf(y, fmaf(x.b.x, y, x.a.w), x.a.z);
+    const float gam = x.b.y * y, al = x.b.z * y, be = Dy * fmaf(x.b.w, y, x.c.x);
+    const float Q0 = fmaf(gam, u0, Qc), dQ = gam * g.dz;
+    // (the event's coefficients give aCb; the exponent has it times kA)
+    float A0 = fmaf(al, u0, be), dA = al * g.dz;
+    if (GRAD) {
+        gc->B0 = make_float2(A0, A0);
+        gc->dB = make_float2(dA, dA);
+    }
+    A0 *= g.kA;
+    dA *= g.kA;
+    const float C0 = fmaf(-x.c.y * Dy, Dy, x.c.z);
+    const float su0 = x.c.w * u0, dsu = x.c.w * g.dz;
+    const float e0 = GRAD ? C0 : fmaf(-su0, su0, C0), e1 = GRAD ? su0 : -2.0f * su0 * dsu,
+                e2 = GRAD ? dsu : -(dsu * dsu);
+    PairC c;
+    c.Q0 = make_float2(Q0, Q0);
+    c.dQ = make_float2(dQ, dQ);
+    c.A0 = make_float2(A0, A0);
+    c.dA = make_float2(dA, dA);
+    c.e0 = make_float2(e0, e0);
+    c.e1 = make_float2(e1, e1);
+    c.e2 = make_float2(e2, e2);
+    c.inc = make_float2((float)pair_step0<TRAV>(), (float)pair_step1<TRAV>());
+    return c;
+}
+
+// Pass 1 of the MLEM and log-likelihood forms: pairs 1 .. kmax, P rho' kept in
+// tensor memory (ST) and summed.  Chunks of eight and four pairs without any
+// test up to kfast, then chunks of four and two that zero P beyond each
+// stream's last pair.  Returns the number of pairs stored.
+template <int TRAV, int LMAX, bool ST>
+__device__ __forceinline__ int rec_pass1(unsigned base, int la, int lb, const PairC& c, int kfast,
+                                         int kmax, float2& D2, unsigned tma)
+{
+    constexpr int s0 = 4 * pair_step0<TRAV>(), s1 = 4 * pair_step1<TRAV>();
+    unsigned a0 = base + (unsigned)(4 * pair_d0<TRAV>(1));
+    unsigned a1 = base + (unsigned)(4 * pair_d1<TRAV>(1));
+    float2 kk = make_float2((float)pair_d0<TRAV>(1), (float)pair_d1<TRAV>(1));
+    unsigned col = tma;
+    int k = 1;
+#define TSP_P1(PRED, J) \
+    p1_pair<true, false, PRED, true, (J) * s0, (J) * s1>(a0, a1, k + (J), la, lb, c, kk, D2)
+    if constexpr (LMAX >= 24) {
+        for (; k + 7 <= kfast; k += 8) {
+            float x[16];
+            float2 t;
+            t = TSP_P1(false, 0), x[0] = t.x, x[1] = t.y;
+            t = TSP_P1(false, 1), x[2] = t.x, x[3] = t.y;
+            t = TSP_P1(false, 2), x[4] = t.x, x[5] = t.y;
+            t = TSP_P1(false, 3), x[6] = t.x, x[7] = t.y;
+            t = TSP_P1(false, 4), x[8] = t.x, x[9] = t.y;
+            t = TSP_P1(false, 5), x[10] = t.x, x[11] = t.y;
+            t = TSP_P1(false, 6), x[12] = t.x, x[13] = t.y;
+            t = TSP_P1(false, 7), x[14] = t.x, x[15] = t.y;
+            if constexpr (ST) tm_st16(col, x);
+            a0 += (unsigned)(8 * s0);
+            a1 += (unsigned)(8 * s1);
+            col += 16;
+        }
+    }
+    for (; k + 3 <= kfast; k += 4) {
+        const float2 pa = TSP_P1(false, 0), pb = TSP_P1(false, 1);
+        const float2 pc = TSP_P1(false, 2), pd = TSP_P1(false, 3);
+        if constexpr (ST) tm_st8(col, pa.x, pa.y, pb.x, pb.y, pc.x, pc.y, pd.x, pd.y);
+        a0 += (unsigned)(4 * s0);
+        a1 += (unsigned)(4 * s1);
+        col += 8;
+    }
+    for (; k + 2 <= kmax; k += 4) {
+        const float2 pa = TSP_P1(true, 0), pb = TSP_P1(true, 1);
+        const float2 pc = TSP_P1(true, 2), pd = TSP_P1(true, 3);
+        if constexpr (ST) tm_st8(col, pa.x, pa.y, pb.x, pb.y, pc.x, pc.y, pd.x, pd.y);
+        a0 += (unsigned)(4 * s0);
+        a1 += (unsigned)(4 * s1);
+        col += 8;
+    }
+    for (; k <= kmax; k += 2) {
+        const float2 pa = TSP_P1(true, 0), pb = TSP_P1(true, 1);
+        if constexpr (ST) tm_st4(col, pa.x, pa.y, pb.x, pb.y);
+        a0 += (unsigned)(2 * s0);
+        a1 += (unsigned)(2 * s1);
+        col += 4;
+    }
+#undef TSP_P1
+    return k - 1;
+}
+
+// Pass 2 in fixed point (see kAccWords): the values of pairs 1 .. n (n a
+// multiple of two), 0 beyond each stream's last pair, scaled by s2 = 2^12 / D
+// and sl = 2^32 / D and added to the item's two-word accumulator (H words at
+// base).
+template <int TRAV>
+__device__ __forceinline__ void rec_pass2(unsigned base, int n, unsigned tma, float2 s2, float2 sl)
+{
+    constexpr int s0 = 4 * pair_step0<TRAV>(), s1 = 4 * pair_step1<TRAV>();
+    unsigned a0 = base + (unsigned)(4 * pair_d0<TRAV>(1));
+    unsigned a1 = base + (unsigned)(4 * pair_d1<TRAV>(1));
+    unsigned col = tma;
+    int k = n;
+    for (; k >= 8; k -= 8) {
+        float x[16];
+        tm_ld16(col, x);
+        tm_wait_ld();
+        fx4<s0, s1>(a0, a1, make_float2(x[0], x[1]), make_float2(x[2], x[3]), s2, sl);
+        fx4<s0, s1>(a0 + (unsigned)(2 * s0), a1 + (unsigned)(2 * s1), make_float2(x[4], x[5]),
+                    make_float2(x[6], x[7]), s2, sl);
+        fx4<s0, s1>(a0 + (unsigned)(4 * s0), a1 + (unsigned)(4 * s1), make_float2(x[8], x[9]),
+                    make_float2(x[10], x[11]), s2, sl);
+        fx4<s0, s1>(a0 + (unsigned)(6 * s0), a1 + (unsigned)(6 * s1), make_float2(x[12], x[13]),
+                    make_float2(x[14], x[15]), s2, sl);
+        a0 += (unsigned)(8 * s0);
+        a1 += (unsigned)(8 * s1);
+        col += 16;
+    }
+    if (k >= 4) {
+        float x[8];
+        tm_ld8(col, x);
+        tm_wait_ld();
+        fx4<s0, s1>(a0, a1, make_float2(x[0], x[1]), make_float2(x[2], x[3]), s2, sl);
+        fx4<s0, s1>(a0 + (unsigned)(2 * s0), a1 + (unsigned)(2 * s1), make_float2(x[4], x[5]),
+                    make_float2(x[6], x[7]), s2, sl);
+        a0 += (unsigned)(4 * s0);
+        a1 += (unsigned)(4 * s1);
+        col += 8;
+        k -= 4;
+    }
+    if (k >= 2) {
+        float x0, x1, x2, x3;
+        tm_ld4(col, x0, x1, x2, x3);
+        tm_wait_ld();
+        fx4<s0, s1>(a0, a1, make_float2(x0, x1), make_float2(x2, x3), s2, sl);
+    }
+}
+
+// Sum over the group's G warps of each warp's value (lane 0's), the same in
+// every lane: slots of a power of two >= G floats (the unused ones stay zero),
+// summed by a butterfly.
+__device__ __forceinline__ float group_sum(float v, int G, int Gp, int wig, int lane, int bar_id,
+                                           float* slot)
+{
+    if (lane == 0) slot[wig] = v;
+    named_barrier(bar_id, G * 32);
+    v = slot[lane & (Gp - 1)];
+    for (int o = Gp >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Gradient pass, one pair: the kernel value's pair (0 beyond the streams' last
+// pairs), and the sums that D and the sigma gradients are made of.  With
+// X = aCb / Q and S = X^2 + 1/Q, every term of the derivatives is a polynomial in
+// the offset d times 1, X or S (see rec_grad_row), so the moments
+//   sum v, sum v d, sum v d^2, sum v X, sum v X d, sum v S, sum v S d   (v = P rho')
+// are all that the loop has to sum: eleven packed operations a pair beside the
+// kernel's own, against fifteen when the derivatives are formed per pixel.  The
+// exponent is formed as C0 - s^2 with s linear in d, not as a quadratic in d, and
+// X from aCb itself, not from the scaled one of the exponent: with windows wide
+// enough that the truncated tails are negligible the derivatives nearly cancel
+// over a window, and the rounding of a coefficient that is the same for every
+// event would show in their sum.
+struct GradSums {
+    float2 m0, m1, m2, x0, x1, s0, s1;
+    float pmax;
+};
+
+template <bool PRED, int OFF0, int OFF1>
+__device__ __forceinline__ float2 p1g_pair(unsigned a0, unsigned a1, int k, int la, int lb,
+                                           const PairC& c, const GradC& g, float2& kk,
+                                           GradSums& m)
+{
+    float2 q = __ffma2_rn(kk, c.dQ, c.Q0);
+    if constexpr (PRED) {
+        // keeps X and S finite where P is set to 0 below
+        q.x = k <= la ? q.x : 1.0f;
+        q.y = k <= lb ? q.y : 1.0f;
+    }
+    float2 rq;
+    rq.x = rsqrt_approx(q.x);
+    rq.y = rsqrt_approx(q.y);
+    const float2 a = __ffma2_rn(kk, c.dA, c.A0);
+    const float2 su = __ffma2_rn(kk, c.e2, c.e1);
+    const float2 e = __ffma2_rn(su, __fmul2_rn(su, make_float2(-1.0f, -1.0f)), c.e0);
+    const float2 w = __fmul2_rn(a, rq);
+    const float2 ar = __ffma2_rn(w, w, e);
+    float2 x;
+    x.x = ex2_approx(ar.x);
+    x.y = ex2_approx(ar.y);
+    float2 p = __fmul2_rn(rq, x);
+    if constexpr (PRED) {
+        p.x = k <= la ? p.x : 0.0f;
+        p.y = k <= lb ? p.y : 0.0f;
+    }
+    float2 v;
+    v.x = ld_rhop<true, false, false, OFF0>(a0, k, la);
+    v.y = ld_rhop<true, false, false, OFF1>(a1, k, lb);
+    const float2 pv = __fmul2_rn(p, v), pvd = __fmul2_rn(pv, kk);
+    const float2 iq = __fmul2_rn(rq, rq);
+    const float2 X = __fmul2_rn(__ffma2_rn(kk, g.dB, g.B0), iq), S = __ffma2_rn(X, X, iq);
+    m.m0 = __fadd2_rn(m.m0, pv);
+    m.m1 = __fadd2_rn(m.m1, pvd);
+    m.m2 = __ffma2_rn(pvd, kk, m.m2);
+    m.x0 = __ffma2_rn(pv, X, m.x0);
+    m.x1 = __ffma2_rn(pvd, X, m.x1);
+    m.s0 = __ffma2_rn(pv, S, m.s0);
+    m.s1 = __ffma2_rn(pvd, S, m.s1);
+    m.pmax = fmaxf(m.pmax, fmaxf(p.x, p.y));
+    kk = __fadd2_rn(kk, c.inc);
+    return p;
+}
+
+// Gradient pass over pairs 1 .. kmax, P kept in tensor memory, two pairs a step
+// (the sums and constants leave no registers for more).  Returns the number of
+// pairs stored.
+template <int TRAV>
+__device__ __forceinline__ int rec_pass1_grad(unsigned base, int la, int lb, const PairC& c,
+                                              const GradC& g, int kfast, int kmax, GradSums& m,
+                                              unsigned tma)
+{
+    constexpr int s0 = 4 * pair_step0<TRAV>(), s1 = 4 * pair_step1<TRAV>();
+    unsigned a0 = base + (unsigned)(4 * pair_d0<TRAV>(1));
+    unsigned a1 = base + (unsigned)(4 * pair_d1<TRAV>(1));
+    float2 kk = make_float2((float)pair_d0<TRAV>(1), (float)pair_d1<TRAV>(1));
+    unsigned col = tma;
+    int k = 1;
+    for (; k + 1 <= kfast; k += 2) {
+        const float2 pa = p1g_pair<false, 0, 0>(a0, a1, k, la, lb, c, g, kk, m);
+        const float2 pb = p1g_pair<false, s0, s1>(a0, a1, k + 1, la, lb, c, g, kk, m);
+        tm_st4(col, pa.x, pa.y, pb.x, pb.y);
+        a0 += (unsigned)(2 * s0);
+        a1 += (unsigned)(2 * s1);
+        col += 4;
+    }
+    for (; k <= kmax; k += 2) {
+        const float2 pa = p1g_pair<true, 0, 0>(a0, a1, k, la, lb, c, g, kk, m);
+        const float2 pb = p1g_pair<true, s0, s1>(a0, a1, k + 1, la, lb, c, g, kk, m);
+        tm_st4(col, pa.x, pa.y, pb.x, pb.y);
+        a0 += (unsigned)(2 * s0);
+        a1 += (unsigned)(2 * s1);
+        col += 4;
+    }
+    return k - 1;
+}
+
+// (Ez, El) of a lane from its moments: the sums of v dlogP/d(iz) and
+// v dlogP/d(il),
+//   d log P / d iz = 1/iz - u^2 + X Cz - (Qz/2) S
+//   d log P / d il = 1/(2 il) - Bl/2 + X Cl - (Ql/2) S
+// with u, Cz and Qz linear in d (formulas in make_row), the z terms with
+// respect to the base iz (times inv_f2).
+__device__ __forceinline__ float2 rec_grad_row(const Geo& g, const float4& ev, float y, float Dy,
+                                               float u0, const GradSums& m)
+{
+    const EvSig es = ev_sig(g, ev);
+    const float t = ev.z, c2i = ev.w, y2 = y * y, dz = g.dz;
+    const float m0 = m.m0.x + m.m0.y, m1 = m.m1.x + m.m1.y, m2 = m.m2.x + m.m2.y;
+    const float x0 = m.x0.x + m.x0.y, x1 = m.x1.x + m.x1.y;
+    const float s0 = m.s0.x + m.s0.y, s1 = m.s1.x + m.s1.y;
+    const float qzs = -2.0f * y * t * c2i, qz0 = fmaf(qzs, u0, (g.R * g.R + y2) * c2i * c2i);
+    const float czs = -2.0f * y * c2i;
+    // sum v u^2 = u0^2 m0 + 2 u0 dz m1 + dz^2 m2
+    const float vu2 = fmaf(u0, fmaf(u0, m0, 2.0f * dz * m1), dz * dz * m2);
+    const float Ez = fmaf(es.ldz, m0, -vu2) + czs * fmaf(u0, x0, dz * x1) - fmaf(qz0, s0, qzs * dz * s1);
+    const float Bl = 4.0f * Dy * Dy * c2i;
+    const float cl = 4.0f * y * t * Dy * c2i;
+    const float qlh = 2.0f * y2 * t * t * c2i + 2.0f * y * fmaf(2.0f * t, t, 1.0f) * Dy * c2i;
+    const float El = fmaf(es.ldl - 0.5f * Bl, m0, fmaf(cl, x0, -qlh * s0));
+    return make_float2(Ez * es.inv_f2, El);
+}
+
+// The scatter of an event whose largest P / D exceeds the gradient pass's fixed
+// point unit (see k_tiles_rec): float adds to the global A, each pixel under its
+// predicate.
+template <int TRAV>
+__device__ __forceinline__ void rec_scatter_global(const Inst& I, const Frame& f, unsigned idx,
+                                                   int la, int lb, int kmax, unsigned tma,
+                                                   float invD)
+{
+    const int rr = (int)idx / f.stride, col = (int)idx - rr * f.stride;
+    const int iy = f.oy + rr;
+    const int iz = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0))) + col;
+    RowP<false> q;
+    q.base = (unsigned long long)(I.A + ((long long)iy * I.g.nz + iz));
+    q.gbase = 0;
+    q.la = la;
+    q.lb = lb;
+    pass2_pairs<TRAV, false>(q, 0, 0, kmax, tma, make_float2(invD, invD));
+}
+
+// The events first + grp, first + grp + ngroups, ... of an item, by one group
+// of G warps.  GRAD: inv_unit is 1 over the unit of the fixed-point terms P / D.
+template <int TRAV, int LMAX, int MODE, int NSEG>
+__device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int first, int count,
+                                           int grp, int ngroups, int wig, int lane,
+                                           unsigned rp_addr, unsigned acc_off, unsigned slot,
+                                           float* part, BlockSums* bs, unsigned tma, float inv_unit)
+{
+    constexpr bool GRAD = MODE == kGrad;
+    const Geo& g = I.g;
+    const int G = I.G;
+    int left = (count - grp + ngroups - 1) / ngroups;
+    if (left <= 0) return;
+    // the row block of a warp is rotated by its group (see process_event)
+    int blk;
+    if constexpr (NSEG == 1) {
+        blk = wig + grp % G;
+        blk -= blk >= G ? G : 0;
+    } else {
+        const int nb = G >> 1;
+        blk = (wig >> 1) + grp % nb;
+        blk -= blk >= nb ? nb : 0;
+    }
+    const float rowoff = (float)lane_row(blk * 32 + lane);
+    const int Gp = G > 1 ? 1 << (32 - __clz(G - 1)) : 1;
+    const int rslot = NSEG == 1 ? blk * 32 + lane : (blk * 2 + (wig & 1)) * 32 + lane;
+    const uint2* rp = I.evs.recs + (size_t)(first + grp) * (32 * G) + rslot;
+    const float4* ep = I.evs.evc + (size_t)(first + grp) * kEvcFloat4;
+    rec_fetch(slot, rp, ep, lane);
+    unsigned used = 0;
+    double logD = 0.0, giz = 0.0, gil = 0.0;
+    int parity = 0;
+    for (;;) {
+        RecIn x;
+        rec_wait();
+        rec_take(x, slot, lane);
+        float y, Dy, u0;
+        GradC gc;
+        const PairC c = rec_row<TRAV, GRAD>(g, x, rowoff, y, Dy, u0, &gc);
+        const unsigned idx = x.r.y & 0xffffu, base = rp_addr + 4u * idx;
+        const int la = (x.r.y >> 16) & 0xff, lb = x.r.y >> 24;
+        const int kmax = __reduce_max_sync(0xffffffffu, max(la, lb));
+        const int kfast = __reduce_min_sync(0xffffffffu, min(la, lb));
+        float4 ev;
+        if constexpr (GRAD) ev = lds128(slot + 304u);
+        __syncwarp();   // every lane has its values: the slot may be refilled
+        if (--left > 0) {
+            rp += (size_t)ngroups * (32 * G);
+            ep += ngroups * kEvcFloat4;
+            rec_fetch(slot, rp, ep, lane);
+        }
+        int n;
+        float D, pmax = 0.0f;
+        float2 E = make_float2(0.0f, 0.0f);
+        if constexpr (GRAD) {
+            GradSums m;
+            m.m0 = m.m1 = m.m2 = m.x0 = m.x1 = m.s0 = m.s1 = make_float2(0.0f, 0.0f);
+            m.pmax = 0.0f;
+            n = rec_pass1_grad<TRAV>(base, la, lb, c, gc, kfast, kmax, m, tma);
+            E = rec_grad_row(g, ev, y, Dy, u0, m);
+            D = warp_sum(m.m0.x + m.m0.y);
+            E.x = warp_sum(E.x);
+            E.y = warp_sum(E.y);
+            // (bits of non-negative floats order as integers)
+            pmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m.pmax)));
+        } else {
+            float2 D2 = make_float2(0.0f, 0.0f);
+            n = rec_pass1<TRAV, LMAX, MODE != kLoglik>(base, la, lb, c, kfast, kmax, D2, tma);
+            D = warp_sum(D2.x + D2.y);
+        }
+        if (MODE != kLoglik) tm_wait_st();
+        if (G > 1) {
+            if constexpr (GRAD) {
+                float4* sl = reinterpret_cast<float4*>(part) + (parity ? G : 0);
+                if (lane == 0) sl[wig] = make_float4(D, E.x, E.y, pmax);
+                named_barrier(1 + grp, G * 32);
+                D = E.x = E.y = pmax = 0.0f;
+                for (int w = 0; w < G; ++w) {
+                    const float4 v = sl[w];
+                    D += v.x;
+                    E.x += v.y;
+                    E.y += v.z;
+                    pmax = fmaxf(pmax, v.w);
+                }
+            } else {
+                D = group_sum(D, G, Gp, wig, lane, 1 + grp, part + parity * Gp);
+            }
+            parity ^= 1;
+        }
+        if (D > 0.0f) {
+            ++used;
+            if (MODE != kMlem && wig == 0 && lane == 0) {
+                logD += (double)logf(D);
+                if (GRAD) {
+                    giz += (double)(E.x / D);
+                    gil += (double)(E.y / D);
+                }
+            }
+            if (MODE != kLoglik) {
+                const float invD = 1.0f / D;
+                const float r = GRAD ? invD * inv_unit : invD;
+                if (!GRAD || pmax * r <= 1.0f) {
+                    const float s = r * 4096.0f, sl = r * 0x1p32f;
+                    rec_pass2<TRAV>(base + acc_off, n, tma, make_float2(s, s), make_float2(sl, sl));
+                } else {
+                    rec_scatter_global<TRAV>(I, f, idx, la, lb, kmax, tma, invD);
+                }
+            }
+        }
+        if (left == 0) break;
+    }
+    if (wig == 0 && lane == 0) {
+        if (used) atomicAdd(&bs->used, (unsigned long long)used);
+        if (MODE != kMlem) atomicAdd(&bs->logD, logD);
+        if (GRAD) {
+            atomicAdd(&bs->giz, giz);
+            atomicAdd(&bs->gil, gil);
+        }
+    }
+}
+
+// Persistent tile kernel over window records.  Work
+// items, batches and the two-word accumulator are those of k_tiles; the first
+// item of a block is its index, later ones come from the queue, asked for while
+// an item is worked on.
+//
+// The gradient pass needs sum P / D also where rho' = 0, so its terms are not the
+// bounded responsibilities P rho' / D.  It adds P / D in units of
+//   U = (N / sum rho') max(1, 64 npix / W)       (W: the list's window pixels):
+// N / sum rho' is the rho'-weighted mean of the result A (sum_l rho'_l A_l = N),
+// and with few events a single term is larger than that, on the average by up to
+// some 4 npix / W times.  The quantum U 2^-32 is far below the rounding of float
+// sums of the size of A; an event whose largest term exceeds U (its window
+// nearly empty of activity, or of a far brighter spot) is scattered by float adds
+// to global memory instead.  The largest P is taken from the evaluated values.
+template <int LMAX, int MODE, int NSEG, bool BATCH>
+__global__ void __launch_bounds__(pass_threads(LMAX, MODE, NSEG, BATCH), 1)
+k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ items, int n_items,
+            int* queue)
+{
+    constexpr int kThreads = pass_threads(LMAX, MODE, NSEG, BATCH);
+    constexpr int kWarps = kThreads / 32;
+    extern __shared__ float4 smem_f4[];
+    float* const smem = reinterpret_cast<float*>(smem_f4);
+    float* const s_part = smem;
+    float* const s_rp = smem + kPartFloats + kMaxWarps * kRecSlotFloats + kPadFloats;
+    __shared__ int s_item[2];
+    __shared__ BlockSums s_sums;
+    __shared__ Inst s_inst;
+    __shared__ unsigned s_tmem;
+    __shared__ float2 s_unit;
+    const Inst& I = BATCH ? s_inst : p;
+
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    constexpr int kCols = tm_block_cols(LMAX, kWarps);
+    if (warp == 0) tm_alloc<kCols>(&s_tmem);
+    init_block_sums(&s_sums);
+#ifdef TSP_DEBUG_CHECKS
+    if (tid == 0) tsp_dbg_word = 0ull;
+#endif
+    // slots of warps that a group does not have stay zero (group_sum)
+    for (int k = tid; k < kPartFloats; k += kThreads) s_part[k] = 0.0f;
+    int cur = -1, it = blockIdx.x, par = 0;
+    bool fresh = true;
+    tm_sync_threads();
+    const unsigned tma = tm_thread_addr<LMAX>(s_tmem, warp);
+
+    while (it < n_items) {
+        int next = 0;
+        if (tid == 0) next = (int)gridDim.x + atomicAdd(queue, 1);
+        const int4 item = items[it];
+        if (BATCH && item.w != cur) {
+            if (cur >= 0 && tid == 0) {
+                flush_block_sums(&s_sums, s_inst.accum, MODE);
+                init_block_sums(&s_sums);
+#ifdef TSP_DEBUG_CHECKS
+                if (tsp_dbg_word) atomicCAS(&s_inst.accum->dbg, 0ull, tsp_dbg_word);
+                tsp_dbg_word = 0ull;
+#endif
+            }
+            __syncthreads();
+            const unsigned long long* src = reinterpret_cast<const unsigned long long*>(table + item.w);
+            unsigned long long* dst = reinterpret_cast<unsigned long long*>(&s_inst);
+            for (int k = tid; k < (int)(sizeof(Inst) / 8); k += kThreads) dst[k] = src[k];
+            cur = item.w;
+            fresh = true;
+            __syncthreads();
+        }
+        const Geo& g = I.g;
+        const Tiling& tl = I.tl;
+        const int region = tl.RH * tl.RS;
+        float* const s_acc = s_rp + region + 2 * kPadFloats;
+        unsigned* const s_accL = reinterpret_cast<unsigned*>(s_acc) + kAccWords;
+        if (fresh) {
+            // the slack around the regions is read (times P = 0) and added
+            // zeros to by the unpredicated accesses: finite values
+            for (int k = tid; k < kPadFloats; k += kThreads) {
+                s_rp[-kPadFloats + k] = 0.0f;
+                s_rp[region + k] = 0.0f;
+                s_acc[-kPadFloats + k] = 0.0f;
+                s_acc[region + k] = 0.0f;
+            }
+            fresh = false;
+            // the groups' slots change their layout with G
+            if (BATCH)
+                for (int k = tid; k < kPartFloats; k += kThreads) s_part[k] = 0.0f;
+        }
+        const Frame f = tile_frame(g, tl, item.x);
+        for (int rr = warp; rr < tl.RH; rr += kWarps) {
+            const int iy = f.oy + rr;
+            const bool row_in = iy >= 0 && iy < g.ny;
+            const int z0row = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0)));
+            for (int cc = lane; cc < tl.RS; cc += 32) {
+                const int iz = z0row + cc;
+                float v = 0.0f;
+                if (row_in && cc < tl.RW && iz >= 0 && iz < g.nz)
+                    v = I.rhop[(size_t)iy * g.nz + iz];
+                s_rp[rr * tl.RS + cc] = v;
+                if (MODE != kLoglik) {
+                    s_acc[rr * tl.RS + cc] = 0.0f;
+                    s_accL[rr * tl.RS + cc] = 0u;
+                }
+            }
+        }
+        if (tid == 0) {
+            s_item[par] = next;
+            if (MODE == kGrad) {
+                const double sum = I.accum->sum_rhop;
+                const float u = (float)(I.grad_unit / sum);
+                const bool ok = sum > 0.0 && u >= 1e-30f && u <= 1e30f;
+                // (no usable scale: every event takes the float scatter)
+                s_unit = ok ? make_float2(u, 1.0f / u) : make_float2(1.0f, INFINITY);
+            }
+            // pixels that the records left out, counted once a pass
+            if (item.y == 0) {
+                s_sums.qclip += I.accum->rec_qclip;
+                s_sums.lclip += I.accum->rec_lclip;
+            }
+        }
+        __syncthreads();
+        {
+            const int G = I.G;
+            const int ngroups = group_count(kWarps, G);
+            const int grp = warp / G, wig = warp - grp * G;
+            float* part = s_part + grp * (kPartFloats / kWarps) * G;
+            const unsigned rp_addr = (unsigned)__cvta_generic_to_shared(s_rp);
+            const unsigned acc_off = 4u * (unsigned)(region + 2 * kPadFloats);
+            const unsigned slot =
+                (unsigned)__cvta_generic_to_shared(smem + kPartFloats + warp * kRecSlotFloats);
+            const float inv_unit = MODE == kGrad ? s_unit.y : 0.0f;
+#define TSP_REC_EVENTS(TRAV) \
+    rec_events<TRAV, LMAX, MODE, NSEG>(I, f, item.y, item.z, grp, ngroups, wig, lane, rp_addr, \
+                                       acc_off, slot, part, &s_sums, tma, inv_unit)
+            if (grp < ngroups) {
+                if (NSEG == 1)
+                    TSP_REC_EVENTS(kAlt);
+                else if ((wig & 1) == 0)
+                    TSP_REC_EVENTS(kPos);
+                else
+                    TSP_REC_EVENTS(kNeg);
+            }
+#undef TSP_REC_EVENTS
+        }
+        __syncthreads();
+        it = s_item[par];
+        par ^= 1;
+        if (MODE != kLoglik) {
+            for (int rr = warp; rr < tl.RH; rr += kWarps) {
+                const int iy = f.oy + rr;
+                if (iy < 0 || iy >= g.ny) continue;
+                const int z0row = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0)));
+                for (int cc = lane; cc < tl.RW; cc += 32) {
+                    const int iz = z0row + cc;
+                    const int k = rr * tl.RS + cc;
+                    // A += X / rho' (the fixed-point sums, see kAccWords)
+                    const unsigned wh = __float_as_uint(s_acc[k]), wl = s_accL[k];
+                    const unsigned sh = wh & 0xFFFFFFu, sl = wl - (wh & 0xFF000000u);
+                    const float X = fmaf((float)sl, 0x1p-32f, (float)sh * 0x1p-12f);
+                    float v;
+                    if (MODE == kGrad) {
+                        v = X * s_unit.x;           // terms P / D in units of s_unit.x
+                    } else {
+                        const float rp = s_rp[k];
+                        v = rp > 0.0f ? X / rp : 0.0f;
+                    }
+                    if (iz >= 0 && iz < g.nz && v != 0.0f)
+                        atomicAdd(I.A + (size_t)iy * g.nz + iz, v);
+                }
+            }
+            __syncthreads();
+        }
+    }
+    tm_sync_threads();
+    if (!BATCH || cur >= 0) flush_block_sums(&s_sums, I.accum, MODE);
+#ifdef TSP_DEBUG_CHECKS
+    if (tid == 0 && tsp_dbg_word && (!BATCH || cur >= 0))
+        atomicCAS(&I.accum->dbg, 0ull, tsp_dbg_word);
+#endif
+    if (warp == 0) tm_dealloc<kCols>(s_tmem);
+}
+
+}  // namespace tsp

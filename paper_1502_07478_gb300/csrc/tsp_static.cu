@@ -175,12 +175,15 @@ extern "C" int tsp_mlem_update_noalloc(const tsp_params* params, const float* zu
     a.evs.geo = geo;
     a.evs.geo64 = geo64;
     a.evs.rows = rows;
+    a.evs.recs = nullptr;
+    a.evs.evc = nullptr;
     a.items = nullptr;
     a.n_items = 0;
     a.outlier_first = 0;
     a.rhop = rhop;
     a.A = A;
     a.accum = accum;
+    a.grad_unit = 0.0;
     a.G = G;
     a.nseg = nseg;
     a.gld = 0;
