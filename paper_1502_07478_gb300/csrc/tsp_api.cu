@@ -217,10 +217,32 @@ int refresh_rhop(tsp_ctx* c, cudaStream_t st)
     return TSP_OK;
 }
 
-double grad_unit(const tsp_ctx* c)
+// Events over a pixel of the image, on the average.
+double coverage(const tsp_ctx* c)
 {
-    const double w = (double)c->counters_h[3];     // in-window pixels of the list
-    return (double)c->n * std::max(1.0, w > 0.0 ? 64.0 * c->npix / w : 1.0);
+    return (double)c->counters_h[3] / c->npix;     // in-window pixels of the list
+}
+
+// A Gaussian cut at its n-sigma ellipse has the mean (1 - e^(-n^2/2)) / (n^2/2) of
+// its maximum.
+float fx_peak(const tsp_ctx* c)
+{
+    const double n = (double)(c->n - (long long)c->counters_h[1]);   // events with a window
+    const double h = 0.5 * c->g.cut2d, mean = (1.0 - std::exp(-h)) / h;
+    return c->counters_h[3] ? (float)(n / (mean * (double)c->counters_h[3])) : 1.0f;
+}
+
+// An ordinary event's largest term takes fx_bits bits.  Its mean term is then some
+// 2^(fx_bits - 2.2) quanta, each rounded to the nearest one, and over the cov events
+// of a pixel the rounding of A is 0.3 x 2^(2.2 - fx_bits) / sqrt(cov) of it: with
+//   fx_bits = 22.9 - log2(cov / 64) / 2
+// some 2e-8 for every list (less than 1e-7 at 64 events a pixel, where 21 bits are
+// the most), which the float sums of the denominators (some 3e-7) hide.  The rest up
+// to 2^24 is the headroom of single events.
+int fx_bits(const tsp_ctx* c)
+{
+    const double cov = std::max(coverage(c), 1.0);
+    return std::max(12, std::min(21, (int)std::lround(22.9 - 0.5 * std::log2(cov / 64.0))));
 }
 
 PassArgs pass_args(tsp_ctx* c)
@@ -240,12 +262,15 @@ PassArgs pass_args(tsp_ctx* c)
     a.rhop = c->rhop;
     a.A = c->A;
     a.accum = c->accum;
-    a.grad_unit = grad_unit(c);
+    a.fx_peak = fx_peak(c);
+    a.fx_bits = fx_bits(c);
+    a.scratch = c->scratch;
     a.G = c->G;
     a.nseg = c->nseg;
     a.gld = c->gld;
     a.grid = c->num_sms;
     a.smem = c->smem;
+    a.rec_smem = rec_smem_floats(c->tl.RH, c->tl.RS, c->gld != 0) * sizeof(float);
     return a;
 }
 
@@ -282,12 +307,20 @@ int prep_chunk(tsp_ctx* c, long long first, long long n, cudaStream_t st)
 // Window records of the placed events.  They are kept when they take at most a
 // quarter of the memory that is free when their buffer has to grow (6e7 events
 // at 1 mm on an empty 280 GB); otherwise, or when the allocation fails, the
-// passes set the rows up themselves.
+// passes set the rows up themselves.  So do those of sparse lists, with fewer than
+// kRecCoverage events over a pixel: one word of fixed point has no room for both
+// the headroom and the precision that a sum of few terms needs (see fx_bits), and
+// the two-word accumulator of the general passes has.
+constexpr double kRecCoverage = 64.0;
+
 int build_records(tsp_ctx* c, cudaStream_t st)
 {
     c->rec = false;
     const long long placed = c->outlier_first;
-    if (c->gld || c->n_items == 0 || placed == 0) return TSP_OK;
+    if (c->n_items == 0 || placed == 0 || coverage(c) < kRecCoverage) return TSP_OK;
+    // (a batch takes the events of such a member through global memory)
+    if (c->gld && c->batch_member) return TSP_OK;
+    if (c->gld && c->tl.RH > kScrRows) return TSP_OK;
     const size_t per = record_bytes(c->G);
     const size_t need = (per + kEvcBytes) * (size_t)placed;
     if (sim_fault() == kSimRecords) return TSP_OK;
@@ -302,6 +335,19 @@ int build_records(tsp_ctx* c, cudaStream_t st)
             return TSP_OK;
         }
         c->rec_cap = need;
+    }
+    if (c->gld) {
+        const size_t scr = (size_t)c->num_sms * c->tl.RS * kScrRows;
+        if (scr > c->scratch_cap) {
+            dfree(c->scratch);
+            c->scratch_cap = 0;
+            if (dmalloc(&c->scratch, scr * sizeof(float)) != cudaSuccess) {
+                cudaGetLastError();
+                c->scratch = nullptr;
+                return TSP_OK;
+            }
+            c->scratch_cap = scr;
+        }
     }
     c->recs = reinterpret_cast<uint2*>(c->recbuf);
     c->evc = reinterpret_cast<float4*>(c->recbuf + per * (size_t)placed);
@@ -570,6 +616,7 @@ void tsp_destroy(tsp_ctx* c)
     dfree(c->geo_u); dfree(c->geo); dfree(c->geo64_u); dfree(c->geo64);
     dfree(c->rows_u); dfree(c->rows); dfree(c->key);
     dfree(c->recbuf);
+    dfree(c->scratch);
     dfree(c->items); dfree(c->bin_count); dfree(c->offsets); dfree(c->cursor);
     delete c;
 }

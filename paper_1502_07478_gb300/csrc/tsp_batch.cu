@@ -169,7 +169,9 @@ int rebuild(tsp_batch* b, cudaStream_t st)
         t.A = c->A;
         t.accum = c->accum;
         t.G = c->G;
-        t.grad_unit = grad_unit(c);
+        t.fx_peak = fx_peak(c);
+        t.fx_bits = fx_bits(c);
+        t.scratch = nullptr;
         BatchImg& m = imgs[i];
         m.rho = c->rho;
         m.rhop = c->rhop;
@@ -475,6 +477,7 @@ int tsp_batch_create(const tsp_params* params, int k, tsp_batch** out)
         }
         b->inst.push_back(c);
         c->sched = b->sched;
+        c->batch_member = true;
     }
     cudaError_t e = dmalloc(&b->table, sizeof(Inst) * k);
     if (e == cudaSuccess) e = dmalloc(&b->imgs, sizeof(BatchImg) * k);

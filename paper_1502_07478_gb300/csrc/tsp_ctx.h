@@ -66,6 +66,9 @@ struct tsp_ctx {
     uint2* recs = nullptr;
     float4* evc = nullptr;
     bool rec = false;
+    bool batch_member = false;        // the batch launches the passes
+    float* scratch = nullptr;         // transposed rho' regions of the blocks (gld)
+    size_t scratch_cap = 0;           // in floats
     int4* items = nullptr;
     int n_items = 0, items_cap = 0;
     std::vector<int> bin_cnt;          // events per bin (host copy; last = outliers)
@@ -150,8 +153,9 @@ std::vector<int4> tile_items(const tsp_ctx* c, long long E, int w);
 long long item_events(long long placed, int items_per_sm, int sms);
 int ensure_sensitivity(tsp_ctx* c, cudaStream_t st);
 int refresh_rhop(tsp_ctx* c, cudaStream_t st);
-// The gradient pass's fixed-point unit times sum rho' (Inst::grad_unit).
-double grad_unit(const tsp_ctx* c);
+// The fixed point of the passes over window records (Inst::fx_peak, fx_bits).
+float fx_peak(const tsp_ctx* c);
+int fx_bits(const tsp_ctx* c);
 void clear_graphs(tsp_ctx* c);
 
 }  // namespace tsp_host

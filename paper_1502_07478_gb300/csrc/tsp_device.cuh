@@ -67,6 +67,9 @@ struct Geo {
     // z-dependent resolution (Sec. 3): an event at z~ has sigma_z f,
     // f = 1 + kz min(1, zs2 z~^2); kz = 0 keeps sigma_z constant
     float kz, zs2;          // kappa_z, (2/L)^2
+    // the passes over window records hold P 2^-pshift (a whole number; 0 with
+    // lengths in mm), so that a kernel value is near 2^-22 in any unit of length
+    float pshift, pad0;
     // double-precision copies for the exact window decision near its boundary
     double y0d, z0d, dyd, dzd, Rd, izd, ild, cut2d;
     double Ld;              // strip length
@@ -197,6 +200,20 @@ __host__ __device__ constexpr size_t tiles_smem_floats(int RH, int RS)
            (size_t)RH * RS + kPadFloats + kPartFloats + kMaxWarps * kRecSlotFloats;
 }
 
+// Shared memory of the passes over window records, in 32-bit words: the groups'
+// reduction slots, the warps' staging slots, then the rho' region (not with
+// `gld`) and the one-word accumulator, each with kPadFloats of slack around it.
+__host__ __device__ constexpr size_t rec_smem_floats(int RH, int RS, bool gld)
+{
+    return (size_t)kPartFloats + kMaxWarps * kRecSlotFloats +
+           (gld ? 1 : 2) * ((size_t)RH * RS + 2 * kPadFloats);
+}
+
+// Rows of a block's transposed rho' region in global memory (gld): a
+// compile-time column stride, for the loops' immediate offsets.  A window has at
+// most 256 rows and a tile at most 128, so a region has at most 128 + 2 * 130.
+constexpr int kScrRows = 416;
+
 // A staged region fits the two-word accumulator layout.
 __host__ __device__ constexpr bool tiles_region_fits(int RH, int RS)
 {
@@ -292,7 +309,12 @@ struct Inst {
     const float* rhop;
     float* A;
     Accum* accum;
-    double grad_unit;   // N max(1, 64 npix / W): the gradient pass's unit times sum rho'
+    // fixed point of the passes over window records (see k_tiles_rec): 1 / (mean
+    // of P / max P over a window x mean pixels of a window), and the bits of an
+    // ordinary event's largest term
+    float fx_peak;
+    int fx_bits;
+    float* scratch;     // rho' regions of the blocks, transposed (kScrRows), or null
     int G;
     int pad;
 };

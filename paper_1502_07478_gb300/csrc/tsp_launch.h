@@ -112,11 +112,14 @@ struct PassArgs {
     const float* rhop;
     float* A;
     Accum* accum;
-    double grad_unit;  // see Inst
+    float fx_peak;     // see Inst
+    int fx_bits;
+    float* scratch;
     int G, nseg;
     int gld;           // tiles stage only A; rho' read from global (nseg = 2)
     int grid;          // persistent blocks
     size_t smem;       // dynamic shared memory of the tile kernel
+    size_t rec_smem;   // and of its form over window records
 };
 
 // Window records of a list's binned events (tsp_rec.cuh): written once per

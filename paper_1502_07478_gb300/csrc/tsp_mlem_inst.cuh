@@ -25,19 +25,15 @@ cudaError_t run_pass(const PassArgs& a, cudaStream_t st)
         p.A = a.A;
         p.accum = a.accum;
         p.G = a.G;
-        p.grad_unit = a.grad_unit;
+        p.fx_peak = a.fx_peak;
+        p.fx_bits = a.fx_bits;
+        p.scratch = a.scratch;
         p.pad = 0;
-        bool done = false;
-        if constexpr (!GLD) {
-            if (a.evs.recs) {
-                k_tiles_rec<LMAX, MODE, NSEG, false>
-                    <<<a.grid, pass_threads(LMAX, MODE, NSEG, false), a.smem, st>>>(
-                    p, nullptr, a.items, a.n_items, &a.accum->queue);
-                done = true;
-            }
-        }
-        if (done) {
-        } else if (a.g.kz != 0.0f)
+        if (a.evs.recs)
+            k_tiles_rec<LMAX, MODE, NSEG, false, GLD>
+                <<<a.grid, pass_threads(LMAX, MODE, NSEG, false), a.rec_smem, st>>>(
+                p, nullptr, a.items, a.n_items, &a.accum->queue);
+        else if (a.g.kz != 0.0f)
             k_tiles<LMAX, MODE, NSEG, false, GLD, true>
                 <<<a.grid, pass_threads(LMAX, MODE, NSEG, false), a.smem, st>>>(
                 p, nullptr, a.items, a.n_items, &a.accum->queue);
@@ -68,10 +64,13 @@ cudaError_t set_smem(size_t smem)
 {
     cudaError_t e = set_smem_one<LMAX, MODE, NSEG, false, false>(smem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_tiles_rec<LMAX, MODE, NSEG, false>,
+        e = cudaFuncSetAttribute(k_tiles_rec<LMAX, MODE, NSEG, false, false>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = set_smem_one<LMAX, MODE, NSEG, false, true>(smem);
     if constexpr (NSEG == 2) {
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_tiles_rec<LMAX, MODE, NSEG, false, true>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e == cudaSuccess) e = set_smem_one<LMAX, MODE, NSEG, true, false>(smem);
         if (e == cudaSuccess) e = set_smem_one<LMAX, MODE, NSEG, true, true>(smem);
     }
@@ -86,7 +85,7 @@ cudaError_t run_batch(const BatchArgs& a, cudaStream_t st)
     Inst none{};
     if (a.n_items > 0) {
         if (a.rec)
-            k_tiles_rec<LMAX, MODE, NSEG, true>
+            k_tiles_rec<LMAX, MODE, NSEG, true, false>
                 <<<a.grid, pass_threads(LMAX, MODE, NSEG, true), a.smem, st>>>(
                     none, a.table, a.items, a.n_items, a.queue);
         else if (a.kz)
@@ -125,9 +124,9 @@ cudaError_t batch_smem(size_t smem)
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_tiles<LMAX, kMlem, NSEG, true, false, true>, at, v);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_tiles_rec<LMAX, kMlem, NSEG, true>, at, v);
+        e = cudaFuncSetAttribute(k_tiles_rec<LMAX, kMlem, NSEG, true, false>, at, v);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_tiles_rec<LMAX, kGrad, NSEG, true>, at, v);
+        e = cudaFuncSetAttribute(k_tiles_rec<LMAX, kGrad, NSEG, true, false>, at, v);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_tiles<LMAX, kGrad, NSEG, true, false, false>, at, v);
     if (e == cudaSuccess)

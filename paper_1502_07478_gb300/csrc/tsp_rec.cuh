@@ -29,9 +29,34 @@ namespace tsp {
 //   Q(u) = q0 + y (q1 + q2 y) + g1 y u,    aCb = a1 y u + Dy (b1 y + b2),
 //   C0 = log2K - hB Dy^2,   ksu = sqrt(log2(e) iz) of the event,
 // stored as float4 (y~, mid, q0, q1), (q2, g1, a1, b1), (b2, hB, log2K, ksu) and
-// the event's geometry (y~, z~, t, c2i), which the gradient pass needs;
-// mid is the middle row of the window (lane rows count outward from it).
+// (max, z~, t, c2i): an upper bound of P over the window, and the event's geometry,
+// which the gradient pass needs;
+// mid is the middle row of the window (lane rows count outward from it).  P is
+// held times 2^-pshift (see Geo).
 constexpr int kEvcFloat4 = 4;
+
+// An upper bound of P over the event's window.  With C^-1 positive definite
+// (aCb)^2 <= aCa bCb, and aCa = Q - 2 oCb, so
+//   (aCb)^2 / Q - bCb <= bCb |2 oCb| / Q <= cut^2 m / Qmin,
+// m a bound of |2 oCb| over the window's ellipse (Dy / hy)^2 + (u / umax)^2 <= 1 (of
+// l1 Dy/hy + l2 u/umax at most hypot(l1, l2)) and Qmin = min aCa - m.  Infinite where
+// Qmin is not clearly positive.  The bound is some 1.2 times the largest value at
+// the paper's 350 mm radius, up to a few times at 130 mm.
+__device__ __forceinline__ float p_bound(const Geo& g, const EvSig& es, const float4& ev,
+                                         float log2K)
+{
+    const float t = fabsf(ev.z), c2i = ev.w;
+    const float hy = g.hy_coef * rsqrtf(c2i) * 1.001f + g.dy;
+    const float umax = sqrtf(g.cut2) * es.inv_sqrt_2iz + g.dz;
+    const float ymax = fabsf(ev.x) + hy;
+    const float gam = fabsf(g.gR8) * t * c2i * sqrtf(c2i);
+    const float lead = 2.0f * es.iz * g.R * g.R * c2i * c2i;
+    const float l1 = 4.0f * g.il * ymax * fmaf(2.0f * t, t, 1.0f) * hy * c2i + gam * hy;
+    const float l2 = 4.0f * es.iz * ymax * t * c2i * umax;
+    const float m = sqrtf(fmaf(l1, l1, l2 * l2)), q = lead - gam * ymax - m;
+    if (!(q > 1e-3f * lead)) return INFINITY;
+    return 1.001f * exp2f(fmaf(g.half_log2e * g.cut2, m / q, log2K)) * rsqrtf(q);
+}
 
 __device__ __forceinline__ void make_evc(const Geo& g, const EvSig& es, const float4& ev, int mid,
                                          float4* __restrict__ out)
@@ -51,8 +76,9 @@ __device__ __forceinline__ void make_evc(const Geo& g, const EvSig& es, const fl
     }
     out[0] = make_float4(yt, (float)mid, q0, q1);
     out[1] = make_float4(q2, -2.0f * iz2 * t, -iz2, il4 * t);
-    out[2] = make_float4(b2, g.half_log2e * il4, es.log2K, es.ksu);
-    out[3] = ev;
+    const float log2K = es.log2K - g.pshift;
+    out[2] = make_float4(b2, g.half_log2e * il4, log2K, es.ksu);
+    out[3] = make_float4(p_bound(g, es, ev, log2K), ev.y, t, c2i);
 }
 
 // Lane rows count outward from the middle of the window (see event_rows).
@@ -136,6 +162,13 @@ __device__ __forceinline__ void rec_wait()
     __syncwarp();
 }
 
+__device__ __forceinline__ float lds32(unsigned a)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+
 __device__ __forceinline__ float4 lds128(unsigned a)
 {
     float4 v;
@@ -201,22 +234,24 @@ __device__ __forceinline__ PairC rec_row(const Geo& g, const RecIn& x, float row
     return c;
 }
 
-// Pass 1 of the MLEM and log-likelihood forms: pairs 1 .. kmax, P rho' kept in
-// tensor memory (ST) and summed.  Chunks of eight and four pairs without any
+// Pass 1 of the MLEM and log-likelihood forms: pairs 1 .. kmax, P kept in tensor
+// memory (ST), P rho' summed.  GLD: the rho' region is the block's transposed one in
+// global memory, a pixel step a column of it.  Chunks of eight and four pairs without any
 // test up to kfast, then chunks of four and two that zero P beyond each
 // stream's last pair.  Returns the number of pairs stored.
-template <int TRAV, int LMAX, bool ST>
-__device__ __forceinline__ int rec_pass1(unsigned base, int la, int lb, const PairC& c, int kfast,
+template <int TRAV, int LMAX, bool ST, bool GLD, class Addr>
+__device__ __forceinline__ int rec_pass1(Addr base, int la, int lb, const PairC& c, int kfast,
                                          int kmax, float2& D2, unsigned tma)
 {
-    constexpr int s0 = 4 * pair_step0<TRAV>(), s1 = 4 * pair_step1<TRAV>();
-    unsigned a0 = base + (unsigned)(4 * pair_d0<TRAV>(1));
-    unsigned a1 = base + (unsigned)(4 * pair_d1<TRAV>(1));
+    constexpr int kStep = GLD ? 4 * kScrRows : 4;
+    constexpr int s0 = kStep * pair_step0<TRAV>(), s1 = kStep * pair_step1<TRAV>();
+    Addr a0 = base + (Addr)(long long)(kStep * pair_d0<TRAV>(1));
+    Addr a1 = base + (Addr)(long long)(kStep * pair_d1<TRAV>(1));
     float2 kk = make_float2((float)pair_d0<TRAV>(1), (float)pair_d1<TRAV>(1));
     unsigned col = tma;
     int k = 1;
 #define TSP_P1(PRED, J) \
-    p1_pair<true, false, PRED, true, (J) * s0, (J) * s1>(a0, a1, k + (J), la, lb, c, kk, D2)
+    p1_pair<!GLD, false, PRED, false, (J) * s0, (J) * s1>(a0, a1, k + (J), la, lb, c, kk, D2)
     if constexpr (LMAX >= 24) {
         for (; k + 7 <= kfast; k += 8) {
             float x[16];
@@ -230,8 +265,8 @@ __device__ __forceinline__ int rec_pass1(unsigned base, int la, int lb, const Pa
             t = TSP_P1(false, 6), x[12] = t.x, x[13] = t.y;
             t = TSP_P1(false, 7), x[14] = t.x, x[15] = t.y;
             if constexpr (ST) tm_st16(col, x);
-            a0 += (unsigned)(8 * s0);
-            a1 += (unsigned)(8 * s1);
+            a0 += (Addr)(long long)(8 * s0);
+            a1 += (Addr)(long long)(8 * s1);
             col += 16;
         }
     }
@@ -239,35 +274,55 @@ __device__ __forceinline__ int rec_pass1(unsigned base, int la, int lb, const Pa
         const float2 pa = TSP_P1(false, 0), pb = TSP_P1(false, 1);
         const float2 pc = TSP_P1(false, 2), pd = TSP_P1(false, 3);
         if constexpr (ST) tm_st8(col, pa.x, pa.y, pb.x, pb.y, pc.x, pc.y, pd.x, pd.y);
-        a0 += (unsigned)(4 * s0);
-        a1 += (unsigned)(4 * s1);
+        a0 += (Addr)(long long)(4 * s0);
+        a1 += (Addr)(long long)(4 * s1);
         col += 8;
     }
     for (; k + 2 <= kmax; k += 4) {
         const float2 pa = TSP_P1(true, 0), pb = TSP_P1(true, 1);
         const float2 pc = TSP_P1(true, 2), pd = TSP_P1(true, 3);
         if constexpr (ST) tm_st8(col, pa.x, pa.y, pb.x, pb.y, pc.x, pc.y, pd.x, pd.y);
-        a0 += (unsigned)(4 * s0);
-        a1 += (unsigned)(4 * s1);
+        a0 += (Addr)(long long)(4 * s0);
+        a1 += (Addr)(long long)(4 * s1);
         col += 8;
     }
     for (; k <= kmax; k += 2) {
         const float2 pa = TSP_P1(true, 0), pb = TSP_P1(true, 1);
         if constexpr (ST) tm_st4(col, pa.x, pa.y, pb.x, pb.y);
-        a0 += (unsigned)(2 * s0);
-        a1 += (unsigned)(2 * s1);
+        a0 += (Addr)(long long)(2 * s0);
+        a1 += (Addr)(long long)(2 * s1);
         col += 4;
     }
 #undef TSP_P1
     return k - 1;
 }
 
-// Pass 2 in fixed point (see kAccWords): the values of pairs 1 .. n (n a
-// multiple of two), 0 beyond each stream's last pair, scaled by s2 = 2^12 / D
-// and sl = 2^32 / D and added to the item's two-word accumulator (H words at
-// base).
+// Two pairs' terms (four pixels; pa = pair k, pb = pair k + 1) added to the words at
+// a0, a1, a0 + S0, a1 + S1.  s2 = 2^-149 / (D quantum): the product, rounded to
+// nearest, is a subnormal number (or in the first binade above, of the same
+// spacing), whose bits are the count of quanta, up to 2^24.
+template <int S0, int S1>
+__device__ __forceinline__ void add4(unsigned a0, unsigned a1, float2 pa, float2 pb, float2 s2)
+{
+    const float2 va = __fmul2_rn(pa, s2), vb = __fmul2_rn(pb, s2);
+#ifdef TSP_DEBUG_CHECKS
+    if (!(tsp_sh_ok(a0, 4, 2) && tsp_sh_ok(a1, 4, 2) && tsp_sh_ok(a0 + (unsigned)S0, 4, 2) &&
+          tsp_sh_ok(a1 + (unsigned)S1, 4, 2)))
+        return;
+#endif
+    asm volatile(
+        "red.shared.add.u32 [%0], %4;\n\tred.shared.add.u32 [%1], %5;\n\t"
+        "red.shared.add.u32 [%0+%2], %6;\n\tred.shared.add.u32 [%1+%3], %7;"
+        ::"r"(a0), "r"(a1), "n"(S0), "n"(S1),
+        "r"(__float_as_uint(va.x)), "r"(__float_as_uint(va.y)), "r"(__float_as_uint(vb.x)),
+        "r"(__float_as_uint(vb.y))
+        : "memory");
+}
+
+// Pass 2: the values of pairs 1 .. n (n a multiple of two), 0 beyond each stream's
+// last pair, added to the item's accumulator at base.
 template <int TRAV>
-__device__ __forceinline__ void rec_pass2(unsigned base, int n, unsigned tma, float2 s2, float2 sl)
+__device__ __forceinline__ void rec_pass2(unsigned base, int n, unsigned tma, float2 s2)
 {
     constexpr int s0 = 4 * pair_step0<TRAV>(), s1 = 4 * pair_step1<TRAV>();
     unsigned a0 = base + (unsigned)(4 * pair_d0<TRAV>(1));
@@ -278,13 +333,13 @@ __device__ __forceinline__ void rec_pass2(unsigned base, int n, unsigned tma, fl
         float x[16];
         tm_ld16(col, x);
         tm_wait_ld();
-        fx4<s0, s1>(a0, a1, make_float2(x[0], x[1]), make_float2(x[2], x[3]), s2, sl);
-        fx4<s0, s1>(a0 + (unsigned)(2 * s0), a1 + (unsigned)(2 * s1), make_float2(x[4], x[5]),
-                    make_float2(x[6], x[7]), s2, sl);
-        fx4<s0, s1>(a0 + (unsigned)(4 * s0), a1 + (unsigned)(4 * s1), make_float2(x[8], x[9]),
-                    make_float2(x[10], x[11]), s2, sl);
-        fx4<s0, s1>(a0 + (unsigned)(6 * s0), a1 + (unsigned)(6 * s1), make_float2(x[12], x[13]),
-                    make_float2(x[14], x[15]), s2, sl);
+        add4<s0, s1>(a0, a1, make_float2(x[0], x[1]), make_float2(x[2], x[3]), s2);
+        add4<s0, s1>(a0 + (unsigned)(2 * s0), a1 + (unsigned)(2 * s1), make_float2(x[4], x[5]),
+                     make_float2(x[6], x[7]), s2);
+        add4<s0, s1>(a0 + (unsigned)(4 * s0), a1 + (unsigned)(4 * s1), make_float2(x[8], x[9]),
+                     make_float2(x[10], x[11]), s2);
+        add4<s0, s1>(a0 + (unsigned)(6 * s0), a1 + (unsigned)(6 * s1), make_float2(x[12], x[13]),
+                     make_float2(x[14], x[15]), s2);
         a0 += (unsigned)(8 * s0);
         a1 += (unsigned)(8 * s1);
         col += 16;
@@ -293,9 +348,9 @@ __device__ __forceinline__ void rec_pass2(unsigned base, int n, unsigned tma, fl
         float x[8];
         tm_ld8(col, x);
         tm_wait_ld();
-        fx4<s0, s1>(a0, a1, make_float2(x[0], x[1]), make_float2(x[2], x[3]), s2, sl);
-        fx4<s0, s1>(a0 + (unsigned)(2 * s0), a1 + (unsigned)(2 * s1), make_float2(x[4], x[5]),
-                    make_float2(x[6], x[7]), s2, sl);
+        add4<s0, s1>(a0, a1, make_float2(x[0], x[1]), make_float2(x[2], x[3]), s2);
+        add4<s0, s1>(a0 + (unsigned)(2 * s0), a1 + (unsigned)(2 * s1), make_float2(x[4], x[5]),
+                     make_float2(x[6], x[7]), s2);
         a0 += (unsigned)(4 * s0);
         a1 += (unsigned)(4 * s1);
         col += 8;
@@ -305,7 +360,7 @@ __device__ __forceinline__ void rec_pass2(unsigned base, int n, unsigned tma, fl
         float x0, x1, x2, x3;
         tm_ld4(col, x0, x1, x2, x3);
         tm_wait_ld();
-        fx4<s0, s1>(a0, a1, make_float2(x0, x1), make_float2(x2, x3), s2, sl);
+        add4<s0, s1>(a0, a1, make_float2(x0, x1), make_float2(x2, x3), s2);
     }
 }
 
@@ -336,11 +391,10 @@ __device__ __forceinline__ float group_sum(float v, int G, int Gp, int wig, int 
 // event would show in their sum.
 struct GradSums {
     float2 m0, m1, m2, x0, x1, s0, s1;
-    float pmax;
 };
 
-template <bool PRED, int OFF0, int OFF1>
-__device__ __forceinline__ float2 p1g_pair(unsigned a0, unsigned a1, int k, int la, int lb,
+template <bool GLD, bool PRED, int OFF0, int OFF1, class Addr>
+__device__ __forceinline__ float2 p1g_pair(Addr a0, Addr a1, int k, int la, int lb,
                                            const PairC& c, const GradC& g, float2& kk,
                                            GradSums& m)
 {
@@ -367,8 +421,8 @@ __device__ __forceinline__ float2 p1g_pair(unsigned a0, unsigned a1, int k, int 
         p.y = k <= lb ? p.y : 0.0f;
     }
     float2 v;
-    v.x = ld_rhop<true, false, false, OFF0>(a0, k, la);
-    v.y = ld_rhop<true, false, false, OFF1>(a1, k, lb);
+    v.x = ld_rhop<!GLD, false, GLD && PRED, OFF0>(a0, k, la);
+    v.y = ld_rhop<!GLD, false, GLD && PRED, OFF1>(a1, k, lb);
     const float2 pv = __fmul2_rn(p, v), pvd = __fmul2_rn(pv, kk);
     const float2 iq = __fmul2_rn(rq, rq);
     const float2 X = __fmul2_rn(__ffma2_rn(kk, g.dB, g.B0), iq), S = __ffma2_rn(X, X, iq);
@@ -379,7 +433,6 @@ __device__ __forceinline__ float2 p1g_pair(unsigned a0, unsigned a1, int k, int 
     m.x1 = __ffma2_rn(pvd, X, m.x1);
     m.s0 = __ffma2_rn(pv, S, m.s0);
     m.s1 = __ffma2_rn(pvd, S, m.s1);
-    m.pmax = fmaxf(m.pmax, fmaxf(p.x, p.y));
     kk = __fadd2_rn(kk, c.inc);
     return p;
 }
@@ -387,31 +440,32 @@ __device__ __forceinline__ float2 p1g_pair(unsigned a0, unsigned a1, int k, int 
 // Gradient pass over pairs 1 .. kmax, P kept in tensor memory, two pairs a step
 // (the sums and constants leave no registers for more).  Returns the number of
 // pairs stored.
-template <int TRAV>
-__device__ __forceinline__ int rec_pass1_grad(unsigned base, int la, int lb, const PairC& c,
+template <int TRAV, bool GLD, class Addr>
+__device__ __forceinline__ int rec_pass1_grad(Addr base, int la, int lb, const PairC& c,
                                               const GradC& g, int kfast, int kmax, GradSums& m,
                                               unsigned tma)
 {
-    constexpr int s0 = 4 * pair_step0<TRAV>(), s1 = 4 * pair_step1<TRAV>();
-    unsigned a0 = base + (unsigned)(4 * pair_d0<TRAV>(1));
-    unsigned a1 = base + (unsigned)(4 * pair_d1<TRAV>(1));
+    constexpr int kStep = GLD ? 4 * kScrRows : 4;
+    constexpr int s0 = kStep * pair_step0<TRAV>(), s1 = kStep * pair_step1<TRAV>();
+    Addr a0 = base + (Addr)(long long)(kStep * pair_d0<TRAV>(1));
+    Addr a1 = base + (Addr)(long long)(kStep * pair_d1<TRAV>(1));
     float2 kk = make_float2((float)pair_d0<TRAV>(1), (float)pair_d1<TRAV>(1));
     unsigned col = tma;
     int k = 1;
     for (; k + 1 <= kfast; k += 2) {
-        const float2 pa = p1g_pair<false, 0, 0>(a0, a1, k, la, lb, c, g, kk, m);
-        const float2 pb = p1g_pair<false, s0, s1>(a0, a1, k + 1, la, lb, c, g, kk, m);
+        const float2 pa = p1g_pair<GLD, false, 0, 0>(a0, a1, k, la, lb, c, g, kk, m);
+        const float2 pb = p1g_pair<GLD, false, s0, s1>(a0, a1, k + 1, la, lb, c, g, kk, m);
         tm_st4(col, pa.x, pa.y, pb.x, pb.y);
-        a0 += (unsigned)(2 * s0);
-        a1 += (unsigned)(2 * s1);
+        a0 += (Addr)(long long)(2 * s0);
+        a1 += (Addr)(long long)(2 * s1);
         col += 4;
     }
     for (; k <= kmax; k += 2) {
-        const float2 pa = p1g_pair<true, 0, 0>(a0, a1, k, la, lb, c, g, kk, m);
-        const float2 pb = p1g_pair<true, s0, s1>(a0, a1, k + 1, la, lb, c, g, kk, m);
+        const float2 pa = p1g_pair<GLD, true, 0, 0>(a0, a1, k, la, lb, c, g, kk, m);
+        const float2 pb = p1g_pair<GLD, true, s0, s1>(a0, a1, k + 1, la, lb, c, g, kk, m);
         tm_st4(col, pa.x, pa.y, pb.x, pb.y);
-        a0 += (unsigned)(2 * s0);
-        a1 += (unsigned)(2 * s1);
+        a0 += (Addr)(long long)(2 * s0);
+        a1 += (Addr)(long long)(2 * s1);
         col += 4;
     }
     return k - 1;
@@ -443,32 +497,42 @@ __device__ __forceinline__ float2 rec_grad_row(const Geo& g, const float4& ev, f
     return make_float2(Ez * es.inv_f2, El);
 }
 
-// The scatter of an event whose largest P / D exceeds the gradient pass's fixed
-// point unit (see k_tiles_rec): float adds to the global A, each pixel under its
-// predicate.
-template <int TRAV>
-__device__ __forceinline__ void rec_scatter_global(const Inst& I, const Frame& f, unsigned idx,
-                                                   int la, int lb, int kmax, unsigned tma,
-                                                   float invD)
+// Room of the fixed-point accumulator (see k_tiles_rec), in quanta.
+constexpr float kTopTerm = 0.99f * 0x1p24f;   // one event's largest term
+constexpr float kRoom = 0.99f * 0x1p32f;      // all the events of an item
+
+// The scatter of an event whose terms the item's accumulator has no room for (see
+// k_tiles_rec): float adds to the global A, each pixel under its predicate; with
+// MASK only where rho' > 0 (as the flush does).
+template <int TRAV, bool MASK>
+__device__ __noinline__ void rec_scatter_global(float* A, const float* rhop, int pix, int la,
+                                                int lb, int n, unsigned tma, float invD)
 {
-    const int rr = (int)idx / f.stride, col = (int)idx - rr * f.stride;
-    const int iy = f.oy + rr;
-    const int iz = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0))) + col;
-    RowP<false> q;
-    q.base = (unsigned long long)(I.A + ((long long)iy * I.g.nz + iz));
-    q.gbase = 0;
-    q.la = la;
-    q.lb = lb;
-    pass2_pairs<TRAV, false>(q, 0, 0, kmax, tma, make_float2(invD, invD));
+    auto add = [&](int q, float p) {
+        if (p != 0.0f && (!MASK || rhop[q] > 0.0f)) atomicAdd(A + q, p * invD);
+    };
+    unsigned col = tma;
+    for (int k = 1; k <= n; k += 2) {
+        float x0, x1, x2, x3;
+        tm_ld4(col, x0, x1, x2, x3);
+        tm_wait_ld();
+        if (k <= la) add(pix + pair_d0<TRAV>(k), x0);
+        if (k <= lb) add(pix + pair_d1<TRAV>(k), x1);
+        if (k < la) add(pix + pair_d0<TRAV>(k + 1), x2);
+        if (k < lb) add(pix + pair_d1<TRAV>(k + 1), x3);
+        __syncwarp();
+        col += 4;
+    }
 }
 
 // The events first + grp, first + grp + ngroups, ... of an item, by one group
-// of G warps.  GRAD: inv_unit is 1 over the unit of the fixed-point terms P / D.
-template <int TRAV, int LMAX, int MODE, int NSEG>
+// of G warps.  inv_q: 1 over the quantum of the fixed-point terms P / D.
+template <int TRAV, int LMAX, int MODE, int NSEG, bool GLD>
 __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int first, int count,
                                            int grp, int ngroups, int wig, int lane,
                                            unsigned rp_addr, unsigned acc_off, unsigned slot,
-                                           float* part, BlockSums* bs, unsigned tma, float inv_unit)
+                                           float* part, BlockSums* bs, unsigned tma, float inv_q,
+                                           const float* scr)
 {
     constexpr bool GRAD = MODE == kGrad;
     const Geo& g = I.g;
@@ -492,6 +556,8 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
     const float4* ep = I.evs.evc + (size_t)(first + grp) * kEvcFloat4;
     rec_fetch(slot, rp, ep, lane);
     unsigned used = 0;
+    float spent = 0.0f;
+    const float room = kRoom / (float)ngroups;
     double logD = 0.0, giz = 0.0, gil = 0.0;
     int parity = 0;
     for (;;) {
@@ -505,8 +571,9 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
         const int la = (x.r.y >> 16) & 0xff, lb = x.r.y >> 24;
         const int kmax = __reduce_max_sync(0xffffffffu, max(la, lb));
         const int kfast = __reduce_min_sync(0xffffffffu, min(la, lb));
-        float4 ev;
+        float4 ev = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         if constexpr (GRAD) ev = lds128(slot + 304u);
+        else if (MODE != kLoglik) ev.x = lds32(slot + 304u);
         __syncwarp();   // every lane has its values: the slot may be refilled
         if (--left > 0) {
             rp += (size_t)ngroups * (32 * G);
@@ -514,37 +581,42 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
             rec_fetch(slot, rp, ep, lane);
         }
         int n;
-        float D, pmax = 0.0f;
+        float D;
+        using Addr = typename std::conditional<GLD, unsigned long long, unsigned>::type;
+        Addr rbase;
+        if constexpr (GLD) {
+            const int rr = (int)(x.a.y + rowoff) - f.oy;
+            const int off = min(max(rr, 0), f.rh - 1) * (1 - kScrRows * f.stride) + (int)idx * kScrRows;
+            rbase = (unsigned long long)(scr + off);
+        } else {
+            rbase = base;
+        }
         float2 E = make_float2(0.0f, 0.0f);
         if constexpr (GRAD) {
             GradSums m;
             m.m0 = m.m1 = m.m2 = m.x0 = m.x1 = m.s0 = m.s1 = make_float2(0.0f, 0.0f);
-            m.pmax = 0.0f;
-            n = rec_pass1_grad<TRAV>(base, la, lb, c, gc, kfast, kmax, m, tma);
+            n = rec_pass1_grad<TRAV, GLD>(rbase, la, lb, c, gc, kfast, kmax, m, tma);
             E = rec_grad_row(g, ev, y, Dy, u0, m);
             D = warp_sum(m.m0.x + m.m0.y);
             E.x = warp_sum(E.x);
             E.y = warp_sum(E.y);
-            // (bits of non-negative floats order as integers)
-            pmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m.pmax)));
         } else {
             float2 D2 = make_float2(0.0f, 0.0f);
-            n = rec_pass1<TRAV, LMAX, MODE != kLoglik>(base, la, lb, c, kfast, kmax, D2, tma);
+            n = rec_pass1<TRAV, LMAX, MODE != kLoglik, GLD>(rbase, la, lb, c, kfast, kmax, D2, tma);
             D = warp_sum(D2.x + D2.y);
         }
         if (MODE != kLoglik) tm_wait_st();
         if (G > 1) {
             if constexpr (GRAD) {
                 float4* sl = reinterpret_cast<float4*>(part) + (parity ? G : 0);
-                if (lane == 0) sl[wig] = make_float4(D, E.x, E.y, pmax);
+                if (lane == 0) sl[wig] = make_float4(D, E.x, E.y, 0.0f);
                 named_barrier(1 + grp, G * 32);
-                D = E.x = E.y = pmax = 0.0f;
+                D = E.x = E.y = 0.0f;
                 for (int w = 0; w < G; ++w) {
                     const float4 v = sl[w];
                     D += v.x;
                     E.x += v.y;
                     E.y += v.z;
-                    pmax = fmaxf(pmax, v.w);
                 }
             } else {
                 D = group_sum(D, G, Gp, wig, lane, 1 + grp, part + parity * Gp);
@@ -554,7 +626,7 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
         if (D > 0.0f) {
             ++used;
             if (MODE != kMlem && wig == 0 && lane == 0) {
-                logD += (double)logf(D);
+                logD += (double)logf(D) + (double)g.pshift * 0.69314718055994530942;
                 if (GRAD) {
                     giz += (double)(E.x / D);
                     gil += (double)(E.y / D);
@@ -562,12 +634,17 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
             }
             if (MODE != kLoglik) {
                 const float invD = 1.0f / D;
-                const float r = GRAD ? invD * inv_unit : invD;
-                if (!GRAD || pmax * r <= 1.0f) {
-                    const float s = r * 4096.0f, sl = r * 0x1p32f;
-                    rec_pass2<TRAV>(base + acc_off, n, tma, make_float2(s, s), make_float2(sl, sl));
+                const float s = invD * inv_q, top = s * ev.x;
+                if (top <= kTopTerm && spent + top + 1.0f <= room) {
+                    spent += top + 1.0f;
+                    const float q = s * 0x1p-149f;
+                    rec_pass2<TRAV>(base + acc_off, n, tma, make_float2(q, q));
                 } else {
-                    rec_scatter_global<TRAV>(I, f, idx, la, lb, kmax, tma, invD);
+                    const int rr = (int)idx / f.stride, col = (int)idx - rr * f.stride;
+                    const int iy = f.oy + rr;
+                    const int iz = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0))) + col;
+                    rec_scatter_global<TRAV, MODE == kMlem && !GLD>(I.A, I.rhop, iy * g.nz + iz, la,
+                                                                    lb, n, tma, invD);
                 }
             }
         }
@@ -588,16 +665,27 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
 // item of a block is its index, later ones come from the queue, asked for while
 // an item is worked on.
 //
-// The gradient pass needs sum P / D also where rho' = 0, so its terms are not the
-// bounded responsibilities P rho' / D.  It adds P / D in units of
-//   U = (N / sum rho') max(1, 64 npix / W)       (W: the list's window pixels):
-// N / sum rho' is the rho'-weighted mean of the result A (sum_l rho'_l A_l = N),
-// and with few events a single term is larger than that, on the average by up to
-// some 4 npix / W times.  The quantum U 2^-32 is far below the rounding of float
-// sums of the size of A; an event whose largest term exceeds U (its window
-// nearly empty of activity, or of a far brighter spot) is scattered by float adds
-// to global memory instead.  The largest P is taken from the evaluated values.
-template <int LMAX, int MODE, int NSEG, bool BATCH>
+// The scatter sums P / D in fixed point, one word a pixel, with native integer adds
+// (a float add to shared memory is a compare-and-swap loop).  The quantum is the
+// item's: events of a window's mean rho' r have a largest term of fx_peak / r, and
+// this term, with the region's mean for r, takes t = fx_bits bits (fewer when the item
+// has so many events that 2^t of each would fill more than an eighth of the word).  What an event
+// really adds at most, its bound of P over D, is known before it is added: an event
+// above 2^24 quanta, or one that the group's share of the word has no room left for
+// (with D 1/8 of the estimate at least for all of them), is scattered by float adds
+// to global memory instead, so no sum can overflow.  Two words of the
+// responsibilities P rho' / D, as in k_tiles, need no such estimate, but twice the
+// adds and five more packed operations a pair: 1e7 events at 1 mm 34.3 -> 30.4 ms,
+// five updates of 2e5 at 1 mm 5.07 -> 4.29 ms, three of 3e5 at 2 mm 1.57 -> 1.36 ms.
+//
+// GLD: the windows are too large to stage rho' beside the accumulator.  The block
+// writes the item's rho' region to its own part of global memory, transposed
+// (column-major, kScrRows rows): the lanes of a warp, neighbouring rows at the
+// same sheared column, then read neighbouring words, which a row-major image gives
+// one cache line each.  It stays in the L1 and L2 caches.  2e6 events at
+// 0.5 mm: 64.2 ms with the row-major image, float adds and rows set up in the pass,
+// 28.1 ms now.
+template <int LMAX, int MODE, int NSEG, bool BATCH, bool GLD>
 __global__ void __launch_bounds__(pass_threads(LMAX, MODE, NSEG, BATCH), 1)
 k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ items, int n_items,
             int* queue)
@@ -612,7 +700,7 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
     __shared__ BlockSums s_sums;
     __shared__ Inst s_inst;
     __shared__ unsigned s_tmem;
-    __shared__ float2 s_unit;
+    __shared__ float2 s_sum[kWarps];
     const Inst& I = BATCH ? s_inst : p;
 
     const int tid = threadIdx.x, lane = tid & 31;
@@ -654,8 +742,9 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
         const Geo& g = I.g;
         const Tiling& tl = I.tl;
         const int region = tl.RH * tl.RS;
-        float* const s_acc = s_rp + region + 2 * kPadFloats;
-        unsigned* const s_accL = reinterpret_cast<unsigned*>(s_acc) + kAccWords;
+        float* const s_acc = GLD ? s_rp : s_rp + region + 2 * kPadFloats;
+        unsigned* const s_cnt = reinterpret_cast<unsigned*>(s_acc);
+        float* const scr = GLD ? I.scratch + (size_t)blockIdx.x * tl.RS * kScrRows : nullptr;
         if (fresh) {
             // the slack around the regions is read (times P = 0) and added
             // zeros to by the unpredicated accesses: finite values
@@ -671,31 +760,56 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
                 for (int k = tid; k < kPartFloats; k += kThreads) s_part[k] = 0.0f;
         }
         const Frame f = tile_frame(g, tl, item.x);
-        for (int rr = warp; rr < tl.RH; rr += kWarps) {
-            const int iy = f.oy + rr;
-            const bool row_in = iy >= 0 && iy < g.ny;
-            const int z0row = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0)));
-            for (int cc = lane; cc < tl.RS; cc += 32) {
-                const int iz = z0row + cc;
-                float v = 0.0f;
-                if (row_in && cc < tl.RW && iz >= 0 && iz < g.nz)
-                    v = I.rhop[(size_t)iy * g.nz + iz];
-                s_rp[rr * tl.RS + cc] = v;
-                if (MODE != kLoglik) {
-                    s_acc[rr * tl.RS + cc] = 0.0f;
-                    s_accL[rr * tl.RS + cc] = 0u;
+        float sum = 0.0f;      // rho' over the region's pixels, and their number
+        int inside = 0;
+        if constexpr (GLD) {
+            if (MODE != kLoglik)
+                for (int k = tid; k < region; k += kThreads) s_cnt[k] = 0u;
+            // 32 rows of a run of columns a warp: the image's rows come through L1
+            const int nr = (tl.RH + 31) >> 5;
+            for (int k = warp; k < 4 * nr; k += kWarps) {
+                const int rr = (k >> 2) * 32 + lane, iy = f.oy + rr;
+                if (rr >= tl.RH) continue;
+                const bool row_in = iy >= 0 && iy < g.ny;
+                const int z0row = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0)));
+                const int w = (tl.RW + 3) >> 2, c1 = min(tl.RW, ((k & 3) + 1) * w);
+#pragma unroll 4
+                for (int cc = (k & 3) * w; cc < c1; ++cc) {
+                    const int iz = z0row + cc;
+                    float v = 0.0f;
+                    if (row_in && iz >= 0 && iz < g.nz) {
+                        v = I.rhop[(size_t)iy * g.nz + iz];
+                        ++inside;
+                    }
+                    scr[cc * kScrRows + rr] = v;
+                    sum += v;
+                }
+            }
+        } else {
+            for (int rr = warp; rr < tl.RH; rr += kWarps) {
+                const int iy = f.oy + rr;
+                const bool row_in = iy >= 0 && iy < g.ny;
+                const int z0row = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0)));
+                for (int cc = lane; cc < tl.RS; cc += 32) {
+                    const int iz = z0row + cc;
+                    float v = 0.0f;
+                    if (row_in && cc < tl.RW && iz >= 0 && iz < g.nz) {
+                        v = I.rhop[(size_t)iy * g.nz + iz];
+                        ++inside;
+                    }
+                    s_rp[rr * tl.RS + cc] = v;
+                    if (MODE != kLoglik) s_cnt[rr * tl.RS + cc] = 0u;
+                    sum += v;
                 }
             }
         }
+        if (MODE != kLoglik) {
+            sum = warp_sum(sum);
+            inside = __reduce_add_sync(0xffffffffu, inside);
+            if (lane == 0) s_sum[warp] = make_float2(sum, (float)inside);
+        }
         if (tid == 0) {
             s_item[par] = next;
-            if (MODE == kGrad) {
-                const double sum = I.accum->sum_rhop;
-                const float u = (float)(I.grad_unit / sum);
-                const bool ok = sum > 0.0 && u >= 1e-30f && u <= 1e30f;
-                // (no usable scale: every event takes the float scatter)
-                s_unit = ok ? make_float2(u, 1.0f / u) : make_float2(1.0f, INFINITY);
-            }
             // pixels that the records left out, counted once a pass
             if (item.y == 0) {
                 s_sums.qclip += I.accum->rec_qclip;
@@ -703,19 +817,29 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
             }
         }
         __syncthreads();
+        float quantum = 0.0f, inv_q = 0.0f;
+        if (MODE != kLoglik) {
+            static_assert(kWarps == 32, "a lane a warp's sum");
+            const float2 part = s_sum[lane];
+            const float mean = warp_sum(part.x) / warp_sum(part.y);
+            const int t = min(I.fx_bits, 29 - (32 - __clz(max(item.z - 1, 1))));
+            inv_q = mean / I.fx_peak * (float)(1 << t);
+            quantum = 1.0f / inv_q;
+            // (an image of no usable scale: every event takes the float scatter)
+            if (!(inv_q >= 1e-30f && inv_q <= 1e30f)) quantum = 0.0f, inv_q = INFINITY;
+        }
         {
             const int G = I.G;
             const int ngroups = group_count(kWarps, G);
             const int grp = warp / G, wig = warp - grp * G;
             float* part = s_part + grp * (kPartFloats / kWarps) * G;
             const unsigned rp_addr = (unsigned)__cvta_generic_to_shared(s_rp);
-            const unsigned acc_off = 4u * (unsigned)(region + 2 * kPadFloats);
+            const unsigned acc_off = GLD ? 0u : 4u * (unsigned)(region + 2 * kPadFloats);
             const unsigned slot =
                 (unsigned)__cvta_generic_to_shared(smem + kPartFloats + warp * kRecSlotFloats);
-            const float inv_unit = MODE == kGrad ? s_unit.y : 0.0f;
 #define TSP_REC_EVENTS(TRAV) \
-    rec_events<TRAV, LMAX, MODE, NSEG>(I, f, item.y, item.z, grp, ngroups, wig, lane, rp_addr, \
-                                       acc_off, slot, part, &s_sums, tma, inv_unit)
+    rec_events<TRAV, LMAX, MODE, NSEG, GLD>(I, f, item.y, item.z, grp, ngroups, wig, lane, rp_addr, \
+                                       acc_off, slot, part, &s_sums, tma, inv_q, scr)
             if (grp < ngroups) {
                 if (NSEG == 1)
                     TSP_REC_EVENTS(kAlt);
@@ -737,17 +861,9 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
                 for (int cc = lane; cc < tl.RW; cc += 32) {
                     const int iz = z0row + cc;
                     const int k = rr * tl.RS + cc;
-                    // A += X / rho' (the fixed-point sums, see kAccWords)
-                    const unsigned wh = __float_as_uint(s_acc[k]), wl = s_accL[k];
-                    const unsigned sh = wh & 0xFFFFFFu, sl = wl - (wh & 0xFF000000u);
-                    const float X = fmaf((float)sl, 0x1p-32f, (float)sh * 0x1p-12f);
-                    float v;
-                    if (MODE == kGrad) {
-                        v = X * s_unit.x;           // terms P / D in units of s_unit.x
-                    } else {
-                        const float rp = s_rp[k];
-                        v = rp > 0.0f ? X / rp : 0.0f;
-                    }
+                    float v = (float)s_cnt[k] * quantum;
+                    // (the update is 0 where rho' = 0, whatever A holds)
+                    if (MODE == kMlem && !GLD && !(s_rp[k] > 0.0f)) v = 0.0f;
                     if (iz >= 0 && iz < g.nz && v != 0.0f)
                         atomicAdd(I.A + (size_t)iy * g.nz + iz, v);
                 }

@@ -183,7 +183,10 @@ extern "C" int tsp_mlem_update_noalloc(const tsp_params* params, const float* zu
     a.rhop = rhop;
     a.A = A;
     a.accum = accum;
-    a.grad_unit = 0.0;
+    a.fx_peak = 0.0f;
+    a.fx_bits = 0;
+    a.scratch = nullptr;
+    a.rec_smem = 0;
     a.G = G;
     a.nseg = nseg;
     a.gld = 0;
