@@ -194,6 +194,8 @@ constexpr int kPartFloats = 12 * kMaxWarps;
 // Shared staging of a warp's next window records (256 bytes) and of its event's
 // coefficients (64), in floats (tsp_rec.cuh).
 constexpr int kRecSlotFloats = 80;
+// With two rows a lane: 512 bytes of records, the coefficients of two events.
+__host__ __device__ constexpr int rec_slot_floats(bool two) { return two ? 160 : kRecSlotFloats; }
 __host__ __device__ constexpr size_t tiles_smem_floats(int RH, int RS)
 {
     return (size_t)kPadFloats + (size_t)RH * RS + 2 * kPadFloats + (size_t)kAccWords +
@@ -205,7 +207,7 @@ __host__ __device__ constexpr size_t tiles_smem_floats(int RH, int RS)
 // `gld`) and the one-word accumulator, each with kPadFloats of slack around it.
 __host__ __device__ constexpr size_t rec_smem_floats(int RH, int RS, bool gld)
 {
-    return (size_t)kPartFloats + kMaxWarps * kRecSlotFloats +
+    return (size_t)kPartFloats + kMaxWarps * rec_slot_floats(!gld) +
            (gld ? 1 : 2) * ((size_t)RH * RS + 2 * kPadFloats);
 }
 

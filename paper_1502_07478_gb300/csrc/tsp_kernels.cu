@@ -557,7 +557,7 @@ cudaError_t launch_batch_pass(int lmax, int mode, const BatchArgs& a, cudaStream
     if (cudaError_t f = sim_launch()) return f;
     switch (lmax) {
     case 12: return launch_batch_pass_l<12>(mode, a, st);
-    case 24: return launch_batch_pass_l<24>(mode, a, st);
+    case 32: return launch_batch_pass_l<32>(mode, a, st);
     case 48: return launch_batch_pass_l<48>(mode, a, st);
     case 64: return launch_batch_pass_l<64>(mode, a, st);
     default: return cudaErrorInvalidValue;
@@ -568,7 +568,7 @@ cudaError_t prepare_batch_pass(int lmax, size_t smem)
 {
     switch (lmax) {
     case 12: return prepare_batch_pass_l<12>(smem);
-    case 24: return prepare_batch_pass_l<24>(smem);
+    case 32: return prepare_batch_pass_l<32>(smem);
     case 48: return prepare_batch_pass_l<48>(smem);
     case 64: return prepare_batch_pass_l<64>(smem);
     default: return cudaErrorInvalidValue;
@@ -580,7 +580,7 @@ cudaError_t launch_pass(int lmax, int mode, const PassArgs& a, cudaStream_t st)
     if (cudaError_t f = sim_launch()) return f;
     switch (lmax) {
     case 12: return launch_pass_l<12>(mode, a, st);
-    case 24: return launch_pass_l<24>(mode, a, st);
+    case 32: return launch_pass_l<32>(mode, a, st);
     case 48: return launch_pass_l<48>(mode, a, st);
     case 64: return launch_pass_l<64>(mode, a, st);
     default: return cudaErrorInvalidValue;
@@ -592,7 +592,7 @@ cudaError_t launch_records(int lmax, const RecArgs& a, cudaStream_t st)
     if (cudaError_t f = sim_launch()) return f;
     switch (lmax) {
     case 12: return launch_records_l<12>(a, st);
-    case 24: return launch_records_l<24>(a, st);
+    case 32: return launch_records_l<32>(a, st);
     case 48: return launch_records_l<48>(a, st);
     case 64: return launch_records_l<64>(a, st);
     default: return cudaErrorInvalidValue;
@@ -603,7 +603,7 @@ cudaError_t prepare_pass(int lmax, int mode, size_t smem)
 {
     switch (lmax) {
     case 12: return prepare_pass_l<12>(mode, smem);
-    case 24: return prepare_pass_l<24>(mode, smem);
+    case 32: return prepare_pass_l<32>(mode, smem);
     case 48: return prepare_pass_l<48>(mode, smem);
     case 64: return prepare_pass_l<64>(mode, smem);
     default: return cudaErrorInvalidValue;

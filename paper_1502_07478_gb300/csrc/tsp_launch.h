@@ -48,7 +48,7 @@ cudaError_t dmalloc(T** p, size_t bytes)
 }
 
 // Lane capacities (pixels of one row segment a lane walks) compiled in.
-constexpr int kLmaxList[] = {12, 24, 48, 64};
+constexpr int kLmaxList[] = {12, 32, 48, 64};
 constexpr int kLmaxCount = 4;
 
 // Lane layout of a parameter set's windows, shared by the context planner and

@@ -660,6 +660,324 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
     }
 }
 
+// ---- Two rows a lane -----------------------------------------------------------
+//
+// The MLEM and log-likelihood passes of chords up to 32 pixels: a lane takes two rows, the
+// neighbours of the lane-row order (mid - p and mid + p + 1, of about the same
+// length), as the two components of the packed operations.  An event of up to 32
+// rows (4 mm grids) then takes half a warp, one of 64 (2 mm) one warp and no
+// barrier, where a row a lane took twice as much; its pairs take the same time, but
+// what is done once a warp and event (record, constants, reductions, 1/D, loop
+// control: some 250 instructions of the 370 that an event of a 4 mm grid took) is
+// halved.  Longer chords have no room: a lane has 64 tensor-memory columns.
+//   1e7 events at 4 mm 3.38 -> 2.96 ms, three updates of 3e5 at 2 mm (chords of 25
+//   pixels) 1.36 -> 1.15 ms, 1e6 from host buffers at 2 mm (three updates and the
+//   log-likelihood) 6.53 -> 5.68 ms, mixed batch 18.15 -> 17.99 ms.
+// The gradient pass keeps a row a lane: with two, and its sums, 64 registers a thread
+// spill (1e6 events at 2 mm 3.30 -> 4.37 ms).
+// A window of an odd number of 32-row blocks above one keeps a row a lane: with two it
+// would leave a quarter of the lanes idle and every step predicated (12 mixed
+// reconstructions, one in three of them of such windows: 18.7 ms with two rows a lane
+// for all that their chords allow, 18.0 ms with this rule).
+// Step k of a row is the pixels at k and 1 - k from its origin, as with kAlt.
+
+__device__ __forceinline__ bool two_rows_fit(int G) { return G == 1 || (G & 1) == 0; }
+
+__host__ __device__ constexpr bool two_rows(int lmax, int mode, int nseg, bool gld)
+{
+    return lmax <= 32 && mode != kGrad && nseg == 1 && !gld;
+}
+
+// 1/D to float precision (one Newton step); not finite or 0 where D is far out of
+// range, which the caller's test of the largest term excludes.
+__device__ __forceinline__ float recip(float D)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(D));
+    return fmaf(r, fmaf(-D, r, 1.0f), r);
+}
+
+// The two rows' constants (.x, .y): see rec_row.
+struct Row2 {
+    float2 Q0, dQ, A0, dA, e0, e1, e2;
+};
+
+__device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
+
+__device__ __forceinline__ Row2 rec_row2(const Geo& g, const RecIn& x, float2 rowoff, float2 u0)
+{
+    const float2 y = __ffma2_rn(__fadd2_rn(dup(x.a.y), rowoff), dup(g.dy), dup(g.y0));
+    const float2 Dy = __fadd2_rn(y, dup(-x.a.x));
+    const float2 Qc = __ffma2_rn(y, __ffma2_rn(dup(x.b.x), y, dup(x.a.w)), dup(x.a.z));
+    const float2 gam = __fmul2_rn(dup(x.b.y), y), al = __fmul2_rn(dup(x.b.z), y);
+    const float2 be = __fmul2_rn(Dy, __ffma2_rn(dup(x.b.w), y, dup(x.c.x)));
+    Row2 c;
+    c.Q0 = __ffma2_rn(gam, u0, Qc);
+    c.dQ = __fmul2_rn(gam, dup(g.dz));
+    c.A0 = __fmul2_rn(__ffma2_rn(al, u0, be), dup(g.kA));
+    c.dA = __fmul2_rn(al, dup(g.dz * g.kA));
+    const float2 C0 = __ffma2_rn(__fmul2_rn(dup(-x.c.y), Dy), Dy, dup(x.c.z));
+    const float2 su0 = __fmul2_rn(dup(x.c.w), u0);
+    const float dsu = x.c.w * g.dz;
+    c.e0 = __ffma2_rn(make_float2(-su0.x, -su0.y), su0, C0);
+    c.e1 = __fmul2_rn(su0, dup(-2.0f * dsu));
+    c.e2 = dup(-(dsu * dsu));
+    return c;
+}
+
+// One pixel of each row, at kk from the origins: P, 0 beyond the rows' ends (in0, in1).
+template <int OFF>
+__device__ __forceinline__ float2 p2_eval(unsigned a0, unsigned a1, bool in0, bool in1, float2 kk,
+                                          const Row2& c, float2& D2)
+{
+    const float2 q = __ffma2_rn(kk, c.dQ, c.Q0);
+    // (with 1/sqrt(Q) set to 0 everything after it is finite)
+    const float r0 = rsqrt_approx(q.x), r1 = rsqrt_approx(q.y);
+    const float2 rq = make_float2(in0 ? r0 : 0.0f, in1 ? r1 : 0.0f);
+    const float2 a = __ffma2_rn(kk, c.dA, c.A0);
+    const float2 e = __ffma2_rn(kk, __ffma2_rn(kk, c.e2, c.e1), c.e0);
+    const float2 w = __fmul2_rn(a, rq);
+    const float2 h = __ffma2_rn(w, w, e);
+    const float2 p = __fmul2_rn(rq, make_float2(ex2_approx(h.x), ex2_approx(h.y)));
+    float2 v;
+    v.x = ld_rhop<true, false, false, OFF>(a0, 0, 0);
+    v.y = ld_rhop<true, false, false, OFF>(a1, 0, 0);
+    D2 = __ffma2_rn(p, v, D2);
+    return p;
+}
+
+// Pass 1, steps 1 .. kmax.  a0, a1: addresses of the rows' origins.
+template <int MODE>
+__device__ __forceinline__ void rec2_pass1(unsigned a0, unsigned a1, int la0, int lb0, int la1,
+                                           int lb1, const Row2& c, int kmax, float2& D2,
+                                           unsigned tma)
+{
+    const float2 one = dup(1.0f), mone = dup(-1.0f);
+    float2 kp = one, km = dup(0.0f);
+    unsigned u0 = a0 + 4u, u1 = a1 + 4u, d0 = a0, d1 = a1, col = tma;
+    auto step = [&](auto J, int k, float2& pu, float2& pd) {
+        constexpr int j = decltype(J)::value;
+        const bool i0 = k + j <= la0, i1 = k + j <= la1, j0 = k + j <= lb0, j1 = k + j <= lb1;
+        pu = p2_eval<4 * j>(u0, u1, i0, i1, kp, c, D2);
+        pd = p2_eval<-4 * j>(d0, d1, j0, j1, km, c, D2);
+        kp = __fadd2_rn(kp, one);
+        km = __fadd2_rn(km, mone);
+    };
+    int k = 1;
+    for (; k + 1 <= kmax; k += 2) {
+        float2 p, q, r, s;
+        step(std::integral_constant<int, 0>{}, k, p, q);
+        step(std::integral_constant<int, 1>{}, k, r, s);
+        if (MODE != kLoglik) tm_st8(col, p.x, p.y, q.x, q.y, r.x, r.y, s.x, s.y);
+        u0 += 8u;
+        u1 += 8u;
+        d0 -= 8u;
+        d1 -= 8u;
+        col += 8;
+    }
+    if (k <= kmax) {
+        float2 p, q;
+        step(std::integral_constant<int, 0>{}, k, p, q);
+        if (MODE != kLoglik) tm_st4(col, p.x, p.y, q.x, q.y);
+    }
+}
+
+// The terms of one step (p at k, q at 1 - k): counts of quanta (see add4).
+template <int OFF>
+__device__ __forceinline__ void add2x2(unsigned u0, unsigned u1, unsigned d0, unsigned d1, float2 p,
+                                       float2 q, float2 s2)
+{
+    const float2 vp = __fmul2_rn(p, s2), vq = __fmul2_rn(q, s2);
+#ifdef TSP_DEBUG_CHECKS
+    if (!(tsp_sh_ok(u0 + (unsigned)OFF, 4, 2) && tsp_sh_ok(u1 + (unsigned)OFF, 4, 2) &&
+          tsp_sh_ok(d0 - (unsigned)OFF, 4, 2) && tsp_sh_ok(d1 - (unsigned)OFF, 4, 2)))
+        return;
+#endif
+    asm volatile(
+        "red.shared.add.u32 [%0+%4], %6;\n\tred.shared.add.u32 [%1+%4], %7;\n\t"
+        "red.shared.add.u32 [%2+%5], %8;\n\tred.shared.add.u32 [%3+%5], %9;"
+        ::"r"(u0), "r"(u1), "r"(d0), "r"(d1), "n"(OFF), "n"(-OFF),
+        "r"(__float_as_uint(vp.x)), "r"(__float_as_uint(vp.y)), "r"(__float_as_uint(vq.x)),
+        "r"(__float_as_uint(vq.y))
+        : "memory");
+}
+
+// Pass 2, steps 1 .. n, into the item's accumulator.
+__device__ __forceinline__ void rec2_pass2(unsigned a0, unsigned a1, int n, unsigned tma, float2 s2)
+{
+    unsigned u0 = a0 + 4u, u1 = a1 + 4u, d0 = a0, d1 = a1, col = tma;
+    for (; n >= 4; n -= 4) {
+        float x[16];
+        tm_ld16(col, x);
+        tm_wait_ld();
+        add2x2<0>(u0, u1, d0, d1, make_float2(x[0], x[1]), make_float2(x[2], x[3]), s2);
+        add2x2<4>(u0, u1, d0, d1, make_float2(x[4], x[5]), make_float2(x[6], x[7]), s2);
+        add2x2<8>(u0, u1, d0, d1, make_float2(x[8], x[9]), make_float2(x[10], x[11]), s2);
+        add2x2<12>(u0, u1, d0, d1, make_float2(x[12], x[13]), make_float2(x[14], x[15]), s2);
+        u0 += 16u;
+        u1 += 16u;
+        d0 -= 16u;
+        d1 -= 16u;
+        col += 16;
+    }
+    if (n >= 2) {
+        float x[8];
+        tm_ld8(col, x);
+        tm_wait_ld();
+        add2x2<0>(u0, u1, d0, d1, make_float2(x[0], x[1]), make_float2(x[2], x[3]), s2);
+        add2x2<4>(u0, u1, d0, d1, make_float2(x[4], x[5]), make_float2(x[6], x[7]), s2);
+        u0 += 8u;
+        u1 += 8u;
+        d0 -= 8u;
+        d1 -= 8u;
+        col += 8;
+        n -= 2;
+    }
+    if (n >= 1) {
+        float x0, x1, x2, x3;
+        tm_ld4(col, x0, x1, x2, x3);
+        tm_wait_ld();
+        add2x2<0>(u0, u1, d0, d1, make_float2(x0, x1), make_float2(x2, x3), s2);
+    }
+}
+
+// The scatter of rows that the item's accumulator has no room for (see
+// rec_scatter_global); live: the lane's event is one of those.
+template <bool MASK>
+__device__ __noinline__ void rec2_scatter_global(float* A, const float* rhop, int p0, int p1,
+                                                 int la0, int lb0, int la1, int lb1, int n,
+                                                 unsigned tma, float invD, bool live)
+{
+    auto add = [&](int q, float p) {
+        if (p != 0.0f && (!MASK || rhop[q] > 0.0f)) atomicAdd(A + q, p * invD);
+    };
+    for (int k = 1; k <= n; ++k) {
+        float x0, x1, x2, x3;
+        tm_ld4(tma, x0, x1, x2, x3);
+        tm_wait_ld();
+        if (live) {
+            if (k <= la0) add(p0 + k, x0);
+            if (k <= la1) add(p1 + k, x1);
+            if (k <= lb0) add(p0 + 1 - k, x2);
+            if (k <= lb1) add(p1 + 1 - k, x3);
+        }
+        __syncwarp();
+        tma += 4;
+    }
+}
+
+// The events of an item for this warp: with G = 1 (up to 32 rows) a half warp
+// each, else groups of (G + 1) / 2 warps.
+template <int MODE>
+__device__ __forceinline__ void rec2_events(const Inst& I, const Frame& f, int first, int count,
+                                            int warp, int lane, unsigned rp_addr, unsigned acc_off,
+                                            unsigned slot, float* s_part, BlockSums* bs,
+                                            unsigned tma, float inv_q)
+{
+    const Geo& g = I.g;
+    const int G = I.G;
+    const bool halves = G == 1;
+    const int G2 = (G + 1) >> 1;
+    const int wgrp = warp / G2, wig = warp - wgrp * G2;
+    const int ngroups = halves ? 2 * kMaxWarps : group_count(kMaxWarps, G2);
+    // group, and pair of rows (the row block of a warp is rotated by its group)
+    const int grp = halves ? 2 * warp + (lane >> 4) : wgrp;
+    int blk = wig + wgrp % G2;
+    blk -= blk >= G2 ? G2 : 0;
+    int p = halves ? lane & 15 : blk * 32 + lane;
+    const bool has_rows = p < 16 * G;
+    const float2 rowoff = make_float2((float)-p, (float)(p + 1));
+    p = min(p, 16 * G - 1);
+    // events left of the warp's first group (the second half's may end one sooner)
+    const int lead = halves ? 2 * warp : wgrp;
+    if (!halves && wgrp >= ngroups) return;
+    int left = (count - lead + ngroups - 1) / ngroups;
+    if (left <= 0) return;
+    int e = grp;
+    const uint4* const recs = reinterpret_cast<const uint4*>(I.evs.recs) + p;
+    const float4* const evc = I.evs.evc;
+    const int cl = halves ? lane & 15 : lane;
+    const unsigned cslot = slot + 512u + (halves ? (lane >> 4) * 64u : 0u);
+    auto fetch = [&](int ev) {
+        const long long j = first + min(ev, count - 1);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot + 16u * lane),
+                     "l"(recs + j * (16 * G))
+                     : "memory");
+        if (cl < kEvcFloat4)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(cslot + 16u * cl),
+                         "l"(evc + j * kEvcFloat4 + cl)
+                         : "memory");
+    };
+    fetch(e);
+    const int Gp = G2 > 1 ? 1 << (32 - __clz(G2 - 1)) : 1;
+    float* const part = s_part + wgrp * (kPartFloats / kMaxWarps) * G2;
+    int parity = 0;
+    unsigned used = 0;
+    float spent = 0.0f;
+    const float room = kRoom / (float)ngroups;
+    double logD = 0.0;
+    for (;;) {
+        RecIn x;
+        unsigned w[4];
+        rec_wait();
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(slot + 16u * lane)
+                     : "memory");
+        x.a = lds128(cslot);
+        x.b = lds128(cslot + 16u);
+        x.c = lds128(cslot + 32u);
+        const float pmax = lds32(cslot + 48u);
+        const bool live = e < count && has_rows;
+        __syncwarp();   // every lane has its values: the slot may be refilled
+        e += ngroups;
+        if (--left > 0) fetch(e);
+        const float2 u0 = make_float2(__uint_as_float(w[0]), __uint_as_float(w[2]));
+        const unsigned i0 = w[1] & 0xffffu, i1 = w[3] & 0xffffu;
+        const unsigned n0 = live ? w[1] >> 16 : 0u, n1 = live ? w[3] >> 16 : 0u;
+        const int la0 = n0 & 0xff, lb0 = n0 >> 8, la1 = n1 & 0xff, lb1 = n1 >> 8;
+        const int kmax = __reduce_max_sync(0xffffffffu, max(max(la0, lb0), max(la1, lb1)));
+        const unsigned a0 = rp_addr + 4u * i0, a1 = rp_addr + 4u * i1;
+        float2 D2 = make_float2(0.0f, 0.0f);
+        rec2_pass1<MODE>(a0, a1, la0, lb0, la1, lb1, rec_row2(g, x, rowoff, u0), kmax, D2, tma);
+        float D = D2.x + D2.y;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) D += __shfl_xor_sync(0xffffffffu, D, o);
+        if (!halves) D += __shfl_xor_sync(0xffffffffu, D, 16);
+        if (MODE != kLoglik) tm_wait_st();
+        if (G2 > 1) {
+            D = group_sum(D, G2, Gp, wig, lane, 1 + wgrp, part + parity * Gp);
+            parity ^= 1;
+        }
+        const bool on = D > 0.0f;
+        if (on) {
+            ++used;
+            if (MODE != kMlem && (halves ? (lane & 15) == 0 : wig == 0 && lane == 0))
+                logD += (double)logf(D) + (double)g.pshift * 0.69314718055994530942;
+        }
+        if (MODE != kLoglik) {
+            const float r = recip(D), s = r * inv_q, top = s * pmax;
+            // (false for a NaN, and for a D that recip has no value of)
+            const bool fit = on && top > 0.0f && top <= kTopTerm && spent + top + 1.0f <= room;
+            if (fit) spent += top + 1.0f;
+            if (__any_sync(0xffffffffu, fit))
+                rec2_pass2(a0 + acc_off, a1 + acc_off, kmax, tma, dup(fit ? s * 0x1p-149f : 0.0f));
+            if (__any_sync(0xffffffffu, on && !fit)) {
+                auto pix = [&](unsigned i) {
+                    const int rr = (int)i / f.stride, iy = f.oy + rr;
+                    return iy * g.nz + f.zbase +
+                           (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0))) + (int)i - rr * f.stride;
+                };
+                rec2_scatter_global<MODE == kMlem>(I.A, I.rhop, pix(i0), pix(i1), la0, lb0, la1,
+                                                   lb1, kmax, tma, 1.0f / D, on && !fit);
+            }
+        }
+        if (left == 0) break;
+    }
+    if (used && (halves ? (lane & 15) == 0 : wig == 0 && lane == 0))
+        atomicAdd(&bs->used, (unsigned long long)used);
+    if (MODE != kMlem && logD != 0.0) atomicAdd(&bs->logD, logD);
+}
+
 // Persistent tile kernel over window records.  Work
 // items, batches and the two-word accumulator are those of k_tiles; the first
 // item of a block is its index, later ones come from the queue, asked for while
@@ -692,10 +1010,13 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
 {
     constexpr int kThreads = pass_threads(LMAX, MODE, NSEG, BATCH);
     constexpr int kWarps = kThreads / 32;
+    constexpr bool kTwo = two_rows(LMAX, MODE, NSEG, GLD);
+    constexpr int kSlot = rec_slot_floats(kTwo);
+    constexpr int kTm = kTwo ? 2 * LMAX : LMAX;    // tensor-memory columns of a lane
     extern __shared__ float4 smem_f4[];
     float* const smem = reinterpret_cast<float*>(smem_f4);
     float* const s_part = smem;
-    float* const s_rp = smem + kPartFloats + kMaxWarps * kRecSlotFloats + kPadFloats;
+    float* const s_rp = smem + kPartFloats + kMaxWarps * kSlot + kPadFloats;
     __shared__ int s_item[2];
     __shared__ BlockSums s_sums;
     __shared__ Inst s_inst;
@@ -705,7 +1026,7 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
 
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-    constexpr int kCols = tm_block_cols(LMAX, kWarps);
+    constexpr int kCols = tm_block_cols(kTm, kWarps);
     if (warp == 0) tm_alloc<kCols>(&s_tmem);
     init_block_sums(&s_sums);
 #ifdef TSP_DEBUG_CHECKS
@@ -716,7 +1037,7 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
     int cur = -1, it = blockIdx.x, par = 0;
     bool fresh = true;
     tm_sync_threads();
-    const unsigned tma = tm_thread_addr<LMAX>(s_tmem, warp);
+    const unsigned tma = tm_thread_addr<kTm>(s_tmem, warp);
 
     while (it < n_items) {
         int next = 0;
@@ -829,18 +1150,22 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
             if (!(inv_q >= 1e-30f && inv_q <= 1e30f)) quantum = 0.0f, inv_q = INFINITY;
         }
         {
+            const unsigned rp_addr = (unsigned)__cvta_generic_to_shared(s_rp);
+            const unsigned acc_off = GLD ? 0u : 4u * (unsigned)(region + 2 * kPadFloats);
+            const unsigned slot =
+                (unsigned)__cvta_generic_to_shared(smem + kPartFloats + warp * kSlot);
             const int G = I.G;
             const int ngroups = group_count(kWarps, G);
             const int grp = warp / G, wig = warp - grp * G;
             float* part = s_part + grp * (kPartFloats / kWarps) * G;
-            const unsigned rp_addr = (unsigned)__cvta_generic_to_shared(s_rp);
-            const unsigned acc_off = GLD ? 0u : 4u * (unsigned)(region + 2 * kPadFloats);
-            const unsigned slot =
-                (unsigned)__cvta_generic_to_shared(smem + kPartFloats + warp * kRecSlotFloats);
 #define TSP_REC_EVENTS(TRAV) \
     rec_events<TRAV, LMAX, MODE, NSEG, GLD>(I, f, item.y, item.z, grp, ngroups, wig, lane, rp_addr, \
-                                       acc_off, slot, part, &s_sums, tma, inv_q, scr)
-            if (grp < ngroups) {
+                                            acc_off, slot, part, &s_sums, tma, inv_q, scr)
+            if (kTwo && two_rows_fit(G)) {
+                if constexpr (kTwo)
+                    rec2_events<MODE>(I, f, item.y, item.z, warp, lane, rp_addr, acc_off, slot,
+                                      s_part, &s_sums, tma, inv_q);
+            } else if (grp < ngroups) {
                 if (NSEG == 1)
                     TSP_REC_EVENTS(kAlt);
                 else if ((wig & 1) == 0)
