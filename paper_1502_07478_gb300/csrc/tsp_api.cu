@@ -170,10 +170,13 @@ int plan(tsp_ctx* c)
     // to this context's size, which could lower it below another context's).
     const size_t limit = dyn_smem_limit(c->dev);
     if (c->smem > limit) return fail(c, TSP_EINVAL, "tile region exceeds the shared memory");
-    for (int mode = 0; mode < 3; ++mode) {
-        cudaError_t e = prepare_pass(c->lmax, mode, limit);
-        if (e != cudaSuccess)
-            return fail(c, TSP_ECUDA, std::string("prepare_pass: ") + cudaGetErrorString(e));
+    if (!(c->prepared >> (c->lmax - 1) & 1)) {
+        for (int mode = 0; mode < 3; ++mode) {
+            cudaError_t e = prepare_pass(c->lmax, mode, limit);
+            if (e != cudaSuccess)
+                return fail(c, TSP_ECUDA, std::string("prepare_pass: ") + cudaGetErrorString(e));
+        }
+        c->prepared |= 1ull << (c->lmax - 1);
     }
     return TSP_OK;
 }
@@ -282,14 +285,18 @@ PassArgs pass_args(tsp_ctx* c)
 int prep_begin(tsp_ctx* c, cudaStream_t st)
 {
     const int nbins = c->nbins;
-    dfree(c->bin_count);
-    dfree(c->offsets);
-    dfree(c->cursor);
-    TSP_CUDA(c, dmalloc(&c->bin_count, sizeof(int) * nbins));
-    TSP_CUDA(c, dmalloc(&c->offsets, sizeof(long long) * nbins));
-    TSP_CUDA(c, dmalloc(&c->cursor, sizeof(int) * nbins));
-    TSP_CUDA(c, cudaMemsetAsync(c->bin_count, 0, sizeof(int) * nbins, st));
-    TSP_CUDA(c, cudaMemsetAsync(c->cursor, 0, sizeof(int) * nbins, st));
+    if (nbins > c->bins_cap) {
+        dfree(c->bin_count);
+        dfree(c->offsets);
+        c->bins_cap = 0;
+        TSP_CUDA(c, dmalloc(&c->bin_count, 2 * sizeof(int) * nbins));
+        TSP_CUDA(c, dmalloc(&c->offsets, sizeof(long long) * nbins));
+        c->bins_cap = nbins;
+    }
+    // work queued on any stream that reads an earlier preparation
+    TSP_CUDA(c, cudaDeviceSynchronize());
+    c->cursor = c->bin_count + nbins;
+    TSP_CUDA(c, cudaMemsetAsync(c->bin_count, 0, 2 * sizeof(int) * nbins, st));
     TSP_CUDA(c, cudaMemsetAsync(c->counters, 0, sizeof(unsigned long long) * 4, st));
     return TSP_OK;
 }
@@ -617,7 +624,7 @@ void tsp_destroy(tsp_ctx* c)
     dfree(c->rows_u); dfree(c->rows); dfree(c->key);
     dfree(c->recbuf);
     dfree(c->scratch);
-    dfree(c->items); dfree(c->bin_count); dfree(c->offsets); dfree(c->cursor);
+    dfree(c->items); dfree(c->bin_count); dfree(c->offsets);
     delete c;
 }
 

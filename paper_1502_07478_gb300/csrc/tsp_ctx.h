@@ -78,7 +78,9 @@ struct tsp_ctx {
     unsigned long long* counters = nullptr;
     int* bin_count = nullptr;
     long long* offsets = nullptr;
-    int* cursor = nullptr;
+    int* cursor = nullptr;            // second half of bin_count
+    int bins_cap = 0;
+    unsigned long long prepared = 0;  // lane capacities whose kernels have their limits raised
     int* flag = nullptr;
     bool uploaded = false, sens_ready = false;
     bool appending = false;           // between tsp_begin_events and tsp_end_events

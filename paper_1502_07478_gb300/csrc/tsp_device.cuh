@@ -186,10 +186,10 @@ constexpr int kAccWords = 18432;
 // Shared-memory layout of the tile kernel, in 32-bit words: kPadFloats slack,
 // the rho' region (RH*RS), 2*kPadFloats slack, the accumulator's H region
 // (RH*RS; the float accumulator of the other passes), its L region at
-// kAccWords words from the H region, kPadFloats slack, and kPartFloats for the
-// groups' reduction slots (first in the passes over window records, which read
-// them as float4; last in the others, which use half of them: warps/G groups x
-// 2 parities x 3G floats).
+// kAccWords words from the H region, kPadFloats slack, then the groups'
+// reduction slots (warps/G groups x 2 parities x 3G floats <= 6*kMaxWarps).  The
+// passes over window records need less (rec_smem_floats): their reduction slots
+// (kPartFloats, read as float4) come first, their accumulator has one word.
 constexpr int kPartFloats = 12 * kMaxWarps;
 // Shared staging of a warp's next window records (256 bytes) and of its event's
 // coefficients (64), in floats (tsp_rec.cuh).
@@ -199,7 +199,7 @@ __host__ __device__ constexpr int rec_slot_floats(bool two) { return two ? 160 :
 __host__ __device__ constexpr size_t tiles_smem_floats(int RH, int RS)
 {
     return (size_t)kPadFloats + (size_t)RH * RS + 2 * kPadFloats + (size_t)kAccWords +
-           (size_t)RH * RS + kPadFloats + kPartFloats + kMaxWarps * kRecSlotFloats;
+           (size_t)RH * RS + kPadFloats + 6 * kMaxWarps;
 }
 
 // Shared memory of the passes over window records, in 32-bit words: the groups'

@@ -17,8 +17,9 @@
 // per pass at 32 G lanes x 8 bytes an event (1 KB at 1 mm, 512 B at 2 mm, 256 B
 // at 4 mm), 10 GB a pass for 1e7 events at 1 mm, copied to shared memory an
 // event ahead.  MLEM passes: 1e7 events at 1 mm 42.9 -> 34.4 ms, 1e7 at 4 mm
-// 6.22 -> 3.53 ms, 1e6 at 2 mm 2.28 -> 1.66 ms.  Writing them costs an upload
-// about as much as one pass's row setup did (1.3 ms per 1e6 events at 1 mm).
+// 6.22 -> 3.53 ms, 1e6 at 2 mm 2.28 -> 1.66 ms (before the steps below).  Writing
+// them costs an upload 1.1 ms per 1e6 events at 1 mm (1.5 with the coefficients
+// worked out by one lane a warp), 0.65 at 2 mm.
 #pragma once
 
 #include "tsp_mlem.cuh"
@@ -87,56 +88,75 @@ __device__ __forceinline__ int lane_row(int rowi)
     return (rowi & 1) ? (rowi >> 1) + 1 : -(rowi >> 1);
 }
 
-// Records of the events of the plain items.  One warp per (event, 32-lane
-// block); item blocks of one warp count each so that short lists still spread.
+// Records of the events of the plain items: a block takes an item, or (grid.y > 1,
+// short lists) every grid.y-th run of 8 of its events.  A thread an event for the
+// coefficients, then a warp per (event, 32-lane block).  (The coefficients by one
+// lane of the warp that has an event's first block were 5 to 20% of the kernel's
+// instructions, and so was the division of the task index by G.)
 template <int LMAX, int NSEG>
 __global__ void __launch_bounds__(256)
 k_records(Inst p, const int4* __restrict__ items, int n_items, uint2* __restrict__ recs,
           float4* __restrict__ evc)
 {
+    constexpr int kRun = 8;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const Geo& g = p.g;
     const int G = p.G;
     for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
         const int4 item = items[it];
         const Frame f = tile_frame(g, p.tl, item.x);
-        const int tasks = item.z * G;
-        for (int k = warp + 8 * blockIdx.y; k < tasks; k += 8 * gridDim.y) {
-            const int j = k / G, blk = k - j * G, e = item.y + j;
+        for (int k = threadIdx.x; k < item.z; k += 256) {
+            if ((k / kRun) % gridDim.y != blockIdx.y) continue;
+            const int e = item.y + k;
             const float4 ev = p.evs.geo[e];
-            int2 rws = p.evs.rows[e];
-            const int evflags = rws.y & ~kEvRowsMask;
-            rws.y &= kEvRowsMask;
-            const EvSig es = ev_sig(g, ev);
-            const int mid = (rws.y - 1) >> 1;
-            const int rowi = (NSEG == 1 ? blk : blk >> 1) * 32 + lane;
-            const int ri = mid + lane_row(rowi);
-            const bool valid = ri >= 0 && ri < rws.y;
-            unsigned long long* qc = &p.accum->rec_qclip;
-            unsigned long long* lc = &p.accum->rec_lclip;
-            RowSpan sp;
-            if constexpr (NSEG == 1)
-                sp = row_span<kAlt, LMAX, true>(g, es, ev, p.evs.geo64 + e, rws.x + ri, valid,
-                                                evflags, f, qc, lc);
-            else if ((blk & 1) == 0)
-                sp = row_span<kPos, LMAX, true>(g, es, ev, p.evs.geo64 + e, rws.x + ri, valid,
-                                                evflags, f, qc, lc);
-            else
-                sp = row_span<kNeg, LMAX, true>(g, es, ev, p.evs.geo64 + e, rws.x + ri, valid,
-                                                evflags, f, qc, lc);
-            int la, lb;
-            if constexpr (NSEG == 1) {
-                la = sp.lim_odd >> 1;
-                lb = (sp.lim_even + 1) >> 1;
-            } else {
-                la = (sp.lim_odd + 1) >> 1;
-                lb = sp.lim_odd >> 1;
+            const int2 rws = p.evs.rows[e];
+            make_evc(g, ev_sig(g, ev), ev, rws.x + (((rws.y & kEvRowsMask) - 1) >> 1),
+                     evc + (size_t)e * kEvcFloat4);
+        }
+        for (int j0 = blockIdx.y * kRun; j0 < item.z; j0 += kRun * gridDim.y) {
+            const int jn = min(kRun, item.z - j0);
+            int j = 0, blk = warp;
+            for (;; blk += 8) {
+                while (blk >= G) {
+                    blk -= G;
+                    ++j;
+                }
+                if (j >= jn) break;
+                const int e = item.y + j0 + j;
+                const float4 ev = p.evs.geo[e];
+                int2 rws = p.evs.rows[e];
+                const int evflags = rws.y & ~kEvRowsMask;
+                rws.y &= kEvRowsMask;
+                const EvSig es = ev_sig(g, ev);
+                const int mid = (rws.y - 1) >> 1;
+                const int rowi = (NSEG == 1 ? blk : blk >> 1) * 32 + lane;
+                const int ri = mid + lane_row(rowi);
+                const bool valid = ri >= 0 && ri < rws.y;
+                unsigned long long* qc = &p.accum->rec_qclip;
+                unsigned long long* lc = &p.accum->rec_lclip;
+                RowSpan sp;
+                if constexpr (NSEG == 1)
+                    sp = row_span<kAlt, LMAX, true>(g, es, ev, p.evs.geo64 + e, rws.x + ri, valid,
+                                                    evflags, f, qc, lc);
+                else if ((blk & 1) == 0)
+                    sp = row_span<kPos, LMAX, true>(g, es, ev, p.evs.geo64 + e, rws.x + ri, valid,
+                                                    evflags, f, qc, lc);
+                else
+                    sp = row_span<kNeg, LMAX, true>(g, es, ev, p.evs.geo64 + e, rws.x + ri, valid,
+                                                    evflags, f, qc, lc);
+                int la, lb;
+                if constexpr (NSEG == 1) {
+                    la = sp.lim_odd >> 1;
+                    lb = (sp.lim_even + 1) >> 1;
+                } else {
+                    la = (sp.lim_odd + 1) >> 1;
+                    lb = sp.lim_odd >> 1;
+                }
+                const float u0 = sp.has ? fmaf((float)sp.o, g.dz, g.z0) - sp.c.zc : 0.0f;
+                recs[((size_t)e * G + blk) * 32 + lane] =
+                    make_uint2(__float_as_uint(u0), (unsigned)sp.sidx | (unsigned)la << 16 |
+                                                        (unsigned)lb << 24);
             }
-            const float u0 = sp.has ? fmaf((float)sp.o, g.dz, g.z0) - sp.c.zc : 0.0f;
-            recs[((size_t)e * G + blk) * 32 + lane] =
-                make_uint2(__float_as_uint(u0), (unsigned)sp.sidx | (unsigned)la << 16 |
-                                                    (unsigned)lb << 24);
-            if (blk == 0 && lane == 0) make_evc(g, es, ev, rws.x + mid, evc + (size_t)e * kEvcFloat4);
         }
     }
 }
