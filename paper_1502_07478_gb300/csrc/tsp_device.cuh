@@ -189,8 +189,9 @@ constexpr int kAccWords = 18432;
 // kAccWords words from the H region, kPadFloats slack, then the groups'
 // reduction slots (warps/G groups x 2 parities x 3G floats <= 6*kMaxWarps).  The
 // passes over window records need less (rec_smem_floats): their reduction slots
-// (kPartFloats, read as float4) come first, their accumulator has one word.
-constexpr int kPartFloats = 12 * kMaxWarps;
+// (kPartFloats: 2 parities x kMinWarps for each of at most 15 groups) come first,
+// their accumulator has one word.
+constexpr int kPartFloats = 2 * kMinWarps * 15;
 // Shared staging of a warp's next window records (256 bytes) and of its event's
 // coefficients (64), in floats (tsp_rec.cuh).
 constexpr int kRecSlotFloats = 80;

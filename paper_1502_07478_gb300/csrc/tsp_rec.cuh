@@ -231,13 +231,14 @@ __device__ __forceinline__ PairC rec_row(const Geo& g, const RecIn& x, float row
     const float gam = x.b.y * y, al = x.b.z * y, be = Dy * fmaf(x.b.w, y, x.c.x);
     const float Q0 = fmaf(gam, u0, Qc), dQ = gam * g.dz;
     // (the event's coefficients give aCb; the exponent has it times kA)
-    float A0 = fmaf(al, u0, be), dA = al * g.dz;
+    float A0 = fmaf(al, u0, be);
     if (GRAD) {
+        const float dB = al * g.dz;
         gc->B0 = make_float2(A0, A0);
-        gc->dB = make_float2(dA, dA);
+        gc->dB = make_float2(dB, dB);
     }
     A0 *= g.kA;
-    dA *= g.kA;
+    const float dA = al * (g.kA * g.dz);
     const float C0 = fmaf(-x.c.y * Dy, Dy, x.c.z);
     const float su0 = x.c.w * u0, dsu = x.c.w * g.dz;
     const float e0 = GRAD ? C0 : fmaf(-su0, su0, C0), e1 = GRAD ? su0 : -2.0f * su0 * dsu,
@@ -384,17 +385,27 @@ __device__ __forceinline__ void rec_pass2(unsigned base, int n, unsigned tma, fl
     }
 }
 
-// Sum over the group's G warps of each warp's value (lane 0's), the same in
-// every lane: slots of a power of two >= G floats (the unused ones stay zero),
-// summed by a butterfly.
-__device__ __forceinline__ float group_sum(float v, int G, int Gp, int wig, int lane, int bar_id,
-                                           float* slot)
+// Sum over the group's warps of each warp's value (lane 0's), the same in every
+// lane: kMinWarps slots of which those beyond the group's warps stay zero, summed by
+// a butterfly without a loop's control.
+__device__ __forceinline__ float group_sum(float v, int G, int wig, int lane, int bar_id, float* slot)
 {
+    static_assert(kMinWarps == 16, "four steps");
     if (lane == 0) slot[wig] = v;
     named_barrier(bar_id, G * 32);
-    v = slot[lane & (Gp - 1)];
-    for (int o = Gp >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    v = slot[lane & (kMinWarps - 1)];
+#pragma unroll
+    for (int o = kMinWarps / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
+}
+
+// 1/D to float precision (one Newton step); not finite or 0 where D is far out of
+// range, which the callers' test of the largest term excludes.
+__device__ __forceinline__ float recip(float D)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(D));
+    return fmaf(r, fmaf(-D, r, 1.0f), r);
 }
 
 // Gradient pass, one pair: the kernel value's pair (0 beyond the streams' last
@@ -418,15 +429,15 @@ __device__ __forceinline__ float2 p1g_pair(Addr a0, Addr a1, int k, int la, int 
                                            const PairC& c, const GradC& g, float2& kk,
                                            GradSums& m)
 {
-    float2 q = __ffma2_rn(kk, c.dQ, c.Q0);
-    if constexpr (PRED) {
-        // keeps X and S finite where P is set to 0 below
-        q.x = k <= la ? q.x : 1.0f;
-        q.y = k <= lb ? q.y : 1.0f;
-    }
+    const float2 q = __ffma2_rn(kk, c.dQ, c.Q0);
     float2 rq;
     rq.x = rsqrt_approx(q.x);
     rq.y = rsqrt_approx(q.y);
+    if constexpr (PRED) {
+        // (with 1/sqrt(Q) set to 0 P is 0 and everything else finite)
+        rq.x = k <= la ? rq.x : 0.0f;
+        rq.y = k <= lb ? rq.y : 0.0f;
+    }
     const float2 a = __ffma2_rn(kk, c.dA, c.A0);
     const float2 su = __ffma2_rn(kk, c.e2, c.e1);
     const float2 e = __ffma2_rn(su, __fmul2_rn(su, make_float2(-1.0f, -1.0f)), c.e0);
@@ -435,11 +446,7 @@ __device__ __forceinline__ float2 p1g_pair(Addr a0, Addr a1, int k, int la, int 
     float2 x;
     x.x = ex2_approx(ar.x);
     x.y = ex2_approx(ar.y);
-    float2 p = __fmul2_rn(rq, x);
-    if constexpr (PRED) {
-        p.x = k <= la ? p.x : 0.0f;
-        p.y = k <= lb ? p.y : 0.0f;
-    }
+    const float2 p = __fmul2_rn(rq, x);
     float2 v;
     v.x = ld_rhop<!GLD, false, GLD && PRED, OFF0>(a0, k, la);
     v.y = ld_rhop<!GLD, false, GLD && PRED, OFF1>(a1, k, lb);
@@ -570,7 +577,6 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
         blk -= blk >= nb ? nb : 0;
     }
     const float rowoff = (float)lane_row(blk * 32 + lane);
-    const int Gp = G > 1 ? 1 << (32 - __clz(G - 1)) : 1;
     const int rslot = NSEG == 1 ? blk * 32 + lane : (blk * 2 + (wig & 1)) * 32 + lane;
     const uint2* rp = I.evs.recs + (size_t)(first + grp) * (32 * G) + rslot;
     const float4* ep = I.evs.evc + (size_t)(first + grp) * kEvcFloat4;
@@ -618,8 +624,6 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
             n = rec_pass1_grad<TRAV, GLD>(rbase, la, lb, c, gc, kfast, kmax, m, tma);
             E = rec_grad_row(g, ev, y, Dy, u0, m);
             D = warp_sum(m.m0.x + m.m0.y);
-            E.x = warp_sum(E.x);
-            E.y = warp_sum(E.y);
         } else {
             float2 D2 = make_float2(0.0f, 0.0f);
             n = rec_pass1<TRAV, LMAX, MODE != kLoglik, GLD>(rbase, la, lb, c, kfast, kmax, D2, tma);
@@ -627,35 +631,24 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
         }
         if (MODE != kLoglik) tm_wait_st();
         if (G > 1) {
-            if constexpr (GRAD) {
-                float4* sl = reinterpret_cast<float4*>(part) + (parity ? G : 0);
-                if (lane == 0) sl[wig] = make_float4(D, E.x, E.y, 0.0f);
-                named_barrier(1 + grp, G * 32);
-                D = E.x = E.y = 0.0f;
-                for (int w = 0; w < G; ++w) {
-                    const float4 v = sl[w];
-                    D += v.x;
-                    E.x += v.y;
-                    E.y += v.z;
-                }
-            } else {
-                D = group_sum(D, G, Gp, wig, lane, 1 + grp, part + parity * Gp);
-            }
-            parity ^= 1;
+            D = group_sum(D, G, wig, lane, 1 + grp, part + parity);
+            parity ^= kMinWarps;
         }
         if (D > 0.0f) {
             ++used;
-            if (MODE != kMlem && wig == 0 && lane == 0) {
-                logD += (double)logf(D) + (double)g.pshift * 0.69314718055994530942;
-                if (GRAD) {
-                    giz += (double)(E.x / D);
-                    gil += (double)(E.y / D);
-                }
-            }
+            if (MODE != kMlem && wig == 0 && lane == 0) logD += (double)logf(D);
             if (MODE != kLoglik) {
-                const float invD = 1.0f / D;
-                const float s = invD * inv_q, top = s * ev.x;
-                if (top <= kTopTerm && spent + top + 1.0f <= room) {
+                const float r = recip(D), s = r * inv_q, top = s * ev.x;
+                // (false for a NaN, and for a D that recip has no value of)
+                const bool fit = top > 0.0f && top <= kTopTerm && spent + top + 1.0f <= room;
+                if (GRAD) {
+                    // per-lane sums: the rows' terms of an event cancel to a small
+                    // part of themselves, so they are added in double precision
+                    const float w = fit ? r : 1.0f / D;
+                    giz += (double)(E.x * w);
+                    gil += (double)(E.y * w);
+                }
+                if (fit) {
                     spent += top + 1.0f;
                     const float q = s * 0x1p-149f;
                     rec_pass2<TRAV>(base + acc_off, n, tma, make_float2(q, q));
@@ -664,7 +657,7 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
                     const int iy = f.oy + rr;
                     const int iz = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0))) + col;
                     rec_scatter_global<TRAV, MODE == kMlem && !GLD>(I.A, I.rhop, iy * g.nz + iz, la,
-                                                                    lb, n, tma, invD);
+                                                                    lb, n, tma, 1.0f / D);
                 }
             }
         }
@@ -672,8 +665,14 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
     }
     if (wig == 0 && lane == 0) {
         if (used) atomicAdd(&bs->used, (unsigned long long)used);
-        if (MODE != kMlem) atomicAdd(&bs->logD, logD);
-        if (GRAD) {
+        if (MODE != kMlem) atomicAdd(&bs->logD, logD + used * (g.pshift * 0.69314718055994530942));
+    }
+    if (GRAD) {
+        for (int o = 16; o > 0; o >>= 1) {
+            giz += __shfl_xor_sync(0xffffffffu, giz, o);
+            gil += __shfl_xor_sync(0xffffffffu, gil, o);
+        }
+        if (lane == 0) {
             atomicAdd(&bs->giz, giz);
             atomicAdd(&bs->gil, gil);
         }
@@ -706,15 +705,6 @@ __device__ __forceinline__ bool two_rows_fit(int G) { return G == 1 || (G & 1) =
 __host__ __device__ constexpr bool two_rows(int lmax, int mode, int nseg, bool gld)
 {
     return lmax <= 32 && mode != kGrad && nseg == 1 && !gld;
-}
-
-// 1/D to float precision (one Newton step); not finite or 0 where D is far out of
-// range, which the caller's test of the largest term excludes.
-__device__ __forceinline__ float recip(float D)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(D));
-    return fmaf(r, fmaf(-D, r, 1.0f), r);
 }
 
 // The two rows' constants (.x, .y): see rec_row.
@@ -929,8 +919,7 @@ __device__ __forceinline__ void rec2_events(const Inst& I, const Frame& f, int f
                          : "memory");
     };
     fetch(e);
-    const int Gp = G2 > 1 ? 1 << (32 - __clz(G2 - 1)) : 1;
-    float* const part = s_part + wgrp * (kPartFloats / kMaxWarps) * G2;
+    float* const part = s_part + wgrp * 2 * kMinWarps;
     int parity = 0;
     unsigned used = 0;
     float spent = 0.0f;
@@ -965,14 +954,14 @@ __device__ __forceinline__ void rec2_events(const Inst& I, const Frame& f, int f
         if (!halves) D += __shfl_xor_sync(0xffffffffu, D, 16);
         if (MODE != kLoglik) tm_wait_st();
         if (G2 > 1) {
-            D = group_sum(D, G2, Gp, wig, lane, 1 + wgrp, part + parity * Gp);
-            parity ^= 1;
+            D = group_sum(D, G2, wig, lane, 1 + wgrp, part + parity);
+            parity ^= kMinWarps;
         }
         const bool on = D > 0.0f;
         if (on) {
             ++used;
             if (MODE != kMlem && (halves ? (lane & 15) == 0 : wig == 0 && lane == 0))
-                logD += (double)logf(D) + (double)g.pshift * 0.69314718055994530942;
+                logD += (double)logf(D);
         }
         if (MODE != kLoglik) {
             const float r = recip(D), s = r * inv_q, top = s * pmax;
@@ -993,9 +982,10 @@ __device__ __forceinline__ void rec2_events(const Inst& I, const Frame& f, int f
         }
         if (left == 0) break;
     }
-    if (used && (halves ? (lane & 15) == 0 : wig == 0 && lane == 0))
+    if (used && (halves ? (lane & 15) == 0 : wig == 0 && lane == 0)) {
         atomicAdd(&bs->used, (unsigned long long)used);
-    if (MODE != kMlem && logD != 0.0) atomicAdd(&bs->logD, logD);
+        if (MODE != kMlem) atomicAdd(&bs->logD, logD + used * (g.pshift * 0.69314718055994530942));
+    }
 }
 
 // Persistent tile kernel over window records.  Work
@@ -1177,7 +1167,7 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
             const int G = I.G;
             const int ngroups = group_count(kWarps, G);
             const int grp = warp / G, wig = warp - grp * G;
-            float* part = s_part + grp * (kPartFloats / kWarps) * G;
+            float* part = s_part + grp * 2 * kMinWarps;
 #define TSP_REC_EVENTS(TRAV) \
     rec_events<TRAV, LMAX, MODE, NSEG, GLD>(I, f, item.y, item.z, grp, ngroups, wig, lane, rp_addr, \
                                             acc_off, slot, part, &s_sums, tma, inv_q, scr)
