@@ -72,6 +72,19 @@ size_t dyn_smem_limit(int dev)
     return (size_t)optin - 2048;    // room for the kernels' static shared memory
 }
 
+// Sparse lists, with fewer than kRecCoverage events over a pixel, keep the general
+// passes: one word of fixed point has no room for both the headroom and the precision
+// that a sum of few terms needs (see fx_bits), and their two-word accumulator has.
+constexpr double kRecCoverage = 64.0;
+
+// Whether the declared list will have window records, by a margin: the mean window is
+// 0.9 of the cut ellipse's area (the mean cosine of the accepted angles).
+static bool dense_list(const tsp_ctx* c, double umax, double hy, double dy, double dz)
+{
+    const double pixels = 0.9 * 3.14159265358979 * umax * hy / (dy * dz);
+    return c->n_total * pixels >= 2.0 * kRecCoverage * c->p.ny * c->p.nz;
+}
+
 // Derive the kernel constants, lane capacity, group size and tiling from the
 // parameters.  Returns TSP_OK or TSP_EINVAL.
 int plan(tsp_ctx* c)
@@ -118,19 +131,34 @@ int plan(tsp_ctx* c)
     tl.HZ = (int)std::ceil(w + 1.5 + 0.5 * t_max * (dy / dz) + 0.5 * dtb * (dy / dz) * tl.HY) + 1;
     int RS = 33;
     while (RS - 2 * tl.HZ < std::min(16, p.nz)) RS += 32;
-    tl.RS = RS;
-    tl.RW = RS;
-    tl.TZ = RS - 2 * tl.HZ;
     const size_t budget = 224 * 1024;
-    auto fits = [&](int ty) {
-        return tiles_region_fits(ty + 2 * tl.HY, RS) &&
-               tiles_smem_floats(ty + 2 * tl.HY, RS) * sizeof(float) <= budget;
+    auto fits = [&](int ty, int rs) {
+        if (c->wide) return rec_smem_floats(ty + 2 * tl.HY, rs, false) * sizeof(float) <= budget;
+        return tiles_region_fits(ty + 2 * tl.HY, rs) &&
+               tiles_smem_floats(ty + 2 * tl.HY, rs) * sizeof(float) <= budget;
     };
     int TY = std::max(4, std::min(128, c->sched.ty_cap) / 4 * 4);
     const int ty0 = TY;
-    while (TY > 4 && !fits(TY)) TY -= 4;
+    // Wide tiles: the one-word accumulator leaves room for regions 1.4 times those
+    // of the general passes.  An item costs some 10 us beside its events (staging,
+    // flush, the groups' unequal ends), as much as 20 events at 1 mm, so a list
+    // is cut into as few tiles as the shared memory allows until a tile has some 64
+    // events: MEASURED_WIDE.
+    c->wide = !c->no_wide && dense_list(c, umax, hy, dy, dz);
+    while (TY > 4 && !fits(TY, RS)) TY -= 4;
     c->gld = 0;
-    if (!fits(TY)) {
+    if (!fits(TY, RS) || RS - 1 - 2 * tl.HZ < 1) c->wide = false;
+    if (c->wide)
+        for (;; RS += 32) {
+            const double tiles = (double)tl.nb * ((p.ny + TY - 1) / TY) *
+                                 ((p.nz + 2 * tl.zs_off) / (RS - 1 - 2 * tl.HZ) + 1);
+            if (!fits(TY, RS + 32) || RS - 2 * tl.HZ >= p.nz || c->n_total >= 64.0 * tiles) break;
+        }
+    tl.RS = RS;
+    // (of the odd row stride, a multiple of 32 columns: whole warps stage and flush)
+    tl.RW = c->wide ? RS - 1 : RS;
+    tl.TZ = tl.RW - 2 * tl.HZ;
+    if (!fits(TY, RS)) {
         // windows too large to stage rho' and the accumulator (very fine
         // grids): stage only the accumulator and read rho' from global memory,
         // with two lanes per row; if even that does not fit, no angle bins, so
@@ -162,7 +190,9 @@ int plan(tsp_ctx* c)
     tl.tiles_y = (p.ny + tl.TY - 1) / tl.TY;
     tl.tiles_z = (p.nz + 2 * tl.zs_off + tl.TZ - 1) / tl.TZ;
     c->smem = tl.nb == 0 ? 0
-              : (c->gld ? tiles_acc_smem_floats(tl.RH, tl.RS) : tiles_smem_floats(tl.RH, tl.RS)) *
+              : (c->gld    ? tiles_acc_smem_floats(tl.RH, tl.RS)
+                 : c->wide ? rec_smem_floats(tl.RH, tl.RS, false)
+                           : tiles_smem_floats(tl.RH, tl.RS)) *
                     sizeof(float);
     c->nbins = tl.nb * tl.tiles_y * tl.tiles_z + 1;
     // The dynamic shared-memory limit is a property of the kernel function,
@@ -238,14 +268,14 @@ float fx_peak(const tsp_ctx* c)
 // An ordinary event's largest term takes fx_bits bits.  Its mean term is then some
 // 2^(fx_bits - 2.2) quanta, each rounded to the nearest one, and over the cov events
 // of a pixel the rounding of A is 0.3 x 2^(2.2 - fx_bits) / sqrt(cov) of it: with
-//   fx_bits = 22.9 - log2(cov / 64) / 2
-// some 2e-8 for every list (less than 1e-7 at 64 events a pixel, where 21 bits are
+//   fx_bits = 24.4 - log2(cov / 64) / 2
+// some 1e-8 for every list (4e-8 at 64 events a pixel, where 22 bits are
 // the most), which the float sums of the denominators (some 3e-7) hide.  The rest up
 // to 2^24 is the headroom of single events.
 int fx_bits(const tsp_ctx* c)
 {
     const double cov = std::max(coverage(c), 1.0);
-    return std::max(12, std::min(21, (int)std::lround(22.9 - 0.5 * std::log2(cov / 64.0))));
+    return std::max(12, std::min(22, (int)std::lround(24.4 - 0.5 * std::log2(cov / 64.0))));
 }
 
 PassArgs pass_args(tsp_ctx* c)
@@ -314,12 +344,7 @@ int prep_chunk(tsp_ctx* c, long long first, long long n, cudaStream_t st)
 // Window records of the placed events.  They are kept when they take at most a
 // quarter of the memory that is free when their buffer has to grow (6e7 events
 // at 1 mm on an empty 280 GB); otherwise, or when the allocation fails, the
-// passes set the rows up themselves.  So do those of sparse lists, with fewer than
-// kRecCoverage events over a pixel: one word of fixed point has no room for both
-// the headroom and the precision that a sum of few terms needs (see fx_bits), and
-// the two-word accumulator of the general passes has.
-constexpr double kRecCoverage = 64.0;
-
+// passes set the rows up themselves.  So do those of sparse lists (kRecCoverage).
 int build_records(tsp_ctx* c, cudaStream_t st)
 {
     c->rec = false;
@@ -422,6 +447,12 @@ int prep_finish(tsp_ctx* c, cudaStream_t st)
     c->launches += n > 0 ? 1 : 0;
     clear_graphs(c);
     if (int rc = build_records(c, st)) return rc;
+    if (c->wide && !c->rec && c->n_items > 0) {
+        // the general passes need their own tiles
+        c->no_wide = true;
+        if (int rc = plan(c)) return rc;
+        return prepare_events(c, st);
+    }
     c->uploaded = true;
     return TSP_OK;
 }
@@ -645,9 +676,11 @@ int tsp_begin_events(tsp_ctx* c, int64_t n_total, void* stream)
     TSP_CUDA(c, cudaEventRecord(c->copy_ev, st));
     TSP_CUDA(c, cudaStreamWaitEvent(c->copy_stream, c->copy_ev, 0));
     if ((rc = ensure_event_capacity(c, std::max<long long>(n_total, 1)))) return rc;
-    if ((rc = prep_begin(c, st))) return rc;
     c->n = 0;
     c->n_total = n_total;
+    c->no_wide = false;
+    if ((rc = plan(c))) return rc;
+    if ((rc = prep_begin(c, st))) return rc;
     c->appending = true;
     return TSP_OK;
 }

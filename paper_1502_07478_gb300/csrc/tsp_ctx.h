@@ -67,6 +67,9 @@ struct tsp_ctx {
     float4* evc = nullptr;
     bool rec = false;
     bool batch_member = false;        // the batch launches the passes
+    // tiles that only the passes over window records have room for (plan); not
+    // after they were planned for the list at hand and its records could not be had
+    bool wide = false, no_wide = false;
     float* scratch = nullptr;         // transposed rho' regions of the blocks (gld)
     size_t scratch_cap = 0;           // in floats
     int4* items = nullptr;

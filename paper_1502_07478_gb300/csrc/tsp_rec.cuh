@@ -1085,6 +1085,11 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
                 s_acc[-kPadFloats + k] = 0.0f;
                 s_acc[region + k] = 0.0f;
             }
+            for (int rr = tid; rr < tl.RH; rr += kThreads)
+                for (int cc = tl.RW; cc < tl.RS; ++cc) {
+                    if (!GLD) s_rp[rr * tl.RS + cc] = 0.0f;
+                    s_cnt[rr * tl.RS + cc] = 0u;
+                }
             fresh = false;
             // the groups' slots change their layout with G
             if (BATCH)
@@ -1109,7 +1114,7 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
                     const int iz = z0row + cc;
                     float v = 0.0f;
                     if (row_in && iz >= 0 && iz < g.nz) {
-                        v = I.rhop[(size_t)iy * g.nz + iz];
+                        v = __ldg(I.rhop + (size_t)iy * g.nz + iz);
                         ++inside;
                     }
                     scr[cc * kScrRows + rr] = v;
@@ -1121,11 +1126,13 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
                 const int iy = f.oy + rr;
                 const bool row_in = iy >= 0 && iy < g.ny;
                 const int z0row = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0)));
-                for (int cc = lane; cc < tl.RS; cc += 32) {
+#pragma unroll 4
+                for (int cc = lane; cc < tl.RW; cc += 32) {
                     const int iz = z0row + cc;
                     float v = 0.0f;
-                    if (row_in && cc < tl.RW && iz >= 0 && iz < g.nz) {
-                        v = I.rhop[(size_t)iy * g.nz + iz];
+                    // (the read-only path: loads may pass the stores of earlier columns)
+                    if (row_in && iz >= 0 && iz < g.nz) {
+                        v = __ldg(I.rhop + (size_t)iy * g.nz + iz);
                         ++inside;
                     }
                     s_rp[rr * tl.RS + cc] = v;

@@ -76,3 +76,22 @@ def test_dense_list_high_contrast(ny, nz, scale, lengths):
     rho[60 * f:70 * f, 40 * f:60 * f] = 1e3
     rho[75 * f:90 * f, 30 * f:50 * f] = 0.0
     _check(w, w.events(), (scale * rho).astype(np.float32), {}, lengths)
+
+
+@pytest.mark.parametrize("ny,nz", [(140, 100), (699, 503)])
+def test_dense_list_without_records(ny, nz, monkeypatch):
+    """A dense list whose records cannot be held is tiled again for the general
+    passes, and a later upload for the records."""
+    from paper_1502_07478_gb300 import Recon
+    w = replace(make_workload("small_5mm"), ny=ny, nz=nz, n_events=8000)
+    ev = w.events()
+    ref, _ = oracle.mlem(Setup.from_workload(w), ev, 1)
+    m = ref > 0.01 * ref.max()
+    r = Recon.from_workload(w)
+    for fault in ("records", ""):
+        monkeypatch.setenv("TSP_SIM_FAULT", fault)
+        r.upload_events(*ev)
+        r.iterate(1)
+        img = r.read_image().cpu().numpy().astype(np.float64)
+        assert np.max(np.abs(img[m] - ref[m]) / ref[m]) <= 1e-4
+    r.close()
