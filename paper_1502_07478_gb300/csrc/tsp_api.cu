@@ -143,7 +143,8 @@ int plan(tsp_ctx* c)
     // of the general passes.  An item costs some 10 us beside its events (staging,
     // flush, the groups' unequal ends), as much as 20 events at 1 mm, so a list
     // is cut into as few tiles as the shared memory allows until a tile has some 64
-    // events: MEASURED_WIDE.
+    // events: five updates of 2e5 events at 1 mm 4.18 -> 4.04 ms, one of 1e6 3.50 ->
+    // 3.35 ms, five of 2e4 at 5 mm 275 -> 262 us.
     c->wide = !c->no_wide && dense_list(c, umax, hy, dy, dz);
     while (TY > 4 && !fits(TY, RS)) TY -= 4;
     c->gld = 0;

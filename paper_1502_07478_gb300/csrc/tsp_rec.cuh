@@ -238,7 +238,8 @@ __device__ __forceinline__ PairC rec_row(const Geo& g, const RecIn& x, float row
         gc->dB = make_float2(dB, dB);
     }
     A0 *= g.kA;
-    const float dA = al * (g.kA * g.dz);
+    // (not al (kA dz): see rec_grad_row)
+    const float dA = al * g.kA * g.dz;
     const float C0 = fmaf(-x.c.y * Dy, Dy, x.c.z);
     const float su0 = x.c.w * u0, dsu = x.c.w * g.dz;
     const float e0 = GRAD ? C0 : fmaf(-su0, su0, C0), e1 = GRAD ? su0 : -2.0f * su0 * dsu,
@@ -514,8 +515,9 @@ __device__ __forceinline__ float2 rec_grad_row(const Geo& g, const float4& ev, f
     const float s0 = m.s0.x + m.s0.y, s1 = m.s1.x + m.s1.y;
     const float qzs = -2.0f * y * t * c2i, qz0 = fmaf(qzs, u0, (g.R * g.R + y2) * c2i * c2i);
     const float czs = -2.0f * y * c2i;
-    // sum v u^2 = u0^2 m0 + 2 u0 dz m1 + dz^2 m2
-    const float vu2 = fmaf(u0, fmaf(u0, m0, 2.0f * dz * m1), dz * dz * m2);
+    // sum v u^2 = u0^2 m0 + 2 u0 dz m1 + dz^2 m2 (dz dz, rounded the same for every
+    // event, would move the sum of these nearly cancelling terms by up to 1e-6)
+    const float vu2 = fmaf(u0, fmaf(u0, m0, 2.0f * dz * m1), dz * (dz * m2));
     const float Ez = fmaf(es.ldz, m0, -vu2) + czs * fmaf(u0, x0, dz * x1) - fmaf(qz0, s0, qzs * dz * s1);
     const float Bl = 4.0f * Dy * Dy * c2i;
     const float cl = 4.0f * y * t * Dy * c2i;
