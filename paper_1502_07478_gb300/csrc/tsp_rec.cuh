@@ -530,6 +530,40 @@ __device__ __forceinline__ float2 rec_grad_row(const Geo& g, const float4& ev, f
 constexpr float kTopTerm = 0.99f * 0x1p24f;   // one event's largest term
 constexpr float kRoom = 0.99f * 0x1p32f;      // all the events of an item
 
+// How a pass over an item's events scatters: in one word a term (kWhole), or, for an
+// item whose rho' has a peak that events share (see k_tiles_rec), in two passes, the
+// terms' whole quanta (kHigh) and what these leave of them in units 2^-k (kLow; lo =
+// 2^(k - 149)).
+enum Phase : int { kWhole = 0, kHigh = 1, kLow = 2 };
+constexpr float kTopSplit = 0x1p22f;          // one event's largest term, in two passes
+
+__device__ __forceinline__ void add_split(unsigned a, float p, float s, int phase, float lo)
+{
+    const float t = __fmaf_rz(p, s, kFxMagic);          // bits: magic + floor(p s)
+    unsigned v = __float_as_uint(t) - kFxMagicBits;
+    if (phase == kLow) v = __float_as_uint(__fmaf_rn(p, s, kFxMagic - t) * lo);
+#ifdef TSP_DEBUG_CHECKS
+    if (!tsp_sh_ok(a, 4, 2)) return;
+#endif
+    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+
+template <int TRAV>
+__device__ __noinline__ void rec_pass2_split(unsigned base, int n, unsigned tma, float s, int phase,
+                                             float lo)
+{
+    for (int k = 1; k <= n; k += 2) {
+        float x0, x1, x2, x3;
+        tm_ld4(tma, x0, x1, x2, x3);
+        tm_wait_ld();
+        add_split(base + (unsigned)(4 * pair_d0<TRAV>(k)), x0, s, phase, lo);
+        add_split(base + (unsigned)(4 * pair_d1<TRAV>(k)), x1, s, phase, lo);
+        add_split(base + (unsigned)(4 * pair_d0<TRAV>(k + 1)), x2, s, phase, lo);
+        add_split(base + (unsigned)(4 * pair_d1<TRAV>(k + 1)), x3, s, phase, lo);
+        tma += 4;
+    }
+}
+
 // The scatter of an event whose terms the item's accumulator has no room for (see
 // k_tiles_rec): float adds to the global A, each pixel under its predicate; with
 // MASK only where rho' > 0 (as the flush does).
@@ -641,9 +675,11 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
             if (MODE != kMlem && wig == 0 && lane == 0) logD += (double)logf(D);
             if (MODE != kLoglik) {
                 const float r = recip(D), s = r * inv_q, top = s * ev.x;
+                const int phase = bs->phase;
                 // (false for a NaN, and for a D that recip has no value of)
-                const bool fit = top > 0.0f && top <= kTopTerm && spent + top + 1.0f <= room;
-                if (GRAD) {
+                const bool fit = top > 0.0f && top <= (phase == kWhole ? kTopTerm : kTopSplit) &&
+                                 spent + top + 1.0f <= room;
+                if (GRAD && phase != kLow) {
                     // per-lane sums: the rows' terms of an event cancel to a small
                     // part of themselves, so they are added in double precision
                     const float w = fit ? r : 1.0f / D;
@@ -653,8 +689,11 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
                 if (fit) {
                     spent += top + 1.0f;
                     const float q = s * 0x1p-149f;
-                    rec_pass2<TRAV>(base + acc_off, n, tma, make_float2(q, q));
-                } else {
+                    if (phase == kWhole)
+                        rec_pass2<TRAV>(base + acc_off, n, tma, make_float2(q, q));
+                    else
+                        rec_pass2_split<TRAV>(base + acc_off, n, tma, s, phase, bs->lo);
+                } else if (phase != kLow) {
                     const int rr = (int)idx / f.stride, col = (int)idx - rr * f.stride;
                     const int iy = f.oy + rr;
                     const int iz = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0))) + col;
@@ -665,6 +704,7 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
         }
         if (left == 0) break;
     }
+    if (bs->phase == kLow) return;      // counted in the first pass
     if (wig == 0 && lane == 0) {
         if (used) atomicAdd(&bs->used, (unsigned long long)used);
         if (MODE != kMlem) atomicAdd(&bs->logD, logD + used * (g.pshift * 0.69314718055994530942));
@@ -853,6 +893,22 @@ __device__ __forceinline__ void rec2_pass2(unsigned a0, unsigned a1, int n, unsi
     }
 }
 
+// In two passes (see Phase).
+static __device__ __noinline__ void rec2_pass2_split(unsigned a0, unsigned a1, int n, unsigned tma, float s,
+                                              int phase, float lo)
+{
+    for (int k = 1; k <= n; ++k) {
+        float x0, x1, x2, x3;
+        tm_ld4(tma, x0, x1, x2, x3);
+        tm_wait_ld();
+        add_split(a0 + 4u * k, x0, s, phase, lo);
+        add_split(a1 + 4u * k, x1, s, phase, lo);
+        add_split(a0 - 4u * (k - 1), x2, s, phase, lo);
+        add_split(a1 - 4u * (k - 1), x3, s, phase, lo);
+        tma += 4;
+    }
+}
+
 // The scatter of rows that the item's accumulator has no room for (see
 // rec_scatter_global); live: the lane's event is one of those.
 template <bool MASK>
@@ -967,12 +1023,20 @@ __device__ __forceinline__ void rec2_events(const Inst& I, const Frame& f, int f
         }
         if (MODE != kLoglik) {
             const float r = recip(D), s = r * inv_q, top = s * pmax;
+            const int phase = bs->phase;
             // (false for a NaN, and for a D that recip has no value of)
-            const bool fit = on && top > 0.0f && top <= kTopTerm && spent + top + 1.0f <= room;
+            const bool fit = on && top > 0.0f && top <= (phase == kWhole ? kTopTerm : kTopSplit) &&
+                             spent + top + 1.0f <= room;
             if (fit) spent += top + 1.0f;
-            if (__any_sync(0xffffffffu, fit))
-                rec2_pass2(a0 + acc_off, a1 + acc_off, kmax, tma, dup(fit ? s * 0x1p-149f : 0.0f));
-            if (__any_sync(0xffffffffu, on && !fit)) {
+            if (__any_sync(0xffffffffu, fit)) {
+                if (phase == kWhole)
+                    rec2_pass2(a0 + acc_off, a1 + acc_off, kmax, tma,
+                               dup(fit ? s * 0x1p-149f : 0.0f));
+                else
+                    rec2_pass2_split(a0 + acc_off, a1 + acc_off, kmax, tma, fit ? s : 0.0f, phase,
+                                     bs->lo);
+            }
+            if (phase != kLow && __any_sync(0xffffffffu, on && !fit)) {
                 auto pix = [&](unsigned i) {
                     const int rr = (int)i / f.stride, iy = f.oy + rr;
                     return iy * g.nz + f.zbase +
@@ -984,6 +1048,7 @@ __device__ __forceinline__ void rec2_events(const Inst& I, const Frame& f, int f
         }
         if (left == 0) break;
     }
+    if (bs->phase == kLow) return;      // counted in the first pass
     if (used && (halves ? (lane & 15) == 0 : wig == 0 && lane == 0)) {
         atomicAdd(&bs->used, (unsigned long long)used);
         if (MODE != kMlem) atomicAdd(&bs->logD, logD + used * (g.pshift * 0.69314718055994530942));
@@ -1007,6 +1072,13 @@ __device__ __forceinline__ void rec2_events(const Inst& I, const Frame& f, int f
 // responsibilities P rho' / D, as in k_tiles, need no such estimate, but twice the
 // adds and five more packed operations a pair: 1e7 events at 1 mm 34.3 -> 30.4 ms,
 // five updates of 2e5 at 1 mm 5.07 -> 4.29 ms, three of 3e5 at 2 mm 1.57 -> 1.36 ms.
+//
+// Where one pixel can take much of an event (rho' at the region's peak above half of
+// what an ordinary window sums to, or above 16 times the mean), the events' terms there
+// are equal multiples 1 / rho' of the quantum, far below the estimate, and their rounding
+// does not average out (a point source from a spike image: 4e-5 of the counts lost).  Such
+// an item takes two passes over its events, floor of the terms first, their remainder in
+// units 2^-19 or less of the quantum second (1e-7); ordinary images have none.
 //
 // GLD: the windows are too large to stage rho' beside the accumulator.  The block
 // writes the item's rho' region to its own part of global memory, transposed
@@ -1033,7 +1105,7 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
     __shared__ BlockSums s_sums;
     __shared__ Inst s_inst;
     __shared__ unsigned s_tmem;
-    __shared__ float2 s_sum[kWarps];
+    __shared__ float4 s_sum[kWarps];
     const Inst& I = BATCH ? s_inst : p;
 
     const int tid = threadIdx.x, lane = tid & 31;
@@ -1098,7 +1170,7 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
                 for (int k = tid; k < kPartFloats; k += kThreads) s_part[k] = 0.0f;
         }
         const Frame f = tile_frame(g, tl, item.x);
-        float sum = 0.0f;      // rho' over the region's pixels, and their number
+        float sum = 0.0f, most = 0.0f;     // rho' over the region's pixels, and their number
         int inside = 0;
         if constexpr (GLD) {
             if (MODE != kLoglik)
@@ -1121,6 +1193,7 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
                     }
                     scr[cc * kScrRows + rr] = v;
                     sum += v;
+                    most = fmaxf(most, v);
                 }
             }
         } else {
@@ -1140,13 +1213,15 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
                     s_rp[rr * tl.RS + cc] = v;
                     if (MODE != kLoglik) s_cnt[rr * tl.RS + cc] = 0u;
                     sum += v;
+                    most = fmaxf(most, v);
                 }
             }
         }
         if (MODE != kLoglik) {
             sum = warp_sum(sum);
             inside = __reduce_add_sync(0xffffffffu, inside);
-            if (lane == 0) s_sum[warp] = make_float2(sum, (float)inside);
+            most = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(most)));
+            if (lane == 0) s_sum[warp] = make_float4(sum, (float)inside, most, 0.0f);
         }
         if (tid == 0) {
             s_item[par] = next;
@@ -1157,18 +1232,28 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
             }
         }
         __syncthreads();
-        float quantum = 0.0f, inv_q = 0.0f;
+        float inv_q = 0.0f;
         if (MODE != kLoglik) {
             static_assert(kWarps == 32, "a lane a warp's sum");
-            const float2 part = s_sum[lane];
+            const float4 part = s_sum[lane];
             const float mean = warp_sum(part.x) / warp_sum(part.y);
-            const int t = min(I.fx_bits, 29 - (32 - __clz(max(item.z - 1, 1))));
+            const float peak = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(part.z)));
+            const bool split = peak > 16.0f * mean || peak * I.fx_peak > 0.5f * mean;
+            // (in two passes the low word has the precision, and 2^22 / 2^14 is the headroom)
+            const int t = min(split ? 14 : I.fx_bits, 29 - (32 - __clz(max(item.z - 1, 1))));
             inv_q = mean / I.fx_peak * (float)(1 << t);
-            quantum = 1.0f / inv_q;
             // (an image of no usable scale: every event takes the float scatter)
-            if (!(inv_q >= 1e-30f && inv_q <= 1e30f)) quantum = 0.0f, inv_q = INFINITY;
+            if (!(inv_q >= 1e-30f && inv_q <= 1e30f)) inv_q = INFINITY;
+            if (tid == 0) {
+                const int k = min(23, 31 - (32 - __clz(max(item.z - 1, 1))));
+                s_sums.phase = split ? kHigh : kWhole;
+                s_sums.quantum = 1.0f / inv_q;
+                s_sums.lo = __uint_as_float(1u << k);            // 2^(k - 149)
+                s_sums.lo_quantum = s_sums.quantum * exp2f((float)-k);
+            }
+            __syncthreads();
         }
-        {
+        for (;;) {
             const unsigned rp_addr = (unsigned)__cvta_generic_to_shared(s_rp);
             const unsigned acc_off = GLD ? 0u : 4u * (unsigned)(region + 2 * kPadFloats);
             const unsigned slot =
@@ -1193,27 +1278,34 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
                     TSP_REC_EVENTS(kNeg);
             }
 #undef TSP_REC_EVENTS
+            __syncthreads();
+            if (MODE == kLoglik) break;
+            {
+                const int phase = s_sums.phase;
+                const float quantum = phase == kLow ? s_sums.lo_quantum : s_sums.quantum;
+                for (int rr = warp; rr < tl.RH; rr += kWarps) {
+                    const int iy = f.oy + rr;
+                    if (iy < 0 || iy >= g.ny) continue;
+                    const int z0row = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0)));
+                    for (int cc = lane; cc < tl.RW; cc += 32) {
+                        const int iz = z0row + cc;
+                        const int k = rr * tl.RS + cc;
+                        float v = (float)s_cnt[k] * quantum;
+                        if (phase == kHigh) s_cnt[k] = 0u;
+                        // (the update is 0 where rho' = 0, whatever A holds)
+                        if (MODE == kMlem && !GLD && !(s_rp[k] > 0.0f)) v = 0.0f;
+                        if (iz >= 0 && iz < g.nz && v != 0.0f)
+                            atomicAdd(I.A + (size_t)iy * g.nz + iz, v);
+                    }
+                }
+                __syncthreads();
+                if (phase != kHigh) break;
+                if (tid == 0) s_sums.phase = kLow;
+                __syncthreads();
+            }
         }
-        __syncthreads();
         it = s_item[par];
         par ^= 1;
-        if (MODE != kLoglik) {
-            for (int rr = warp; rr < tl.RH; rr += kWarps) {
-                const int iy = f.oy + rr;
-                if (iy < 0 || iy >= g.ny) continue;
-                const int z0row = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0)));
-                for (int cc = lane; cc < tl.RW; cc += 32) {
-                    const int iz = z0row + cc;
-                    const int k = rr * tl.RS + cc;
-                    float v = (float)s_cnt[k] * quantum;
-                    // (the update is 0 where rho' = 0, whatever A holds)
-                    if (MODE == kMlem && !GLD && !(s_rp[k] > 0.0f)) v = 0.0f;
-                    if (iz >= 0 && iz < g.nz && v != 0.0f)
-                        atomicAdd(I.A + (size_t)iy * g.nz + iz, v);
-                }
-            }
-            __syncthreads();
-        }
     }
     tm_sync_threads();
     if (!BATCH || cur >= 0) flush_block_sums(&s_sums, I.accum, MODE);
