@@ -313,8 +313,13 @@ PassArgs pass_args(tsp_ctx* c)
 // chunks: clear the bin histogram and counters; per chunk, Eq. 2, windows and
 // bin keys (k_setup) for events [first, first + n); then the bin offsets, the
 // work items and the counting-sort scatter into binned order.
+// From here until prep_finish has succeeded the context has no prepared events: an
+// earlier preparation's items and records belong to another plan (their indexes lie
+// outside this one's buffers and regions), so no pass may run over them.
 int prep_begin(tsp_ctx* c, cudaStream_t st)
 {
+    c->uploaded = false;
+    c->rec = false;
     const int nbins = c->nbins;
     if (nbins > c->bins_cap) {
         dfree(c->bin_count);
@@ -414,7 +419,7 @@ int prep_finish(tsp_ctx* c, cudaStream_t st)
                                 cudaMemcpyDeviceToHost, st));
     TSP_CUDA(c, cudaStreamSynchronize(st));
     if (c->counters_h[0] != 0) {
-        c->uploaded = false;
+        c->listed = false;
         c->n = 0;
         return fail(c, TSP_EINVAL, std::to_string(c->counters_h[0]) + " events are not finite");
     }
@@ -454,7 +459,7 @@ int prep_finish(tsp_ctx* c, cudaStream_t st)
         if (int rc = plan(c)) return rc;
         return prepare_events(c, st);
     }
-    c->uploaded = true;
+    c->uploaded = c->listed = true;
     return TSP_OK;
 }
 
@@ -669,7 +674,7 @@ int tsp_begin_events(tsp_ctx* c, int64_t n_total, void* stream)
     DeviceGuard dg(c->dev);
     cudaStream_t st = (cudaStream_t)stream;
     int rc;
-    c->uploaded = false;
+    c->uploaded = c->listed = false;
     c->appending = false;
     clear_graphs(c);
     // work already queued on the stream (a previous preparation reading the
@@ -895,7 +900,7 @@ int tsp_set_sigma(tsp_ctx* c, double sigma_z, double sigma_dl, void* stream)
         return rc;
     }
     clear_graphs(c);
-    if (c->uploaded) {
+    if (c->listed) {
         if ((rc = prepare_events(c, st))) return rc;
         if ((rc = refresh_rhop(c, st))) return rc;
     }
@@ -1004,7 +1009,7 @@ int tsp_set_schedule(tsp_ctx* c, const tsp_schedule* s, void* stream)
         return rc;
     }
     clear_graphs(c);
-    if (c->uploaded && (rc = prepare_events(c, (cudaStream_t)stream))) return rc;
+    if (c->listed && (rc = prepare_events(c, (cudaStream_t)stream))) return rc;
     return TSP_OK;
 }
 

@@ -163,8 +163,8 @@ int rebuild(tsp_batch* b, cudaStream_t st)
         t.evs.geo = c->geo;
         t.evs.geo64 = c->geo64;
         t.evs.rows = c->rows;
-        t.evs.recs = c->recs;
-        t.evs.evc = c->evc;
+        t.evs.recs = c->rec ? c->recs : nullptr;
+        t.evs.evc = c->rec ? c->evc : nullptr;
         t.rhop = c->rhop;
         t.A = c->A;
         t.accum = c->accum;
@@ -379,20 +379,21 @@ int capture_batch(tsp_batch* b, int n_iter, tsp_ctx::Graph* out)
 // re-bins the events; the item split and order only change the merged items.
 int apply_schedule(tsp_batch* b, const tsp_schedule* s, cudaStream_t st)
 {
-    const bool replan = s->ty_cap != b->sched.ty_cap;
+    b->dirty = true;    // (also when a member fails below)
     b->sched.ty_cap = s->ty_cap;
     b->sched.items_per_sm = s->items_per_sm;
     b->sched.order = s->order;
     for (int i = 0; i < (int)b->inst.size(); ++i) {
         tsp_ctx* c = b->inst[i];
+        const bool replan =
+            c->sched.ty_cap != b->sched.ty_cap || (c->listed && !c->uploaded);
         c->sched = b->sched;
         if (replan) {
             int rc = plan(c);
             if (rc) return bfail_inst(b, i, rc);
-            if (c->uploaded && (rc = prepare_events(c, st))) return bfail_inst(b, i, rc);
+            if (c->listed && (rc = prepare_events(c, st))) return bfail_inst(b, i, rc);
         }
     }
-    b->dirty = true;
     return TSP_OK;
 }
 

@@ -85,7 +85,9 @@ struct tsp_ctx {
     int bins_cap = 0;
     unsigned long long prepared = 0;  // lane capacities whose kernels have their limits raised
     int* flag = nullptr;
-    bool uploaded = false, sens_ready = false;
+    // listed: the raw events of a whole accepted list are there (set_sigma and
+    // set_schedule prepare them again); uploaded: and they are prepared, passes may run
+    bool listed = false, uploaded = false, sens_ready = false;
     bool appending = false;           // between tsp_begin_events and tsp_end_events
     long long n_total = 0;            // events declared by tsp_begin_events
     cudaStream_t copy_stream = nullptr;   // host-to-device event copies
