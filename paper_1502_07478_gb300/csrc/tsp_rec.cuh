@@ -527,75 +527,81 @@ __device__ __forceinline__ float2 rec_grad_row(const Geo& g, const float4& ev, f
 }
 
 // Room of the fixed-point accumulator (see k_tiles_rec), in quanta.
-constexpr float kTopTerm = 0.99f * 0x1p24f;   // one event's largest term, of add4
-constexpr float kRoom = 0.99f * 0x1p32f;      // all the events between two flushes
+constexpr float kTopTerm = 0.99f * 0x1p24f;   // one event's largest term
+constexpr float kRoom = 0.99f * 0x1p32f;      // all the events of an item
 
-// Terms above 2^24 quanta are formed in units of 2^shift of them: at least 22 bits of
-// the event's largest one.
-__device__ __forceinline__ int term_shift(float top)
-{
-    return (int)(__float_as_uint(top) >> 23) - 127 - 22;
-}
+// How a pass over an item's events scatters: in one word a term (kWhole), or, for an
+// item whose rho' has a peak that events share (see k_tiles_rec), in two passes, the
+// terms' whole quanta (kHigh) and what these leave of them in units 2^-k (kLow; lo =
+// 2^(k - 149)).
+enum Phase : int { kWhole = 0, kHigh = 1, kLow = 2 };
+constexpr float kTopSplit = 0x1p22f;          // one event's largest term, in two passes
 
-__device__ __forceinline__ void add_shifted(unsigned a, float v, int shift)
+__device__ __forceinline__ void add_split(unsigned a, float p, float s, int phase, float lo)
 {
+    const float t = __fmaf_rz(p, s, kFxMagic);          // bits: magic + floor(p s)
+    unsigned v = __float_as_uint(t) - kFxMagicBits;
+    if (phase == kLow) v = __float_as_uint(__fmaf_rn(p, s, kFxMagic - t) * lo);
 #ifdef TSP_DEBUG_CHECKS
     if (!tsp_sh_ok(a, 4, 2)) return;
 #endif
-    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"(__float_as_uint(v) << shift) : "memory");
+    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
-// The scatter of an event that add4 has no range for: with shift >= 0 into the
-// accumulator (base: as rec_pass2), w = 2^-149 / (D quantum 2^shift); else, where the
-// accumulator has no room for it at all, by float adds to the global A, w = 1/D, each
-// pixel (pix: of the row's origin) under its predicate; with MASK only where rho' > 0
-// (as the flush does).
-template <int TRAV, bool MASK>
-__device__ __noinline__ void rec_scatter_slow(unsigned base, float* A, const float* rhop, int pix,
-                                              int la, int lb, int n, unsigned tma, float w,
-                                              int shift)
+template <int TRAV>
+__device__ __noinline__ void rec_pass2_split(unsigned base, int n, unsigned tma, float s, int phase,
+                                             float lo)
 {
-    auto add = [&](int q, float p) {
-        if (p != 0.0f && (!MASK || rhop[q] > 0.0f)) atomicAdd(A + q, p * w);
-    };
     for (int k = 1; k <= n; k += 2) {
         float x0, x1, x2, x3;
         tm_ld4(tma, x0, x1, x2, x3);
         tm_wait_ld();
-        const int d0 = pair_d0<TRAV>(k), d1 = pair_d1<TRAV>(k);
-        const int d2 = pair_d0<TRAV>(k + 1), d3 = pair_d1<TRAV>(k + 1);
-        if (shift >= 0) {
-            add_shifted(base + (unsigned)(4 * d0), x0 * w, shift);
-            add_shifted(base + (unsigned)(4 * d1), x1 * w, shift);
-            add_shifted(base + (unsigned)(4 * d2), x2 * w, shift);
-            add_shifted(base + (unsigned)(4 * d3), x3 * w, shift);
-        } else {
-            if (k <= la) add(pix + d0, x0);
-            if (k <= lb) add(pix + d1, x1);
-            if (k < la) add(pix + d2, x2);
-            if (k < lb) add(pix + d3, x3);
-        }
-        __syncwarp();
+        add_split(base + (unsigned)(4 * pair_d0<TRAV>(k)), x0, s, phase, lo);
+        add_split(base + (unsigned)(4 * pair_d1<TRAV>(k)), x1, s, phase, lo);
+        add_split(base + (unsigned)(4 * pair_d0<TRAV>(k + 1)), x2, s, phase, lo);
+        add_split(base + (unsigned)(4 * pair_d1<TRAV>(k + 1)), x3, s, phase, lo);
         tma += 4;
     }
 }
 
-// The last `left` of the events first + grp, first + grp + ngroups, ... of an item, by
-// one group of G warps.  inv_q: 1 over the quantum of the fixed-point terms P / D.
-// Returns the number left over, when the accumulator has no room for more before it is
-// flushed (the event at hand is then evaluated again; a group's first always has room).
+// The scatter of an event whose terms the item's accumulator has no room for (see
+// k_tiles_rec): float adds to the global A, each pixel under its predicate; with
+// MASK only where rho' > 0 (as the flush does).
+template <int TRAV, bool MASK>
+__device__ __noinline__ void rec_scatter_global(float* A, const float* rhop, int pix, int la,
+                                                int lb, int n, unsigned tma, float invD)
+{
+    auto add = [&](int q, float p) {
+        if (p != 0.0f && (!MASK || rhop[q] > 0.0f)) atomicAdd(A + q, p * invD);
+    };
+    unsigned col = tma;
+    for (int k = 1; k <= n; k += 2) {
+        float x0, x1, x2, x3;
+        tm_ld4(col, x0, x1, x2, x3);
+        tm_wait_ld();
+        if (k <= la) add(pix + pair_d0<TRAV>(k), x0);
+        if (k <= lb) add(pix + pair_d1<TRAV>(k), x1);
+        if (k < la) add(pix + pair_d0<TRAV>(k + 1), x2);
+        if (k < lb) add(pix + pair_d1<TRAV>(k + 1), x3);
+        __syncwarp();
+        col += 4;
+    }
+}
+
+// The events first + grp, first + grp + ngroups, ... of an item, by one group
+// of G warps.  inv_q: 1 over the quantum of the fixed-point terms P / D.
 template <int TRAV, int LMAX, int MODE, int NSEG, bool GLD>
-__device__ __forceinline__ int rec_events(const Inst& I, const Frame& f, int first, int count,
-                                          int left, int grp, int ngroups, int wig, int lane,
-                                          unsigned rp_addr, unsigned acc_off, unsigned slot,
-                                          float* part, BlockSums* bs, unsigned tma, float inv_q,
-                                          const float* scr)
+__device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int first, int count,
+                                           int grp, int ngroups, int wig, int lane,
+                                           unsigned rp_addr, unsigned acc_off, unsigned slot,
+                                           float* part, BlockSums* bs, unsigned tma, float inv_q,
+                                           const float* scr)
 {
     constexpr bool GRAD = MODE == kGrad;
     const Geo& g = I.g;
     const int G = I.G;
-    if (left <= 0) return 0;
-    first += grp + ((count - grp + ngroups - 1) / ngroups - left) * ngroups;
+    int left = (count - grp + ngroups - 1) / ngroups;
+    if (left <= 0) return;
     // the row block of a warp is rotated by its group (see process_event)
     int blk;
     if constexpr (NSEG == 1) {
@@ -608,8 +614,8 @@ __device__ __forceinline__ int rec_events(const Inst& I, const Frame& f, int fir
     }
     const float rowoff = (float)lane_row(blk * 32 + lane);
     const int rslot = NSEG == 1 ? blk * 32 + lane : (blk * 2 + (wig & 1)) * 32 + lane;
-    const uint2* rp = I.evs.recs + (size_t)first * (32 * G) + rslot;
-    const float4* ep = I.evs.evc + (size_t)first * kEvcFloat4;
+    const uint2* rp = I.evs.recs + (size_t)(first + grp) * (32 * G) + rslot;
+    const float4* ep = I.evs.evc + (size_t)(first + grp) * kEvcFloat4;
     rec_fetch(slot, rp, ep, lane);
     unsigned used = 0;
     float spent = 0.0f;
@@ -665,56 +671,43 @@ __device__ __forceinline__ int rec_events(const Inst& I, const Frame& f, int fir
             parity ^= kMinWarps;
         }
         if (D > 0.0f) {
+            ++used;
+            if (MODE != kMlem && wig == 0 && lane == 0) logD += (double)logf(D);
             if (MODE != kLoglik) {
                 const float r = recip(D), s = r * inv_q, top = s * ev.x;
+                const int phase = bs->phase;
                 // (false for a NaN, and for a D that recip has no value of)
-                const bool fit = top > 0.0f && top <= room;
-                if (fit && spent > 0.0f && spent + top > room) {
-                    ++left;
-                    break;
-                }
-                if (GRAD) {
+                const bool fit = top > 0.0f && top <= (phase == kWhole ? kTopTerm : kTopSplit) &&
+                                 spent + top + 1.0f <= room;
+                if (GRAD && phase != kLow) {
                     // per-lane sums: the rows' terms of an event cancel to a small
                     // part of themselves, so they are added in double precision
                     const float w = fit ? r : 1.0f / D;
                     giz += (double)(E.x * w);
                     gil += (double)(E.y * w);
                 }
-                // (one more than the bound: the rounding of the terms)
-                if (fit) spent = fmaf(top, 1.0001f, spent + 1.0f);
-                if (top <= kTopTerm && fit) {
+                if (fit) {
+                    spent += top + 1.0f;
                     const float q = s * 0x1p-149f;
-                    rec_pass2<TRAV>(base + acc_off, n, tma, make_float2(q, q));
-                } else {
-                    int pix = 0, shift = -1;
-                    float w;
-                    if (fit) {
-                        shift = term_shift(top);
-                        w = s * 0x1p-149f * __uint_as_float((unsigned)(127 - shift) << 23);
-                    } else {
-                        const int rr = (int)idx / f.stride, col = (int)idx - rr * f.stride;
-                        const int iy = f.oy + rr;
-                        pix = iy * g.nz + f.zbase +
-                              (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0))) + col;
-                        w = 1.0f / D;
-                    }
-                    rec_scatter_slow<TRAV, MODE == kMlem && !GLD>(base + acc_off, I.A, I.rhop, pix,
-                                                                  la, lb, n, tma, w, shift);
+                    if (phase == kWhole)
+                        rec_pass2<TRAV>(base + acc_off, n, tma, make_float2(q, q));
+                    else
+                        rec_pass2_split<TRAV>(base + acc_off, n, tma, s, phase, bs->lo);
+                } else if (phase != kLow) {
+                    const int rr = (int)idx / f.stride, col = (int)idx - rr * f.stride;
+                    const int iy = f.oy + rr;
+                    const int iz = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0))) + col;
+                    rec_scatter_global<TRAV, MODE == kMlem && !GLD>(I.A, I.rhop, iy * g.nz + iz, la,
+                                                                    lb, n, tma, 1.0f / D);
                 }
             }
-            ++used;
-            if (MODE != kMlem && wig == 0 && lane == 0) logD += (double)logf(D);
         }
         if (left == 0) break;
     }
-    rec_wait();
+    if (bs->phase == kLow) return;      // counted in the first pass
     if (wig == 0 && lane == 0) {
         if (used) atomicAdd(&bs->used, (unsigned long long)used);
         if (MODE != kMlem) atomicAdd(&bs->logD, logD + used * (g.pshift * 0.69314718055994530942));
-        if (MODE != kLoglik) {
-            atomicAdd(&bs->spent, spent);
-            if (left) atomicAdd(&bs->left, left);
-        }
     }
     if (GRAD) {
         for (int o = 16; o > 0; o >>= 1) {
@@ -726,7 +719,6 @@ __device__ __forceinline__ int rec_events(const Inst& I, const Frame& f, int fir
             atomicAdd(&bs->gil, gil);
         }
     }
-    return left;
 }
 
 // ---- Two rows a lane -----------------------------------------------------------
@@ -901,71 +893,75 @@ __device__ __forceinline__ void rec2_pass2(unsigned a0, unsigned a1, int n, unsi
     }
 }
 
-// The scatter of rows whose event rec2_pass2 has no range for (see rec_scatter_slow):
-// a lane's shift >= 0 into the accumulator (a0, a1: addresses of the rows' origins), -1
-// to the global A (p0, p1: pixels of the origins), -2 nothing.
+// In two passes (see Phase).
+static __device__ __noinline__ void rec2_pass2_split(unsigned a0, unsigned a1, int n, unsigned tma, float s,
+                                              int phase, float lo)
+{
+    for (int k = 1; k <= n; ++k) {
+        float x0, x1, x2, x3;
+        tm_ld4(tma, x0, x1, x2, x3);
+        tm_wait_ld();
+        add_split(a0 + 4u * k, x0, s, phase, lo);
+        add_split(a1 + 4u * k, x1, s, phase, lo);
+        add_split(a0 - 4u * (k - 1), x2, s, phase, lo);
+        add_split(a1 - 4u * (k - 1), x3, s, phase, lo);
+        tma += 4;
+    }
+}
+
+// The scatter of rows that the item's accumulator has no room for (see
+// rec_scatter_global); live: the lane's event is one of those.
 template <bool MASK>
-__device__ __noinline__ void rec2_scatter_slow(unsigned a0, unsigned a1, float* A,
-                                               const float* rhop, int p0, int p1, unsigned n0,
-                                               unsigned n1, int n, unsigned tma, float w, int shift)
+__device__ __noinline__ void rec2_scatter_global(float* A, const float* rhop, int p0, int p1,
+                                                 int la0, int lb0, int la1, int lb1, int n,
+                                                 unsigned tma, float invD, bool live)
 {
     auto add = [&](int q, float p) {
-        if (p != 0.0f && (!MASK || rhop[q] > 0.0f)) atomicAdd(A + q, p * w);
+        if (p != 0.0f && (!MASK || rhop[q] > 0.0f)) atomicAdd(A + q, p * invD);
     };
     for (int k = 1; k <= n; ++k) {
         float x0, x1, x2, x3;
         tm_ld4(tma, x0, x1, x2, x3);
         tm_wait_ld();
-        if (shift >= 0) {
-            add_shifted(a0 + 4u * k, x0 * w, shift);
-            add_shifted(a1 + 4u * k, x1 * w, shift);
-            add_shifted(a0 - 4u * (k - 1), x2 * w, shift);
-            add_shifted(a1 - 4u * (k - 1), x3 * w, shift);
-        } else if (shift == -1) {
-            if (k <= (int)(n0 & 0xff)) add(p0 + k, x0);
-            if (k <= (int)(n1 & 0xff)) add(p1 + k, x1);
-            if (k <= (int)(n0 >> 8)) add(p0 + 1 - k, x2);
-            if (k <= (int)(n1 >> 8)) add(p1 + 1 - k, x3);
+        if (live) {
+            if (k <= la0) add(p0 + k, x0);
+            if (k <= la1) add(p1 + k, x1);
+            if (k <= lb0) add(p0 + 1 - k, x2);
+            if (k <= lb1) add(p1 + 1 - k, x3);
         }
         __syncwarp();
         tma += 4;
     }
 }
 
-// The groups of the two-row form: with G = 1 (up to 32 rows) a half warp an event, else
-// (G + 1) / 2 warps.  The first group of this warp, and their number.
-__device__ __forceinline__ int2 rec2_groups(int G, int warp)
-{
-    if (G == 1) return make_int2(2 * warp, 2 * kMaxWarps);
-    const int G2 = (G + 1) >> 1;
-    return make_int2(warp / G2, group_count(kMaxWarps, G2));
-}
-
-// The last `left` events of this warp's first group (see rec_events), and the second
-// half's, which may end one sooner.
+// The events of an item for this warp: with G = 1 (up to 32 rows) a half warp
+// each, else groups of (G + 1) / 2 warps.
 template <int MODE>
-__device__ __forceinline__ int rec2_events(const Inst& I, const Frame& f, int first, int count,
-                                           int left, int warp, int lane, unsigned rp_addr,
-                                           unsigned acc_off, unsigned slot, float* s_part,
-                                           BlockSums* bs, unsigned tma, float inv_q)
+__device__ __forceinline__ void rec2_events(const Inst& I, const Frame& f, int first, int count,
+                                            int warp, int lane, unsigned rp_addr, unsigned acc_off,
+                                            unsigned slot, float* s_part, BlockSums* bs,
+                                            unsigned tma, float inv_q)
 {
     const Geo& g = I.g;
     const int G = I.G;
-    if (left <= 0) return 0;
     const bool halves = G == 1;
     const int G2 = (G + 1) >> 1;
     const int wgrp = warp / G2, wig = warp - wgrp * G2;
-    const int2 gr = rec2_groups(G, warp);
-    const int ngroups = gr.y;
-    // (the row block of a warp is rotated by its group)
+    const int ngroups = halves ? 2 * kMaxWarps : group_count(kMaxWarps, G2);
+    // group, and pair of rows (the row block of a warp is rotated by its group)
+    const int grp = halves ? 2 * warp + (lane >> 4) : wgrp;
     int blk = wig + wgrp % G2;
     blk -= blk >= G2 ? G2 : 0;
     int p = halves ? lane & 15 : blk * 32 + lane;
     const bool has_rows = p < 16 * G;
     const float2 rowoff = make_float2((float)-p, (float)(p + 1));
     p = min(p, 16 * G - 1);
-    int e = gr.x + (halves ? lane >> 4 : 0) +
-            ((count - gr.x + ngroups - 1) / ngroups - left) * ngroups;
+    // events left of the warp's first group (the second half's may end one sooner)
+    const int lead = halves ? 2 * warp : wgrp;
+    if (!halves && wgrp >= ngroups) return;
+    int left = (count - lead + ngroups - 1) / ngroups;
+    if (left <= 0) return;
+    int e = grp;
     const uint4* const recs = reinterpret_cast<const uint4*>(I.evs.recs) + p;
     const float4* const evc = I.evs.evc;
     const int cl = halves ? lane & 15 : lane;
@@ -1019,55 +1015,44 @@ __device__ __forceinline__ int rec2_events(const Inst& I, const Frame& f, int fi
             D = group_sum(D, G2, wig, lane, 1 + wgrp, part + parity);
             parity ^= kMinWarps;
         }
-        // (a second half beyond the list has no pixels: D = 0)
         const bool on = D > 0.0f;
-        if (MODE != kLoglik) {
-            const float r = recip(D), s = r * inv_q, top = s * pmax;
-            // (false for a NaN, and for a D that recip has no value of)
-            const bool fit = on && top > 0.0f && top <= room;
-            if (__any_sync(0xffffffffu, fit && spent > 0.0f && spent + top > room)) {
-                ++left;
-                break;
-            }
-            // (one more than the bound: the rounding of the terms)
-            if (fit) spent = fmaf(top, 1.0001f, spent + 1.0f);
-            const bool fast = fit && top <= kTopTerm;
-            if (__any_sync(0xffffffffu, fast))
-                rec2_pass2(a0 + acc_off, a1 + acc_off, kmax, tma, dup(fast ? s * 0x1p-149f : 0.0f));
-            if (__any_sync(0xffffffffu, on && !fast)) {
-                auto pix = [&](unsigned i) {
-                    const int rr = (int)i / f.stride, iy = f.oy + rr;
-                    return iy * g.nz + f.zbase +
-                           (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0))) + (int)i - rr * f.stride;
-                };
-                int shift = on && !fast ? -1 : -2;
-                float v = 1.0f / D;
-                if (fit && !fast) {
-                    shift = term_shift(top);
-                    v = s * 0x1p-149f * __uint_as_float((unsigned)(127 - shift) << 23);
-                }
-                rec2_scatter_slow<MODE == kMlem>(a0 + acc_off, a1 + acc_off, I.A, I.rhop, pix(i0),
-                                                 pix(i1), n0, n1, kmax, tma, v, shift);
-            }
-        }
         if (on) {
             ++used;
             if (MODE != kMlem && (halves ? (lane & 15) == 0 : wig == 0 && lane == 0))
                 logD += (double)logf(D);
         }
+        if (MODE != kLoglik) {
+            const float r = recip(D), s = r * inv_q, top = s * pmax;
+            const int phase = bs->phase;
+            // (false for a NaN, and for a D that recip has no value of)
+            const bool fit = on && top > 0.0f && top <= (phase == kWhole ? kTopTerm : kTopSplit) &&
+                             spent + top + 1.0f <= room;
+            if (fit) spent += top + 1.0f;
+            if (__any_sync(0xffffffffu, fit)) {
+                if (phase == kWhole)
+                    rec2_pass2(a0 + acc_off, a1 + acc_off, kmax, tma,
+                               dup(fit ? s * 0x1p-149f : 0.0f));
+                else
+                    rec2_pass2_split(a0 + acc_off, a1 + acc_off, kmax, tma, fit ? s : 0.0f, phase,
+                                     bs->lo);
+            }
+            if (phase != kLow && __any_sync(0xffffffffu, on && !fit)) {
+                auto pix = [&](unsigned i) {
+                    const int rr = (int)i / f.stride, iy = f.oy + rr;
+                    return iy * g.nz + f.zbase +
+                           (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0))) + (int)i - rr * f.stride;
+                };
+                rec2_scatter_global<MODE == kMlem>(I.A, I.rhop, pix(i0), pix(i1), la0, lb0, la1,
+                                                   lb1, kmax, tma, 1.0f / D, on && !fit);
+            }
+        }
         if (left == 0) break;
     }
-    rec_wait();
-    if (halves ? (lane & 15) == 0 : wig == 0 && lane == 0) {
-        if (used) atomicAdd(&bs->used, (unsigned long long)used);
-        if (MODE != kMlem && used)
-            atomicAdd(&bs->logD, logD + used * (g.pshift * 0.69314718055994530942));
-        if (MODE != kLoglik) {
-            atomicAdd(&bs->spent, spent);
-            if (left) atomicAdd(&bs->left, left);
-        }
+    if (bs->phase == kLow) return;      // counted in the first pass
+    if (used && (halves ? (lane & 15) == 0 : wig == 0 && lane == 0)) {
+        atomicAdd(&bs->used, (unsigned long long)used);
+        if (MODE != kMlem) atomicAdd(&bs->logD, logD + used * (g.pshift * 0.69314718055994530942));
     }
-    return left;
 }
 
 // Persistent tile kernel over window records.  Work
