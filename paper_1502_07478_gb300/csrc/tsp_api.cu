@@ -359,6 +359,9 @@ int build_records(tsp_ctx* c, cudaStream_t st)
     // (a batch takes the events of such a member through global memory)
     if (c->gld && c->batch_member) return TSP_OK;
     if (c->gld && c->tl.RH > kScrRows) return TSP_OK;
+    // (their passes stage some 11 KB that the general ones of accumulator-only tiles do not)
+    if (rec_smem_floats(c->tl.RH, c->tl.RS, c->gld != 0) * sizeof(float) > dyn_smem_limit(c->dev))
+        return TSP_OK;
     const size_t per = record_bytes(c->G);
     const size_t need = (per + kEvcBytes) * (size_t)placed;
     if (sim_fault() == kSimRecords) return TSP_OK;
