@@ -122,7 +122,14 @@ const char* tsp_version(void);
  * 3-sigma window's bounding box of App. B, and the binning of events by the
  * image tile holding their window centre.  zu, zd, dl: n floats each, host or
  * device (on_device).  n = 0 is valid (an empty list).  Non-finite values give
- * TSP_EINVAL and upload nothing.  The image is reset to rho = 1. */
+ * TSP_EINVAL and upload nothing.  The image is reset to rho = 1.
+ *
+ * Device memory: some 130 bytes an event.  For a dense list (64 events over a pixel and
+ * more) window records beside them, 64 bytes and 8 for each row of the highest
+ * window, rounded up to 32 (1.1 KB an event at 1 mm, 0.6 at 2 mm), if that is at most a
+ * quarter of the memory that is then free (of a batch: all its members' together);
+ * otherwise the passes do without, more slowly.  The records' memory is given back when
+ * a list without them follows, or one that needs larger event buffers. */
 int tsp_upload_events(tsp_ctx* ctx, const float* zu, const float* zd, const float* dl,
                       int64_t n, int on_device, void* stream);
 

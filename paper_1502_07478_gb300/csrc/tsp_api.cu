@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "tsp_ctx.h"
+#include "tsp_records_budget.h"
 
 using namespace tsp;
 
@@ -347,29 +348,44 @@ int prep_chunk(tsp_ctx* c, long long first, long long n, cudaStream_t st)
     return TSP_OK;
 }
 
-// Window records of the placed events.  They are kept when they take at most a
-// quarter of the memory that is free when their buffer has to grow (6e7 events
-// at 1 mm on an empty 280 GB); otherwise, or when the allocation fails, the
-// passes set the rows up themselves.  So do those of sparse lists (kRecCoverage).
+// Gives the records' memory back.
+void drop_records(tsp_ctx* c)
+{
+    c->rec = false;
+    dfree(c->recbuf);
+    dfree(c->scratch);
+    c->rec_cap = c->scratch_cap = 0;
+}
+
+// Whether the prepared list is to have window records: not a sparse one (kRecCoverage).
+bool records_wanted(const tsp_ctx* c)
+{
+    if (c->n_items == 0 || c->outlier_first == 0 || coverage(c) < kRecCoverage) return false;
+    // (a batch takes the events of such a member through global memory)
+    if (c->gld && (c->batch_member || c->tl.RH > kScrRows)) return false;
+    // (their passes stage some 11 KB that the general ones of accumulator-only tiles do not)
+    return rec_smem_floats(c->tl.RH, c->tl.RS, c->gld != 0) * sizeof(float) <=
+           dyn_smem_limit(c->dev);
+}
+
+// Window records of the placed events.  They are kept when there is memory for them
+// (records_allowed); otherwise, or when the allocation fails, the passes set the rows up
+// themselves.  The memory is given back when a list without records follows.
 int build_records(tsp_ctx* c, cudaStream_t st)
 {
     c->rec = false;
     const long long placed = c->outlier_first;
-    if (c->n_items == 0 || placed == 0 || coverage(c) < kRecCoverage) return TSP_OK;
-    // (a batch takes the events of such a member through global memory)
-    if (c->gld && c->batch_member) return TSP_OK;
-    if (c->gld && c->tl.RH > kScrRows) return TSP_OK;
-    // (their passes stage some 11 KB that the general ones of accumulator-only tiles do not)
-    if (rec_smem_floats(c->tl.RH, c->tl.RS, c->gld != 0) * sizeof(float) > dyn_smem_limit(c->dev))
+    if (!records_wanted(c) || sim_fault() == kSimRecords) {
+        drop_records(c);
         return TSP_OK;
+    }
     const size_t per = record_bytes(c->G);
     const size_t need = (per + kEvcBytes) * (size_t)placed;
-    if (sim_fault() == kSimRecords) return TSP_OK;
     if (need > c->rec_cap) {
-        dfree(c->recbuf);
-        c->rec_cap = 0;
+        drop_records(c);
         size_t avail = 0, total = 0;
-        if (cudaMemGetInfo(&avail, &total) != cudaSuccess || need > avail / 4 ||
+        if (cudaMemGetInfo(&avail, &total) != cudaSuccess ||
+            !records_allowed(need, c->rec_others, avail) ||
             dmalloc(&c->recbuf, need) != cudaSuccess) {
             cudaGetLastError();
             c->recbuf = nullptr;
@@ -377,7 +393,10 @@ int build_records(tsp_ctx* c, cudaStream_t st)
         }
         c->rec_cap = need;
     }
-    if (c->gld) {
+    if (!c->gld) {
+        dfree(c->scratch);
+        c->scratch_cap = 0;
+    } else {
         const size_t scr = (size_t)c->num_sms * c->tl.RS * kScrRows;
         if (scr > c->scratch_cap) {
             dfree(c->scratch);
@@ -385,6 +404,7 @@ int build_records(tsp_ctx* c, cudaStream_t st)
             if (dmalloc(&c->scratch, scr * sizeof(float)) != cudaSuccess) {
                 cudaGetLastError();
                 c->scratch = nullptr;
+                drop_records(c);
                 return TSP_OK;
             }
             c->scratch_cap = scr;
@@ -505,6 +525,7 @@ std::vector<int4> tile_items(const tsp_ctx* c, long long E, int w)
 int ensure_event_capacity(tsp_ctx* c, long long n)
 {
     if (n <= c->cap) return TSP_OK;
+    drop_records(c);    // (of the last list: the event buffers come first)
     dfree(c->zu);
     dfree(c->zd);
     dfree(c->dl);
@@ -662,8 +683,7 @@ void tsp_destroy(tsp_ctx* c)
     dfree(c->zu); dfree(c->zd); dfree(c->dl);
     dfree(c->geo_u); dfree(c->geo); dfree(c->geo64_u); dfree(c->geo64);
     dfree(c->rows_u); dfree(c->rows); dfree(c->key);
-    dfree(c->recbuf);
-    dfree(c->scratch);
+    drop_records(c);
     dfree(c->items); dfree(c->bin_count); dfree(c->offsets);
     delete c;
 }

@@ -63,6 +63,7 @@ struct tsp_ctx {
     // current upload are there
     unsigned char* recbuf = nullptr;
     size_t rec_cap = 0;               // bytes of recbuf
+    size_t rec_others = 0;            // of the other members of the batch
     uint2* recs = nullptr;
     float4* evc = nullptr;
     bool rec = false;

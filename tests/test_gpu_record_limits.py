@@ -29,3 +29,32 @@ def test_accumulator_tiles_at_the_shared_memory_limit():
     m = ref > 0.01 * ref.max()
     assert st["n_used"] == rs.n_used
     assert np.max(np.abs(img[m] - ref[m]) / ref[m]) <= 1e-4
+
+
+def _free():
+    import torch
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+def test_record_memory_is_given_back():
+    """2e5 dense events at 2 mm hold some 120 MB of records; a sparse list after them none."""
+    from paper_1502_07478_gb300 import Recon
+    w = replace(make_workload("small_5mm"), ny=350, nz=250, n_events=200_000)
+    ev = w.events()
+    few = [x[:1000] for x in ev]
+    r = Recon.from_workload(w)
+    r.begin_events(200_000)             # (event buffers of the long list, no records)
+    r.append_events(*few)
+    r.end_events()
+    base = _free()
+    r.upload_events(*ev)
+    held = base - _free()
+    assert held >= 100 << 20
+    r.upload_events(*few)
+    assert base - _free() <= 8 << 20
+    r.upload_events(*ev)
+    r.iterate(1)
+    st = r.stats()
+    assert st["sum_s_rho"] == pytest.approx(st["n_used"], rel=2e-6)
+    r.close()
