@@ -32,7 +32,8 @@
  *    launch (kernel launches fail before anything is enqueued: TSP_ECUDA),
  *    nan_event (each uploaded chunk gets a NaN z_u: TSP_EINVAL), records (the
  *    window records' buffer cannot be had: no error, the passes then set each
- *    window's rows up themselves) or timeout
+ *    window's rows up themselves), norecords (the same, known when the list is
+ *    declared) or timeout
  *    (tsp_wait gives up at once: TSP_ETIMEOUT) simulates that
  *    failure at every site it reaches while it is set.  A context whose call
  *    failed this way can still be destroyed, and new contexts work once the

@@ -86,6 +86,20 @@ static bool dense_list(const tsp_ctx* c, double umax, double hy, double dy, doub
     return c->n_total * pixels >= 2.0 * kRecCoverage * c->p.ny * c->p.nz;
 }
 
+// Whether the records of the declared list would be allowed (records_allowed), for plan:
+// a list whose records are refused after it was tiled for them is prepared twice.
+// Asked only for lists of more than 1/64 of the device's memory (the query takes longer
+// than a small list's preparation).
+static bool records_fit(const tsp_ctx* c)
+{
+    if (sim_fault() == kSimNoRecords) return false;
+    const size_t need = (record_bytes(c->G) + kEvcBytes) * (size_t)c->n_total;
+    if (need <= std::max(c->rec_cap, c->dev_mem / 64)) return true;
+    size_t avail = 0, total = 0;
+    return cudaMemGetInfo(&avail, &total) == cudaSuccess &&
+           records_allowed(need, c->rec_others, avail + c->rec_cap);
+}
+
 // Derive the kernel constants, lane capacity, group size and tiling from the
 // parameters.  Returns TSP_OK or TSP_EINVAL.
 int plan(tsp_ctx* c)
@@ -146,7 +160,7 @@ int plan(tsp_ctx* c)
     // is cut into as few tiles as the shared memory allows until a tile has some 64
     // events: five updates of 2e5 events at 1 mm 4.18 -> 4.04 ms, one of 1e6 3.50 ->
     // 3.35 ms, five of 2e4 at 5 mm 275 -> 262 us.
-    c->wide = !c->no_wide && dense_list(c, umax, hy, dy, dz);
+    c->wide = !c->no_wide && dense_list(c, umax, hy, dy, dz) && records_fit(c);
     while (TY > 4 && !fits(TY, RS)) TY -= 4;
     c->gld = 0;
     if (!fits(TY, RS) || RS - 1 - 2 * tl.HZ < 1) c->wide = false;
@@ -375,7 +389,7 @@ int build_records(tsp_ctx* c, cudaStream_t st)
 {
     c->rec = false;
     const long long placed = c->outlier_first;
-    if (!records_wanted(c) || sim_fault() == kSimRecords) {
+    if (!records_wanted(c) || sim_fault() == kSimRecords || sim_fault() == kSimNoRecords) {
         drop_records(c);
         return TSP_OK;
     }
@@ -637,6 +651,11 @@ int tsp_create(const tsp_params* params, tsp_ctx** out)
         cudaGetLastError();
         c->err = "cudaDeviceGetAttribute(MultiProcessorCount) failed";
         return bail(TSP_ECUDA);
+    }
+    size_t avail = 0;
+    if (cudaMemGetInfo(&avail, &c->dev_mem) != cudaSuccess) {
+        cudaGetLastError();
+        c->dev_mem = 0;
     }
     if ((rc = plan(c))) return bail(rc);
     c->npix = params->ny * params->nz;

@@ -64,6 +64,7 @@ struct tsp_ctx {
     unsigned char* recbuf = nullptr;
     size_t rec_cap = 0;               // bytes of recbuf
     size_t rec_others = 0;            // of the other members of the batch
+    size_t dev_mem = 0;               // the device's memory
     uint2* recs = nullptr;
     float4* evc = nullptr;
     bool rec = false;

@@ -436,6 +436,7 @@ int sim_fault()
     if (!std::strcmp(v, "nan_event")) return kSimNan;
     if (!std::strcmp(v, "timeout")) return kSimTimeout;
     if (!std::strcmp(v, "records")) return kSimRecords;
+    if (!std::strcmp(v, "norecords")) return kSimNoRecords;
     return kSimNone;
 }
 

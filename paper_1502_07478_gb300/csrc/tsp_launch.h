@@ -27,10 +27,13 @@ bool cinv_valid(const tsp_params& p);
 //              (the event preparation rejects the upload: TSP_EINVAL)
 //   records    the window records' buffer cannot be had (no error: the passes
 //              set the rows up themselves)
+//   norecords  the memory report leaves no room for them: as records, but known when
+//              the list is declared
 //   timeout    the bounded wait (tsp_wait) gives up at once, as when the
 //              enqueued work outlasts the limit (TSP_ETIMEOUT)
 // Unset or any other value: no fault.
-enum SimFault : int { kSimNone = 0, kSimOom = 1, kSimLaunch = 2, kSimNan = 3, kSimTimeout = 4, kSimRecords = 5 };
+enum SimFault : int { kSimNone = 0, kSimOom = 1, kSimLaunch = 2, kSimNan = 3, kSimTimeout = 4, kSimRecords = 5,
+                      kSimNoRecords = 6 };
 int sim_fault();
 
 // The error a launch helper returns under TSP_SIM_FAULT=launch, else success.

@@ -58,3 +58,25 @@ def test_record_memory_is_given_back():
     st = r.stats()
     assert st["sum_s_rho"] == pytest.approx(st["n_used"], rel=2e-6)
     r.close()
+
+
+def test_a_list_without_room_for_records_is_prepared_once(monkeypatch):
+    """A list long enough for wide tiles: refused after the preparation it is prepared
+    again for the general passes (two launches more); when the memory report says so
+    beforehand it is tiled for them at once."""
+    from paper_1502_07478_gb300 import Recon
+    w = make_workload("small_5mm", n_events=20_000)
+    ev = w.events()
+    launches, images = {}, {}
+    for fault in ("", "records", "norecords"):
+        monkeypatch.setenv("TSP_SIM_FAULT", fault)
+        r = Recon.from_workload(w)
+        r.upload_events(*ev)
+        launches[fault] = r.stats()["launches"]
+        r.iterate(1)
+        images[fault] = r.read_image().cpu().numpy().astype(np.float64)
+        r.close()
+    assert launches["norecords"] == launches[""] - 1       # no launch of the records' kernel
+    assert launches["records"] == launches["norecords"] + 2
+    for f in ("records", "norecords"):
+        assert np.abs(images[f] - images[""]).max() <= 2e-5 * images[""].max()
