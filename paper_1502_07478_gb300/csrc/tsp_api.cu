@@ -336,6 +336,7 @@ int prep_begin(tsp_ctx* c, cudaStream_t st)
     c->uploaded = false;
     c->rec = false;
     const int nbins = c->nbins;
+    const bool first = c->bin_count == nullptr;
     if (nbins > c->bins_cap) {
         dfree(c->bin_count);
         dfree(c->offsets);
@@ -345,7 +346,7 @@ int prep_begin(tsp_ctx* c, cudaStream_t st)
         c->bins_cap = nbins;
     }
     // work queued on any stream that reads an earlier preparation
-    TSP_CUDA(c, cudaDeviceSynchronize());
+    if (!first) TSP_CUDA(c, cudaDeviceSynchronize());
     c->cursor = c->bin_count + nbins;
     TSP_CUDA(c, cudaMemsetAsync(c->bin_count, 0, 2 * sizeof(int) * nbins, st));
     TSP_CUDA(c, cudaMemsetAsync(c->counters, 0, sizeof(unsigned long long) * 4, st));

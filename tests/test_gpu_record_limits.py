@@ -65,7 +65,7 @@ def test_a_list_without_room_for_records_is_prepared_once(monkeypatch):
     again for the general passes (two launches more); when the memory report says so
     beforehand it is tiled for them at once."""
     from paper_1502_07478_gb300 import Recon
-    w = make_workload("small_5mm", n_events=20_000)
+    w = make_workload("small_5mm", n_events=800_000)
     ev = w.events()
     launches, images = {}, {}
     for fault in ("", "records", "norecords"):
@@ -80,3 +80,25 @@ def test_a_list_without_room_for_records_is_prepared_once(monkeypatch):
     assert launches["records"] == launches["norecords"] + 2
     for f in ("records", "norecords"):
         assert np.abs(images[f] - images[""]).max() <= 2e-5 * images[""].max()
+
+
+def test_first_upload_does_not_wait_for_other_streams():
+    """A fresh context has nothing that its first preparation could disturb: work of
+    another stream (a bounded spin of some 0.3 s) is still running when it returns."""
+    import torch
+    from paper_1502_07478_gb300 import Recon
+    w = make_workload("small_5mm", n_events=20_000)
+    ev = [torch.from_numpy(x).cuda() for x in w.events()]
+    for _ in range(2):                      # (the first round loads the kernels)
+        r = Recon.from_workload(w)
+        side, mine = torch.cuda.Stream(), torch.cuda.Stream()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(600_000_000)
+            done = torch.cuda.Event()
+            done.record()
+        r.upload_events(*ev, stream=mine)
+        running = not done.query()
+        torch.cuda.synchronize()
+        r.close()
+    assert running
