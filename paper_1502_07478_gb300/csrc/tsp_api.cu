@@ -75,7 +75,7 @@ size_t dyn_smem_limit(int dev)
 
 // Sparse lists, with fewer than kRecCoverage events over a pixel, keep the general
 // passes: one word of fixed point has no room for both the headroom and the precision
-// that a sum of few terms needs (see fx_bits), and their two-word accumulator has.
+// that a sum of few terms needs (see k_tiles_rec), and their two-word accumulator has.
 constexpr double kRecCoverage = 64.0;
 
 // Whether the declared list will have window records, by a margin: the mean window is
@@ -281,17 +281,16 @@ float fx_peak(const tsp_ctx* c)
     return c->counters_h[3] ? (float)(n / (mean * (double)c->counters_h[3])) : 1.0f;
 }
 
-// An ordinary event's largest term takes fx_bits bits.  Its mean term is then some
-// 2^(fx_bits - 2.2) quanta, each rounded to the nearest one, and over the cov events
-// of a pixel the rounding of A is 0.3 x 2^(2.2 - fx_bits) / sqrt(cov) of it: with
-//   fx_bits = 24.4 - log2(cov / 64) / 2
-// some 1e-8 for every list (4e-8 at 64 events a pixel, where 22 bits are
-// the most), which the float sums of the denominators (some 3e-7) hide.  The rest up
-// to 2^24 is the headroom of single events.
+// Bits of an ordinary event's largest term.  Its mean term is then some 2^(fx_bits - 2.2)
+// quanta, each rounded to the nearest one, and over the cov events of a pixel the
+// rounding of A is 0.3 x 2^(2.2 - fx_bits) / sqrt(cov) of it: 4e-8 or less with
+//   fx_bits = 25 - log2(cov) / 2,
+// and 20 at most (1.6e-7 at the 64 events a pixel where the records begin, 4e-8 at 1000),
+// which the float sums of the denominators (some 3e-7) hide.  The rest up to 2^24, the
+// bound of the plain scatter, is the headroom of events that see less than others.
 int fx_bits(const tsp_ctx* c)
 {
-    const double cov = std::max(coverage(c), 1.0);
-    return std::max(12, std::min(22, (int)std::lround(24.4 - 0.5 * std::log2(cov / 64.0))));
+    return std::max(17, std::min(20, (int)std::lround(25.0 - 0.5 * std::log2(std::max(coverage(c), 1.0)))));
 }
 
 PassArgs pass_args(tsp_ctx* c)

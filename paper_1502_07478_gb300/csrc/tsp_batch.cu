@@ -178,8 +178,7 @@ int rebuild(tsp_batch* b, cudaStream_t st)
         t.A = c->A;
         t.accum = c->accum;
         t.G = c->G;
-        t.fx_peak = fx_peak(c);
-        t.fx_bits = fx_bits(c);
+        set_bands(t, fx_peak(c), fx_bits(c));
         t.scratch = nullptr;
         BatchImg& m = imgs[i];
         m.rho = c->rho;

@@ -163,8 +163,8 @@ long long item_events(long long placed, int items_per_sm, int sms);
 int ensure_sensitivity(tsp_ctx* c, cudaStream_t st);
 int refresh_rhop(tsp_ctx* c, cudaStream_t st);
 // The fixed point of the passes over window records (Inst::fx_peak, fx_bits).
-float fx_peak(const tsp_ctx* c);
 int fx_bits(const tsp_ctx* c);
+float fx_peak(const tsp_ctx* c);
 void clear_graphs(tsp_ctx* c);
 
 }  // namespace tsp_host

@@ -67,8 +67,10 @@ struct Geo {
     // z-dependent resolution (Sec. 3): an event at z~ has sigma_z f,
     // f = 1 + kz min(1, zs2 z~^2); kz = 0 keeps sigma_z constant
     float kz, zs2;          // kappa_z, (2/L)^2
-    // the passes over window records hold P 2^-pshift (a whole number; 0 with
-    // lengths in mm), so that a kernel value is near 2^-22 in any unit of length
+    // the passes over window records hold P 2^-pshift (a whole number), so that
+    // a kernel value is near 2^-12 in any unit of length.  (Unscaled, near 2^-22 with
+    // lengths in mm, its exponent is held with 2^-20 rounding; so with half of that.
+    // Nearer to 1 it gains nothing more.)
     float pshift, pad0;
     // double-precision copies for the exact window decision near its boundary
     double y0d, z0d, dyd, dzd, Rd, izd, ild, cut2d;
@@ -312,14 +314,18 @@ struct Inst {
     const float* rhop;
     float* A;
     Accum* accum;
+    float* scratch;     // rho' regions of the blocks, transposed (kScrRows), or null
     // fixed point of the passes over window records (see k_tiles_rec): 1 / (mean
     // of P / max P over a window x mean pixels of a window), and the bits of an
     // ordinary event's largest term
     float fx_peak;
     int fx_bits;
-    float* scratch;     // rho' regions of the blocks, transposed (kScrRows), or null
+    // bands of fx_rows rows of a tile's region, at most 32: those that hold window centres,
+    // the bands on either side that such a window reaches, and 1 over the pixels of the
+    // box of these
+    int fx_rows, fx_first, fx_last, fx_half;
+    float fx_box;
     int G;
-    int pad;
 };
 static_assert(sizeof(Inst) % 8 == 0, "Inst is copied in 8-byte words");
 

@@ -400,7 +400,7 @@ Geo make_geo(const tsp_params& p)
     const double det = iz * iz * il - 2.0 * iz * gm * gm;
     g.log2K = (float)std::log2(std::sqrt(det) / (2.0 * pi * pi));
     g.pshift = (float)std::floor(std::log2(std::sqrt(det) / (2.0 * pi * pi)) -
-                                 0.5 * std::log2(2.0 * iz * p.R * p.R) + 22.5);
+                                 0.5 * std::log2(2.0 * iz * p.R * p.R) + 12.5);
     g.pad0 = 0.0f;
     g.ksu = (float)std::sqrt(log2e * iz);
     g.kA = (float)std::sqrt(log2e / 2.0);

@@ -125,6 +125,19 @@ struct PassArgs {
     size_t rec_smem;   // and of its form over window records
 };
 
+// The fixed point of the passes over window records (Inst::fx_*), once tl is set.
+inline void set_bands(Inst& p, float fx_peak, int fx_bits)
+{
+    const Tiling& tl = p.tl;
+    p.fx_peak = fx_peak;
+    p.fx_bits = fx_bits;
+    p.fx_rows = tl.RH > 32 ? (tl.RH + 31) / 32 : 1;
+    p.fx_first = tl.HY / p.fx_rows;
+    p.fx_last = (tl.HY + tl.TY - 1) / p.fx_rows;
+    p.fx_half = (tl.HY + p.fx_rows - 1) / p.fx_rows;
+    p.fx_box = 1.0f / ((2.0f * p.fx_half + 1.0f) * p.fx_rows * 2.0f * tl.HZ);
+}
+
 // Window records of a list's binned events (tsp_rec.cuh): written once per
 // upload by launch_records, over the plain tile items.
 struct RecArgs {

@@ -84,9 +84,6 @@ struct RowK {
 struct BlockSums {
     unsigned long long used, qclip, lclip, pad;
     double logD, giz, gil, pad2;
-    // the scatter of the item at hand (tsp_rec.cuh: Phase)
-    int phase;
-    float quantum, lo, lo_quantum;
 };
 
 // Extra row constants of the sigma-gradient (adjoint) pass:
@@ -1166,7 +1163,6 @@ __device__ __forceinline__ void init_block_sums(BlockSums* bs)
 {
     if (threadIdx.x == 0) {
         bs->used = bs->qclip = bs->lclip = 0ull;
-        bs->phase = 0;
         bs->logD = bs->giz = bs->gil = 0.0;
     }
 }

@@ -25,10 +25,8 @@ cudaError_t run_pass(const PassArgs& a, cudaStream_t st)
         p.A = a.A;
         p.accum = a.accum;
         p.G = a.G;
-        p.fx_peak = a.fx_peak;
-        p.fx_bits = a.fx_bits;
+        set_bands(p, a.fx_peak, a.fx_bits);
         p.scratch = a.scratch;
-        p.pad = 0;
         if (a.evs.recs)
             k_tiles_rec<LMAX, MODE, NSEG, false, GLD>
                 <<<a.grid, pass_threads(LMAX, MODE, NSEG, false), a.rec_smem, st>>>(

@@ -527,74 +527,93 @@ __device__ __forceinline__ float2 rec_grad_row(const Geo& g, const float4& ev, f
 }
 
 // Room of the fixed-point accumulator (see k_tiles_rec), in quanta.
-constexpr float kTopTerm = 0.99f * 0x1p24f;   // one event's largest term
+constexpr float kTopTerm = 0.99f * 0x1p24f;   // one event's largest term, of add4
 constexpr float kRoom = 0.99f * 0x1p32f;      // all the events of an item
 
-// How a pass over an item's events scatters: in one word a term (kWhole), or, for an
-// item whose rho' has a peak that events share (see k_tiles_rec), in two passes, the
-// terms' whole quanta (kHigh) and what these leave of them in units 2^-k (kLow; lo =
-// 2^(k - 149)).
-enum Phase : int { kWhole = 0, kHigh = 1, kLow = 2 };
-constexpr float kTopSplit = 0x1p22f;          // one event's largest term, in two passes
+// The fixed point of the item at hand, a copy for each warp in shared memory (the pixel
+// loops have no registers for it).
+struct RecScale {
+    float inv_q;        // 1 over the quantum of the terms P / D
+    float plain;        // the same for the plain scatter; infinite in a peaked item, which
+                        // it then takes no event of
+    float share;        // of the word's room, a group's
+    float cap;          // the most of it that one event may take
+};
 
-__device__ __forceinline__ void add_split(unsigned a, float p, float s, int phase, float lo)
+// How the terms of an event that the plain scatter does not take are added: not at all, by
+// float adds to the global A, or in quanta, by a conversion (up to 2^32 of them; add4's
+// arithmetic ends at 2^24).
+enum How : int { kNone, kFloat, kFixed };
+
+// An offset in [-1/2, 1/2) from the bits of an event's D: with it, a term is rounded to
+// the nearest quantum up or down in proportion, and terms that many events have alike
+// (1 / rho' at a pixel that is most of their D) keep their mean.
+__device__ __forceinline__ float dither(float D)
 {
-    const float t = __fmaf_rz(p, s, kFxMagic);          // bits: magic + floor(p s)
-    unsigned v = __float_as_uint(t) - kFxMagicBits;
-    if (phase == kLow) v = __float_as_uint(__fmaf_rn(p, s, kFxMagic - t) * lo);
+    return (float)((__float_as_uint(D) * 2654435761u) >> 8) * 0x1p-24f - 0.5f;
+}
+
+__device__ __forceinline__ void add_fixed(unsigned a, float p, float s, float u)
+{
+    const unsigned v = p > 0.0f ? __float2uint_rn(__fmaf_rn(p, s, u)) : 0u;
 #ifdef TSP_DEBUG_CHECKS
     if (!tsp_sh_ok(a, 4, 2)) return;
 #endif
     asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
-template <int TRAV>
-__device__ __noinline__ void rec_pass2_split(unsigned base, int n, unsigned tma, float s, int phase,
-                                             float lo)
+// Image pixel of a stored index (see Frame).
+__device__ __forceinline__ int frame_pixel(const Frame& f, int nz, int i)
 {
+    const int rr = i / f.stride, iy = f.oy + rr;
+    return iy * nz + f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0))) + i - rr * f.stride;
+}
+
+// The scatter of an event that the plain one does not take (see How): into the accumulator
+// (base: as rec_pass2), s = 1 / (D quantum), or to the global A, s = 1/D, each
+// pixel (idx: stored index of the row's origin) under its predicate; with MASK only where
+// rho' > 0 (as the flush does).  (Called from one place: a second caller costs the pixel
+// loops beside the call 6%.)
+template <int TRAV, bool MASK>
+__device__ __noinline__ void rec_scatter_slow(unsigned base, const Inst* I, const Frame* fp,
+                                              int idx, int la, int lb, int n, unsigned tma,
+                                              float s, float u, int how)
+{
+    const int pix = how == kFloat ? frame_pixel(*fp, I->g.nz, idx) : 0;
+    float* const A = I->A;
+    const float* const rhop = I->rhop;
+    auto add = [&](int q, float p) {
+        if (p != 0.0f && (!MASK || rhop[q] > 0.0f)) atomicAdd(A + q, p * s);
+    };
     for (int k = 1; k <= n; k += 2) {
         float x0, x1, x2, x3;
         tm_ld4(tma, x0, x1, x2, x3);
         tm_wait_ld();
-        add_split(base + (unsigned)(4 * pair_d0<TRAV>(k)), x0, s, phase, lo);
-        add_split(base + (unsigned)(4 * pair_d1<TRAV>(k)), x1, s, phase, lo);
-        add_split(base + (unsigned)(4 * pair_d0<TRAV>(k + 1)), x2, s, phase, lo);
-        add_split(base + (unsigned)(4 * pair_d1<TRAV>(k + 1)), x3, s, phase, lo);
+        const int d0 = pair_d0<TRAV>(k), d1 = pair_d1<TRAV>(k);
+        const int d2 = pair_d0<TRAV>(k + 1), d3 = pair_d1<TRAV>(k + 1);
+        if (how == kFixed) {
+            add_fixed(base + (unsigned)(4 * d0), x0, s, u);
+            add_fixed(base + (unsigned)(4 * d1), x1, s, u);
+            add_fixed(base + (unsigned)(4 * d2), x2, s, u);
+            add_fixed(base + (unsigned)(4 * d3), x3, s, u);
+        } else {
+            if (k <= la) add(pix + d0, x0);
+            if (k <= lb) add(pix + d1, x1);
+            if (k < la) add(pix + d2, x2);
+            if (k < lb) add(pix + d3, x3);
+        }
+        __syncwarp();
         tma += 4;
     }
 }
 
-// The scatter of an event whose terms the item's accumulator has no room for (see
-// k_tiles_rec): float adds to the global A, each pixel under its predicate; with
-// MASK only where rho' > 0 (as the flush does).
-template <int TRAV, bool MASK>
-__device__ __noinline__ void rec_scatter_global(float* A, const float* rhop, int pix, int la,
-                                                int lb, int n, unsigned tma, float invD)
-{
-    auto add = [&](int q, float p) {
-        if (p != 0.0f && (!MASK || rhop[q] > 0.0f)) atomicAdd(A + q, p * invD);
-    };
-    unsigned col = tma;
-    for (int k = 1; k <= n; k += 2) {
-        float x0, x1, x2, x3;
-        tm_ld4(col, x0, x1, x2, x3);
-        tm_wait_ld();
-        if (k <= la) add(pix + pair_d0<TRAV>(k), x0);
-        if (k <= lb) add(pix + pair_d1<TRAV>(k), x1);
-        if (k < la) add(pix + pair_d0<TRAV>(k + 1), x2);
-        if (k < lb) add(pix + pair_d1<TRAV>(k + 1), x3);
-        __syncwarp();
-        col += 4;
-    }
-}
-
 // The events first + grp, first + grp + ngroups, ... of an item, by one group
-// of G warps.  inv_q: 1 over the quantum of the fixed-point terms P / D.
+// of G warps.
 template <int TRAV, int LMAX, int MODE, int NSEG, bool GLD>
-__device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int first, int count,
-                                           int grp, int ngroups, int wig, int lane,
-                                           unsigned rp_addr, unsigned acc_off, unsigned slot,
-                                           float* part, BlockSums* bs, unsigned tma, float inv_q,
+__device__ __forceinline__ void rec_events(const Inst& I, const Frame* fp, const RecScale* sc,
+                                           int first, int count, int grp, int ngroups, int wig,
+                                           int lane, unsigned rp_addr, unsigned acc_off,
+                                           unsigned slot, float* part, BlockSums* bs, unsigned tma,
                                            const float* scr)
 {
     constexpr bool GRAD = MODE == kGrad;
@@ -602,6 +621,7 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
     const int G = I.G;
     int left = (count - grp + ngroups - 1) / ngroups;
     if (left <= 0) return;
+    first += grp;
     // the row block of a warp is rotated by its group (see process_event)
     int blk;
     if constexpr (NSEG == 1) {
@@ -614,12 +634,13 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
     }
     const float rowoff = (float)lane_row(blk * 32 + lane);
     const int rslot = NSEG == 1 ? blk * 32 + lane : (blk * 2 + (wig & 1)) * 32 + lane;
-    const uint2* rp = I.evs.recs + (size_t)(first + grp) * (32 * G) + rslot;
-    const float4* ep = I.evs.evc + (size_t)(first + grp) * kEvcFloat4;
+    // (GRAD: an index, not two pointers that step, which spills less)
+    const uint2* rp = I.evs.recs + (size_t)first * (32 * G) + rslot;
+    const float4* ep = I.evs.evc + (size_t)first * kEvcFloat4;
     rec_fetch(slot, rp, ep, lane);
+    const float inv_q = MODE == kLoglik ? 0.0f : sc->plain;
+    float room = MODE == kLoglik ? 0.0f : sc->share;
     unsigned used = 0;
-    float spent = 0.0f;
-    const float room = kRoom / (float)ngroups;
     double logD = 0.0, giz = 0.0, gil = 0.0;
     int parity = 0;
     for (;;) {
@@ -638,17 +659,23 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
         else if (MODE != kLoglik) ev.x = lds32(slot + 304u);
         __syncwarp();   // every lane has its values: the slot may be refilled
         if (--left > 0) {
-            rp += (size_t)ngroups * (32 * G);
-            ep += ngroups * kEvcFloat4;
-            rec_fetch(slot, rp, ep, lane);
+            if (GRAD) {
+                first += ngroups;
+                rec_fetch(slot, I.evs.recs + (size_t)first * (32 * G) + rslot,
+                          I.evs.evc + (size_t)first * kEvcFloat4, lane);
+            } else {
+                rp += (size_t)ngroups * (32 * G);
+                ep += ngroups * kEvcFloat4;
+                rec_fetch(slot, rp, ep, lane);
+            }
         }
         int n;
         float D;
         using Addr = typename std::conditional<GLD, unsigned long long, unsigned>::type;
         Addr rbase;
         if constexpr (GLD) {
-            const int rr = (int)(x.a.y + rowoff) - f.oy;
-            const int off = min(max(rr, 0), f.rh - 1) * (1 - kScrRows * f.stride) + (int)idx * kScrRows;
+            const int rr = (int)(x.a.y + rowoff) - fp->oy;
+            const int off = min(max(rr, 0), I.tl.RH - 1) * (1 - kScrRows * I.tl.RS) + (int)idx * kScrRows;
             rbase = (unsigned long long)(scr + off);
         } else {
             rbase = base;
@@ -671,40 +698,36 @@ __device__ __forceinline__ void rec_events(const Inst& I, const Frame& f, int fi
             parity ^= kMinWarps;
         }
         if (D > 0.0f) {
-            ++used;
-            if (MODE != kMlem && wig == 0 && lane == 0) logD += (double)logf(D);
             if (MODE != kLoglik) {
                 const float r = recip(D), s = r * inv_q, top = s * ev.x;
-                const int phase = bs->phase;
                 // (false for a NaN, and for a D that recip has no value of)
-                const bool fit = top > 0.0f && top <= (phase == kWhole ? kTopTerm : kTopSplit) &&
-                                 spent + top + 1.0f <= room;
-                if (GRAD && phase != kLow) {
+                float w = r;
+                if ((top > 0.0f) & (top <= room) & (top <= kTopTerm)) {
+                    // (some more than the bound: the rounding of the terms)
+                    room = fmaf(top, -1.0001f, room - 1.0f);
+                    const float q = s * 0x1p-149f;
+                    rec_pass2<TRAV>(base + acc_off, n, tma, make_float2(q, q));
+                } else {
+                    const float s1 = r * sc->inv_q, top1 = s1 * ev.x;
+                    const bool fit = top1 > 0.0f && top1 <= fminf(room, sc->cap);
+                    if (fit) room = fmaf(top1, -1.0001f, room - 1.0f);
+                    else w = 1.0f / D;
+                    rec_scatter_slow<TRAV, MODE == kMlem && !GLD>(
+                        base + acc_off, &I, fp, (int)idx, la, lb, n, tma, fit ? s1 : w, dither(D),
+                        fit ? kFixed : kFloat);
+                }
+                if (GRAD) {
                     // per-lane sums: the rows' terms of an event cancel to a small
                     // part of themselves, so they are added in double precision
-                    const float w = fit ? r : 1.0f / D;
                     giz += (double)(E.x * w);
                     gil += (double)(E.y * w);
                 }
-                if (fit) {
-                    spent += top + 1.0f;
-                    const float q = s * 0x1p-149f;
-                    if (phase == kWhole)
-                        rec_pass2<TRAV>(base + acc_off, n, tma, make_float2(q, q));
-                    else
-                        rec_pass2_split<TRAV>(base + acc_off, n, tma, s, phase, bs->lo);
-                } else if (phase != kLow) {
-                    const int rr = (int)idx / f.stride, col = (int)idx - rr * f.stride;
-                    const int iy = f.oy + rr;
-                    const int iz = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0))) + col;
-                    rec_scatter_global<TRAV, MODE == kMlem && !GLD>(I.A, I.rhop, iy * g.nz + iz, la,
-                                                                    lb, n, tma, 1.0f / D);
-                }
             }
+            ++used;
+            if (MODE != kMlem && wig == 0 && lane == 0) logD += (double)logf(D);
         }
         if (left == 0) break;
     }
-    if (bs->phase == kLow) return;      // counted in the first pass
     if (wig == 0 && lane == 0) {
         if (used) atomicAdd(&bs->used, (unsigned long long)used);
         if (MODE != kMlem) atomicAdd(&bs->logD, logD + used * (g.pshift * 0.69314718055994530942));
@@ -893,63 +916,65 @@ __device__ __forceinline__ void rec2_pass2(unsigned a0, unsigned a1, int n, unsi
     }
 }
 
-// In two passes (see Phase).
-static __device__ __noinline__ void rec2_pass2_split(unsigned a0, unsigned a1, int n, unsigned tma, float s,
-                                              int phase, float lo)
-{
-    for (int k = 1; k <= n; ++k) {
-        float x0, x1, x2, x3;
-        tm_ld4(tma, x0, x1, x2, x3);
-        tm_wait_ld();
-        add_split(a0 + 4u * k, x0, s, phase, lo);
-        add_split(a1 + 4u * k, x1, s, phase, lo);
-        add_split(a0 - 4u * (k - 1), x2, s, phase, lo);
-        add_split(a1 - 4u * (k - 1), x3, s, phase, lo);
-        tma += 4;
-    }
-}
-
-// The scatter of rows that the item's accumulator has no room for (see
-// rec_scatter_global); live: the lane's event is one of those.
+// The scatter of rows whose event rec2_pass2 does not take (see rec_scatter_slow; a0, a1:
+// addresses of the lane's rows' origins, i0, i1: their stored indexes).
 template <bool MASK>
-__device__ __noinline__ void rec2_scatter_global(float* A, const float* rhop, int p0, int p1,
-                                                 int la0, int lb0, int la1, int lb1, int n,
-                                                 unsigned tma, float invD, bool live)
+__device__ __noinline__ void rec2_scatter_slow(unsigned a0, unsigned a1, const Inst* I,
+                                               const Frame* fp, unsigned i0, unsigned i1,
+                                               unsigned n0, unsigned n1, int n, unsigned tma,
+                                               float s, float u, int how)
 {
+    const int p0 = how == kFloat ? frame_pixel(*fp, I->g.nz, (int)i0) : 0;
+    const int p1 = how == kFloat ? frame_pixel(*fp, I->g.nz, (int)i1) : 0;
+    float* const A = I->A;
+    const float* const rhop = I->rhop;
     auto add = [&](int q, float p) {
-        if (p != 0.0f && (!MASK || rhop[q] > 0.0f)) atomicAdd(A + q, p * invD);
+        if (p != 0.0f && (!MASK || rhop[q] > 0.0f)) atomicAdd(A + q, p * s);
     };
     for (int k = 1; k <= n; ++k) {
         float x0, x1, x2, x3;
         tm_ld4(tma, x0, x1, x2, x3);
         tm_wait_ld();
-        if (live) {
-            if (k <= la0) add(p0 + k, x0);
-            if (k <= la1) add(p1 + k, x1);
-            if (k <= lb0) add(p0 + 1 - k, x2);
-            if (k <= lb1) add(p1 + 1 - k, x3);
+        if (how == kFloat) {
+            if (k <= (int)(n0 & 0xff)) add(p0 + k, x0);
+            if (k <= (int)(n1 & 0xff)) add(p1 + k, x1);
+            if (k <= (int)(n0 >> 8)) add(p0 + 1 - k, x2);
+            if (k <= (int)(n1 >> 8)) add(p1 + 1 - k, x3);
+        } else if (how == kFixed) {
+            add_fixed(a0 + 4u * k, x0, s, u);
+            add_fixed(a1 + 4u * k, x1, s, u);
+            add_fixed(a0 - 4u * (k - 1), x2, s, u);
+            add_fixed(a1 - 4u * (k - 1), x3, s, u);
         }
         __syncwarp();
         tma += 4;
     }
 }
 
-// The events of an item for this warp: with G = 1 (up to 32 rows) a half warp
-// each, else groups of (G + 1) / 2 warps.
+// The groups of the two-row form: with G = 1 (up to 32 rows) a half warp an event, else
+// (G + 1) / 2 warps.  The first group of this warp, and their number.
+__device__ __forceinline__ int2 rec2_groups(int G, int warp)
+{
+    if (G == 1) return make_int2(2 * warp, 2 * kMaxWarps);
+    const int G2 = (G + 1) >> 1;
+    return make_int2(warp / G2, group_count(kMaxWarps, G2));
+}
+
+// The events of an item for this warp's groups.
 template <int MODE>
-__device__ __forceinline__ void rec2_events(const Inst& I, const Frame& f, int first, int count,
-                                            int warp, int lane, unsigned rp_addr, unsigned acc_off,
-                                            unsigned slot, float* s_part, BlockSums* bs,
-                                            unsigned tma, float inv_q)
+__device__ __forceinline__ void rec2_events(const Inst& I, const Frame* fp, const RecScale* sc,
+                                            int first, int count, int warp, int lane,
+                                            unsigned rp_addr, unsigned acc_off, unsigned slot,
+                                            float* s_part, BlockSums* bs, unsigned tma)
 {
     const Geo& g = I.g;
     const int G = I.G;
     const bool halves = G == 1;
     const int G2 = (G + 1) >> 1;
     const int wgrp = warp / G2, wig = warp - wgrp * G2;
-    const int ngroups = halves ? 2 * kMaxWarps : group_count(kMaxWarps, G2);
-    // group, and pair of rows (the row block of a warp is rotated by its group)
-    const int grp = halves ? 2 * warp + (lane >> 4) : wgrp;
+    const int2 gr = rec2_groups(G, warp);
+    const int ngroups = gr.y;
+    // (the row block of a warp is rotated by its group)
     int blk = wig + wgrp % G2;
     blk -= blk >= G2 ? G2 : 0;
     int p = halves ? lane & 15 : blk * 32 + lane;
@@ -957,11 +982,9 @@ __device__ __forceinline__ void rec2_events(const Inst& I, const Frame& f, int f
     const float2 rowoff = make_float2((float)-p, (float)(p + 1));
     p = min(p, 16 * G - 1);
     // events left of the warp's first group (the second half's may end one sooner)
-    const int lead = halves ? 2 * warp : wgrp;
-    if (!halves && wgrp >= ngroups) return;
-    int left = (count - lead + ngroups - 1) / ngroups;
+    int left = gr.x < ngroups ? (count - gr.x + ngroups - 1) / ngroups : 0;
     if (left <= 0) return;
-    int e = grp;
+    int e = gr.x + (halves ? lane >> 4 : 0);
     const uint4* const recs = reinterpret_cast<const uint4*>(I.evs.recs) + p;
     const float4* const evc = I.evs.evc;
     const int cl = halves ? lane & 15 : lane;
@@ -979,9 +1002,9 @@ __device__ __forceinline__ void rec2_events(const Inst& I, const Frame& f, int f
     fetch(e);
     float* const part = s_part + wgrp * 2 * kMinWarps;
     int parity = 0;
+    const float inv_q = MODE == kLoglik ? 0.0f : sc->plain;
+    float room = MODE == kLoglik ? 0.0f : sc->share;
     unsigned used = 0;
-    float spent = 0.0f;
-    const float room = kRoom / (float)ngroups;
     double logD = 0.0;
     for (;;) {
         RecIn x;
@@ -1015,70 +1038,112 @@ __device__ __forceinline__ void rec2_events(const Inst& I, const Frame& f, int f
             D = group_sum(D, G2, wig, lane, 1 + wgrp, part + parity);
             parity ^= kMinWarps;
         }
+        // (a second half beyond the list has no pixels: D = 0)
         const bool on = D > 0.0f;
+        if (MODE != kLoglik) {
+            const float r = recip(D), s = r * inv_q, top = s * pmax;
+            // (false for a NaN, and for a D that recip has no value of)
+            const bool fast = on & (top > 0.0f) & (top <= room) & (top <= kTopTerm);
+            if (!__any_sync(0xffffffffu, on & !fast)) {
+                // (some more than the bound: the rounding of the terms)
+                if (on) room = fmaf(top, -1.0001f, room - 1.0f);
+                rec2_pass2(a0 + acc_off, a1 + acc_off, kmax, tma, dup(on ? s * 0x1p-149f : 0.0f));
+            } else {
+                const float s1 = r * sc->inv_q, top1 = s1 * pmax;
+                const bool fit = on && top1 > 0.0f && top1 <= fminf(room, sc->cap);
+                if (fit) room = fmaf(top1, -1.0001f, room - 1.0f);
+                rec2_scatter_slow<MODE == kMlem>(a0 + acc_off, a1 + acc_off, &I, fp, i0, i1, n0, n1,
+                                                 kmax, tma, fit ? s1 : 1.0f / D, dither(D),
+                                                 !on ? kNone : fit ? kFixed : kFloat);
+            }
+        }
         if (on) {
             ++used;
             if (MODE != kMlem && (halves ? (lane & 15) == 0 : wig == 0 && lane == 0))
                 logD += (double)logf(D);
         }
-        if (MODE != kLoglik) {
-            const float r = recip(D), s = r * inv_q, top = s * pmax;
-            const int phase = bs->phase;
-            // (false for a NaN, and for a D that recip has no value of)
-            const bool fit = on && top > 0.0f && top <= (phase == kWhole ? kTopTerm : kTopSplit) &&
-                             spent + top + 1.0f <= room;
-            if (fit) spent += top + 1.0f;
-            if (__any_sync(0xffffffffu, fit)) {
-                if (phase == kWhole)
-                    rec2_pass2(a0 + acc_off, a1 + acc_off, kmax, tma,
-                               dup(fit ? s * 0x1p-149f : 0.0f));
-                else
-                    rec2_pass2_split(a0 + acc_off, a1 + acc_off, kmax, tma, fit ? s : 0.0f, phase,
-                                     bs->lo);
-            }
-            if (phase != kLow && __any_sync(0xffffffffu, on && !fit)) {
-                auto pix = [&](unsigned i) {
-                    const int rr = (int)i / f.stride, iy = f.oy + rr;
-                    return iy * g.nz + f.zbase +
-                           (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0))) + (int)i - rr * f.stride;
-                };
-                rec2_scatter_global<MODE == kMlem>(I.A, I.rhop, pix(i0), pix(i1), la0, lb0, la1,
-                                                   lb1, kmax, tma, 1.0f / D, on && !fit);
-            }
-        }
         if (left == 0) break;
     }
-    if (bs->phase == kLow) return;      // counted in the first pass
     if (used && (halves ? (lane & 15) == 0 : wig == 0 && lane == 0)) {
         atomicAdd(&bs->used, (unsigned long long)used);
         if (MODE != kMlem) atomicAdd(&bs->logD, logD + used * (g.pshift * 0.69314718055994530942));
     }
 }
 
-// Persistent tile kernel over window records.  Work
-// items, batches and the two-word accumulator are those of k_tiles; the first
-// item of a block is its index, later ones come from the queue, asked for while
-// an item is worked on.
+// An item's scale: a lane has the sum and the largest of rho' over its
+// band of rows (Inst::fx_*).  r, the most that an event of the item sees, is the largest
+// mean of rho' over a box of a window's size about the bands that hold window centres.
+// (Not the mean over the region: after a few updates most of it, outside
+// the body, is near 0, and the largest terms would lose four to five bits.)
+__device__ __forceinline__ void item_scale(const Inst& I, float2 band, int n, int ngroups, int lane,
+                                           RecScale* sc)
+{
+    const float peak =
+        __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(band.y))) * I.fx_peak;
+    float S = band.x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float v = __shfl_up_sync(0xffffffffu, S, o);
+        if (lane >= o) S += v;
+    }
+    const float hi = __shfl_sync(0xffffffffu, S, min(lane + I.fx_half, 31));
+    const float lo = __shfl_sync(0xffffffffu, S, max(lane - I.fx_half - 1, 0));
+    float b = lane > I.fx_half ? hi - lo : hi;
+    b = b > 0.0f && lane >= I.fx_first && lane <= I.fx_last ? b : 0.0f;
+    float r = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(b))) * I.fx_box;
+    const bool peaked = peak > 0.5f * r;
+    if (peaked) r = fmaxf(r, peak);
+    const float share = __fdividef(kRoom, (float)ngroups);
+    // an eighth of the share, or what each of a group's events can have, if that is more
+    const float cap = share * fminf(fmaxf(__fdividef((float)ngroups, (float)n), 0.125f), 1.0f);
+    // (peaked: the bits that leave events with a 2^-7.5th of the pixel's largest P, those at
+    // the edge of a window of 3 sigma, within the cap)
+    const int t = peaked ? min(18, (int)(__float_as_uint(cap) >> 23) - 127 - 8)
+                         : min(I.fx_bits, 30 - (32 - __clz(n - 1)));
+    const float v = __fdividef(r, I.fx_peak) * (float)(1 << t);
+    // a power of two, so that neither scaling by it nor the flush rounds (peaked: not above v,
+    // for the cap's sake); infinite for an image of no usable scale, whose events all
+    // take the float scatter
+    const unsigned up = peaked ? 0u : 0x7fffffu;
+    const float inv_q = v >= 1e-30f && v <= 1e30f
+                            ? __uint_as_float((__float_as_uint(v) + up) & 0x7f800000u)
+                            : INFINITY;
+    if (lane == 0) {
+        sc->inv_q = inv_q;
+        sc->plain = peaked ? INFINITY : inv_q;
+        sc->share = share;
+        sc->cap = cap;
+    }
+    __syncwarp();
+}
+
+// Persistent tile kernel over window records.  Work items and batches are those of
+// k_tiles; the first item of a block is its index, later ones come from the queue, asked
+// for while an item is worked on.
 //
 // The scatter sums P / D in fixed point, one word a pixel, with native integer adds
-// (a float add to shared memory is a compare-and-swap loop).  The quantum is the
-// item's: events of a window's mean rho' r have a largest term of fx_peak / r, and
-// this term, with the region's mean for r, takes t = fx_bits bits (fewer when the item
-// has so many events that 2^t of each would fill more than an eighth of the word).  What an event
-// really adds at most, its bound of P over D, is known before it is added: an event
-// above 2^24 quanta, or one that the group's share of the word has no room left for
-// (with D 1/8 of the estimate at least for all of them), is scattered by float adds
-// to global memory instead, so no sum can overflow.  Two words of the
-// responsibilities P rho' / D, as in k_tiles, need no such estimate, but twice the
+// (a float add to shared memory is a compare-and-swap loop).  The quantum is the item's:
+// the largest term of an event that sees a mean rho' of r, the most that one of the item's
+// does (item_scale), is fx_peak / r, and takes t = fx_bits (17 to 20) bits, or fewer to
+// leave the word room for four times the item's events (18 at 4000).  What an event
+// really adds at most, its bound of P over D, is known before it is added, so that no sum
+// can overflow: one above 2^24 quanta takes a slower loop (2% of the events at most, in
+// 50 updates of phantoms), and one that the group's share of the word has no room left for,
+// or an eighth of it, float adds to global memory (0.3%).
+//   A term is rounded to 2^-(t + 1) of the event's largest one, and over the cov events
+// of a pixel the rounding of A is 0.3 x 2^(2.2 - t) / sqrt(cov) of it (fx_bits), within
+// the 2^-22 of a term that its exponential and square root carry.  Two words of the
+// responsibilities P rho' / D, as in k_tiles, need no estimate, but twice the
 // adds and five more packed operations a pair: 1e7 events at 1 mm 34.3 -> 30.4 ms,
 // five updates of 2e5 at 1 mm 5.07 -> 4.29 ms, three of 3e5 at 2 mm 1.57 -> 1.36 ms.
 //
-// Where one pixel can take much of an event (rho' at the region's peak above half of
-// what an ordinary window sums to, or above 16 times the mean), the events' terms there
-// are equal multiples 1 / rho' of the quantum, far below the estimate, and their rounding
-// does not average out (a point source from a spike image: 4e-5 of the counts lost).  Such
-// an item takes two passes over its events, floor of the terms first, their remainder in
-// units 2^-19 or less of the quantum second (1e-7); ordinary images have none.
+// Where one pixel can hold much of an event's D (peaked: the region's largest rho' alone
+// would give half of r), the events' terms there are equal multiples 1 / rho' of the
+// quantum, and rounded to the nearest one they would all err alike (a point source from a
+// spike image: 4e-5 of the counts lost).  The events of such an item all take the
+// slower loop, whose rounding is up or down in proportion (dither), with 15 to 18 bits for
+// that pixel's terms: 0.4 x 2^-t / sqrt(events) = 2e-7 of their sum for 4000 events, 2e-8
+// for 6e5.  (Float adds would not do: they round the many equal terms alike as well.)
 //
 // GLD: the windows are too large to stage rho' beside the accumulator.  The block
 // writes the item's rho' region to its own part of global memory, transposed
@@ -1089,7 +1154,7 @@ __device__ __forceinline__ void rec2_events(const Inst& I, const Frame& f, int f
 // 28.1 ms now.
 template <int LMAX, int MODE, int NSEG, bool BATCH, bool GLD>
 __global__ void __launch_bounds__(pass_threads(LMAX, MODE, NSEG, BATCH), 1)
-k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ items, int n_items,
+k_tiles_rec(const __grid_constant__ Inst p, const Inst* __restrict__ table, const int4* __restrict__ items, int n_items,
             int* queue)
 {
     constexpr int kThreads = pass_threads(LMAX, MODE, NSEG, BATCH);
@@ -1105,7 +1170,9 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
     __shared__ BlockSums s_sums;
     __shared__ Inst s_inst;
     __shared__ unsigned s_tmem;
-    __shared__ float4 s_sum[kWarps];
+    __shared__ Frame s_frame;
+    __shared__ RecScale s_scale[kWarps];
+    __shared__ float2 s_band[kWarps];      // rho' of a 32nd of the region's rows: sum, largest
     const Inst& I = BATCH ? s_inst : p;
 
     const int tid = threadIdx.x, lane = tid & 31;
@@ -1118,6 +1185,7 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
 #endif
     // slots of warps that a group does not have stay zero (group_sum)
     for (int k = tid; k < kPartFloats; k += kThreads) s_part[k] = 0.0f;
+    if (tid < kWarps) s_band[tid] = make_float2(0.0f, 0.0f);
     int cur = -1, it = blockIdx.x, par = 0;
     bool fresh = true;
     tm_sync_threads();
@@ -1170,8 +1238,8 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
                 for (int k = tid; k < kPartFloats; k += kThreads) s_part[k] = 0.0f;
         }
         const Frame f = tile_frame(g, tl, item.x);
-        float sum = 0.0f, most = 0.0f;     // rho' over the region's pixels, and their number
-        int inside = 0;
+        float sum = 0.0f, most = 0.0f;     // rho' over the warp's band of rows
+        const int rpw = I.fx_rows;
         if constexpr (GLD) {
             if (MODE != kLoglik)
                 for (int k = tid; k < region; k += kThreads) s_cnt[k] = 0u;
@@ -1183,21 +1251,20 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
                 const bool row_in = iy >= 0 && iy < g.ny;
                 const int z0row = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0)));
                 const int w = (tl.RW + 3) >> 2, c1 = min(tl.RW, ((k & 3) + 1) * w);
+                float row = 0.0f;
 #pragma unroll 4
                 for (int cc = (k & 3) * w; cc < c1; ++cc) {
                     const int iz = z0row + cc;
                     float v = 0.0f;
-                    if (row_in && iz >= 0 && iz < g.nz) {
-                        v = __ldg(I.rhop + (size_t)iy * g.nz + iz);
-                        ++inside;
-                    }
+                    if (row_in && iz >= 0 && iz < g.nz) v = __ldg(I.rhop + (size_t)iy * g.nz + iz);
                     scr[cc * kScrRows + rr] = v;
-                    sum += v;
+                    row += v;
                     most = fmaxf(most, v);
                 }
+                if (MODE != kLoglik) atomicAdd(&s_band[rr / rpw].x, row);
             }
         } else {
-            for (int rr = warp; rr < tl.RH; rr += kWarps) {
+            for (int rr = warp * rpw; rr < min(tl.RH, (warp + 1) * rpw); ++rr) {
                 const int iy = f.oy + rr;
                 const bool row_in = iy >= 0 && iy < g.ny;
                 const int z0row = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0)));
@@ -1206,10 +1273,7 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
                     const int iz = z0row + cc;
                     float v = 0.0f;
                     // (the read-only path: loads may pass the stores of earlier columns)
-                    if (row_in && iz >= 0 && iz < g.nz) {
-                        v = __ldg(I.rhop + (size_t)iy * g.nz + iz);
-                        ++inside;
-                    }
+                    if (row_in && iz >= 0 && iz < g.nz) v = __ldg(I.rhop + (size_t)iy * g.nz + iz);
                     s_rp[rr * tl.RS + cc] = v;
                     if (MODE != kLoglik) s_cnt[rr * tl.RS + cc] = 0u;
                     sum += v;
@@ -1218,13 +1282,16 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
             }
         }
         if (MODE != kLoglik) {
-            sum = warp_sum(sum);
-            inside = __reduce_add_sync(0xffffffffu, inside);
             most = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(most)));
-            if (lane == 0) s_sum[warp] = make_float4(sum, (float)inside, most, 0.0f);
+            if constexpr (!GLD) sum = warp_sum(sum);
+            if (lane == 0) {
+                if constexpr (!GLD) s_band[warp].x = sum;
+                s_band[warp].y = most;
+            }
         }
         if (tid == 0) {
             s_item[par] = next;
+            s_frame = f;
             // pixels that the records left out, counted once a pass
             if (item.y == 0) {
                 s_sums.qclip += I.accum->rec_qclip;
@@ -1232,77 +1299,55 @@ k_tiles_rec(Inst p, const Inst* __restrict__ table, const int4* __restrict__ ite
             }
         }
         __syncthreads();
-        float inv_q = 0.0f;
+        const int G = I.G;
+        const int ngroups = group_count(kWarps, G);
+        const int grp = warp / G, wig = warp - grp * G;
+        RecScale* const sc = s_scale + warp;
         if (MODE != kLoglik) {
-            static_assert(kWarps == 32, "a lane a warp's sum");
-            const float4 part = s_sum[lane];
-            const float mean = warp_sum(part.x) / warp_sum(part.y);
-            const float peak = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(part.z)));
-            const bool split = peak > 16.0f * mean || peak * I.fx_peak > 0.5f * mean;
-            // (in two passes the low word has the precision, and 2^22 / 2^14 is the headroom)
-            const int t = min(split ? 14 : I.fx_bits, 29 - (32 - __clz(max(item.z - 1, 1))));
-            inv_q = mean / I.fx_peak * (float)(1 << t);
-            // (an image of no usable scale: every event takes the float scatter)
-            if (!(inv_q >= 1e-30f && inv_q <= 1e30f)) inv_q = INFINITY;
-            if (tid == 0) {
-                const int k = min(23, 31 - (32 - __clz(max(item.z - 1, 1))));
-                s_sums.phase = split ? kHigh : kWhole;
-                s_sums.quantum = 1.0f / inv_q;
-                s_sums.lo = __uint_as_float(1u << k);            // 2^(k - 149)
-                s_sums.lo_quantum = s_sums.quantum * exp2f((float)-k);
-            }
-            __syncthreads();
+            static_assert(kWarps == 32, "a lane a band");
+            const int groups = kTwo && two_rows_fit(G) ? rec2_groups(G, warp).y : ngroups;
+            item_scale(I, s_band[lane], item.z, groups, lane, sc);
         }
-        for (;;) {
-            const unsigned rp_addr = (unsigned)__cvta_generic_to_shared(s_rp);
-            const unsigned acc_off = GLD ? 0u : 4u * (unsigned)(region + 2 * kPadFloats);
-            const unsigned slot =
-                (unsigned)__cvta_generic_to_shared(smem + kPartFloats + warp * kSlot);
-            const int G = I.G;
-            const int ngroups = group_count(kWarps, G);
-            const int grp = warp / G, wig = warp - grp * G;
-            float* part = s_part + grp * 2 * kMinWarps;
+        const unsigned rp_addr = (unsigned)__cvta_generic_to_shared(s_rp);
+        const unsigned acc_off = GLD ? 0u : 4u * (unsigned)(region + 2 * kPadFloats);
+        const unsigned slot = (unsigned)__cvta_generic_to_shared(smem + kPartFloats + warp * kSlot);
+        float* part = s_part + grp * 2 * kMinWarps;
 #define TSP_REC_EVENTS(TRAV) \
-    rec_events<TRAV, LMAX, MODE, NSEG, GLD>(I, f, item.y, item.z, grp, ngroups, wig, lane, rp_addr, \
-                                            acc_off, slot, part, &s_sums, tma, inv_q, scr)
-            if (kTwo && two_rows_fit(G)) {
-                if constexpr (kTwo)
-                    rec2_events<MODE>(I, f, item.y, item.z, warp, lane, rp_addr, acc_off, slot,
-                                      s_part, &s_sums, tma, inv_q);
-            } else if (grp < ngroups) {
-                if (NSEG == 1)
-                    TSP_REC_EVENTS(kAlt);
-                else if ((wig & 1) == 0)
-                    TSP_REC_EVENTS(kPos);
-                else
-                    TSP_REC_EVENTS(kNeg);
-            }
+    rec_events<TRAV, LMAX, MODE, NSEG, GLD>(I, &s_frame, sc, item.y, item.z, grp, ngroups, wig, lane, \
+                                            rp_addr, acc_off, slot, part, &s_sums, tma, scr)
+        if (kTwo && two_rows_fit(G)) {
+            if constexpr (kTwo)
+                rec2_events<MODE>(I, &s_frame, sc, item.y, item.z, warp, lane, rp_addr, acc_off, slot,
+                                  s_part, &s_sums, tma);
+        } else if (grp < ngroups) {
+            if (NSEG == 1)
+                TSP_REC_EVENTS(kAlt);
+            else if ((wig & 1) == 0)
+                TSP_REC_EVENTS(kPos);
+            else
+                TSP_REC_EVENTS(kNeg);
+        }
 #undef TSP_REC_EVENTS
-            __syncthreads();
-            if (MODE == kLoglik) break;
-            {
-                const int phase = s_sums.phase;
-                const float quantum = phase == kLow ? s_sums.lo_quantum : s_sums.quantum;
-                for (int rr = warp; rr < tl.RH; rr += kWarps) {
-                    const int iy = f.oy + rr;
-                    if (iy < 0 || iy >= g.ny) continue;
-                    const int z0row = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(iy - f.Y0)));
-                    for (int cc = lane; cc < tl.RW; cc += 32) {
-                        const int iz = z0row + cc;
-                        const int k = rr * tl.RS + cc;
-                        float v = (float)s_cnt[k] * quantum;
-                        if (phase == kHigh) s_cnt[k] = 0u;
-                        // (the update is 0 where rho' = 0, whatever A holds)
-                        if (MODE == kMlem && !GLD && !(s_rp[k] > 0.0f)) v = 0.0f;
-                        if (iz >= 0 && iz < g.nz && v != 0.0f)
-                            atomicAdd(I.A + (size_t)iy * g.nz + iz, v);
-                    }
+        __syncthreads();
+        if (MODE != kLoglik) {
+            if (GLD && tid < kWarps) s_band[tid].x = 0.0f;
+            const float quantum = 1.0f / sc->inv_q;
+            const Frame fl = s_frame;
+            for (int rr = warp; rr < tl.RH; rr += kWarps) {
+                const int iy = fl.oy + rr;
+                if (iy < 0 || iy >= g.ny) continue;
+                const int z0row = fl.zbase + (int)rintf(__fmul_rn(fl.shear, (float)(iy - fl.Y0)));
+                for (int cc = lane; cc < tl.RW; cc += 32) {
+                    const int iz = z0row + cc;
+                    const int k = rr * tl.RS + cc;
+                    float v = (float)s_cnt[k] * quantum;
+                    // (the update is 0 where rho' = 0, whatever A holds)
+                    if (MODE == kMlem && !GLD && !(s_rp[k] > 0.0f)) v = 0.0f;
+                    if (iz >= 0 && iz < g.nz && v != 0.0f)
+                        atomicAdd(I.A + (size_t)iy * g.nz + iz, v);
                 }
-                __syncthreads();
-                if (phase != kHigh) break;
-                if (tid == 0) s_sums.phase = kLow;
-                __syncthreads();
             }
+            __syncthreads();
         }
         it = s_item[par];
         par ^= 1;
