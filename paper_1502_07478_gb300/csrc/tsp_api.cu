@@ -158,9 +158,17 @@ int plan(tsp_ctx* c)
     // of the general passes.  An item costs some 10 us beside its events (staging,
     // flush, the groups' unequal ends), as much as 20 events at 1 mm, so a list
     // is cut into as few tiles as the shared memory allows until a tile has some 64
-    // events: five updates of 2e5 events at 1 mm 4.18 -> 4.04 ms, one of 1e6 3.50 ->
-    // 3.35 ms, five of 2e4 at 5 mm 275 -> 262 us.
-    c->wide = !c->no_wide && dense_list(c, umax, hy, dy, dz) && records_fit(c);
+    // events: one update of 1e6 events at 1 mm 3.50 -> 3.35 ms.
+    // Only for items of 512 events and more: the wider the tiles, the more items reach a
+    // pixel, each with a float add to A, and with small items these adds are what the
+    // result's error is made of.  Five updates of 2e4 events at 5 mm, wide: 262 us and
+    // 6.0e-7 from 64 bits, narrow 275 us and 4.6e-7 (the general passes 5.1e-7); of 2e5
+    // at 1 mm 4.02 ms and 5.0e-7, narrow 4.15 and 4.7e-7 (general 4.8e-7).
+    // (In a batch the load of all members counts, those without a list yet as this one:
+    // 12 mixed members 18.5 ms by each one's own list, 17.4 so.)
+    const long long load = c->n_total * (1 + c->others_open) + c->others_n;
+    c->wide = !c->no_wide && dense_list(c, umax, hy, dy, dz) &&
+              load >= 512ll * c->sched.items_per_sm * c->num_sms && records_fit(c);
     while (TY > 4 && !fits(TY, RS)) TY -= 4;
     c->gld = 0;
     if (!fits(TY, RS) || RS - 1 - 2 * tl.HZ < 1) c->wide = false;

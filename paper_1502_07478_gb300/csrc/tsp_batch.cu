@@ -108,13 +108,20 @@ int check_index(tsp_batch* b, int i)
     return TSP_OK;
 }
 
-// What the other members' window records hold, before a list of member c is prepared:
-// the batch keeps to one context's share of the memory.
-void set_rec_others(const tsp_batch* b, tsp_ctx* c)
+// What the other members hold, before a list of member c is prepared: the batch's
+// window records keep to one context's share of the memory, and its items are cut by the
+// whole load.
+void set_others(const tsp_batch* b, tsp_ctx* c)
 {
     c->rec_others = 0;
-    for (const tsp_ctx* o : b->inst)
-        if (o != c) c->rec_others += o->rec_cap;
+    c->others_n = 0;
+    c->others_open = 0;
+    for (const tsp_ctx* o : b->inst) {
+        if (o == c) continue;
+        c->rec_others += o->rec_cap;
+        if (o->listed) c->others_n += o->n;
+        else c->others_open += 1;
+    }
 }
 
 int validate_schedule(tsp_batch* b, const tsp_schedule* s)
@@ -399,7 +406,7 @@ int apply_schedule(tsp_batch* b, const tsp_schedule* s, cudaStream_t st)
         if (replan) {
             int rc = plan(c);
             if (rc) return bfail_inst(b, i, rc);
-            set_rec_others(b, c);
+            set_others(b, c);
             if (c->listed && (rc = prepare_events(c, st))) return bfail_inst(b, i, rc);
         }
     }
@@ -539,7 +546,7 @@ int tsp_batch_upload_events(tsp_batch* b, int i, const float* zu, const float* z
     int rc = check_index(b, i);
     if (rc) return rc;
     b->dirty = true;
-    set_rec_others(b, b->inst[i]);
+    set_others(b, b->inst[i]);
     if ((rc = tsp_upload_events(b->inst[i], zu, zd, dl, n, on_device, stream)))
         return bfail_inst(b, i, rc);
     return TSP_OK;
@@ -558,7 +565,7 @@ int tsp_batch_set_sigma(tsp_batch* b, int i, double sigma_z, double sigma_dl, vo
     int rc = check_index(b, i);
     if (rc) return rc;
     b->dirty = true;
-    set_rec_others(b, b->inst[i]);
+    set_others(b, b->inst[i]);
     if ((rc = tsp_set_sigma(b->inst[i], sigma_z, sigma_dl, stream))) return bfail_inst(b, i, rc);
     return TSP_OK;
 }

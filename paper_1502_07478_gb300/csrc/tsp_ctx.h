@@ -63,7 +63,11 @@ struct tsp_ctx {
     // current upload are there
     unsigned char* recbuf = nullptr;
     size_t rec_cap = 0;               // bytes of recbuf
-    size_t rec_others = 0;            // of the other members of the batch
+    // the other members of the batch: their records' bytes, their lists' events, and how
+    // many have no list yet
+    size_t rec_others = 0;
+    long long others_n = 0;
+    int others_open = 0;
     size_t dev_mem = 0;               // the device's memory
     uint2* recs = nullptr;
     float4* evc = nullptr;
