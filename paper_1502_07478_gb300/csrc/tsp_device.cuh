@@ -535,6 +535,9 @@ __device__ __forceinline__ void row_acb(const Geo& g, const EvSig& es, const flo
 constexpr int kEvRowsMask = 0xFFFF;
 constexpr int kEvExact = 1 << 29;
 constexpr int kEvQPos = 1 << 30;
+// The event's bound of P over its window at once is not close: window records take it row
+// by row.
+constexpr int kEvLoose = 1 << 28;
 
 // A lower bound of Q = aCa + 2 oCb over every point of the event's window:
 // with y = y~ + Dy, |Dy| <= hy (window half-height) and |u| <= umax (largest
@@ -556,6 +559,36 @@ __device__ __forceinline__ bool q_positive_over_window(const Geo& g, const EvSig
     if (g.gR8 != 0.0f) q -= fabsf(g.gR8) * t * c2i * sqrtf(c2i) * (ymax + hy);
     return q > 1e-3f * lead;
 }
+
+// An upper bound of P over the event's window, for the fixed-point scatter of the passes
+// over window records.  With C^-1 positive definite
+// (aCb)^2 <= aCa bCb, and aCa = Q - 2 oCb, so
+//   (aCb)^2 / Q - bCb <= bCb |2 oCb| / Q <= cut^2 m / Qmin,
+// m a bound of |2 oCb| over the window's ellipse (Dy / hy)^2 + (u / umax)^2 <= 1 (of
+// l1 Dy/hy + l2 u/umax at most hypot(l1, l2)) and Qmin = min aCa - m.  slack is that
+// exponent's half, infinite where Qmin is not clearly positive.  The bound is 1.2 times
+// the largest value at the paper's 350 mm radius and 3 sigma, but 100 times and more at
+// 130 mm and 5 sigma.
+struct WindowBound {
+    float slack, q;
+};
+
+__device__ __forceinline__ WindowBound window_bound(const Geo& g, const EvSig& es, const float4& ev)
+{
+    const float t = fabsf(ev.z), c2i = ev.w;
+    const float hy = g.hy_coef * rsqrtf(c2i) * 1.001f + g.dy;
+    const float umax = sqrtf(g.cut2) * es.inv_sqrt_2iz + g.dz;
+    const float ymax = fabsf(ev.x) + hy;
+    const float gam = fabsf(g.gR8) * t * c2i * sqrtf(c2i);
+    const float lead = 2.0f * es.iz * g.R * g.R * c2i * c2i;
+    const float l1 = 4.0f * g.il * ymax * fmaf(2.0f * t, t, 1.0f) * hy * c2i + gam * hy;
+    const float l2 = 4.0f * es.iz * ymax * t * c2i * umax;
+    const float m = sqrtf(fmaf(l1, l1, l2 * l2)), q = lead - gam * ymax - m;
+    return WindowBound{q > 1e-3f * lead ? 0.5f * g.cut2 * m / q : INFINITY, q};
+}
+
+// Up to a factor of 4 the bound over the window will do (two of the fixed point's bits).
+__device__ __forceinline__ bool loose_bound(const WindowBound& b) { return !(b.slack < 1.386f); }
 
 // Bounding box of the event's window in pixel rows and columns, clipped to the
 // grid (App. B half-extents, widened by 1e-5 relative so that FP32 rounding

@@ -120,7 +120,8 @@ __global__ void k_setup(Geo g, Tiling tl, long long n, const float* __restrict__
             } else {
                 pix += cnt;
                 rw = make_int2(first, (last - first + 1) | (unsure ? 0 : kEvExact) |
-                                          (q_positive_over_window(g, es, ev) ? kEvQPos : 0));
+                                          (q_positive_over_window(g, es, ev) ? kEvQPos : 0) |
+                                          (loose_bound(window_bound(g, es, ev)) ? kEvLoose : 0));
                 k = fits ? (b * tl.tiles_y + ty) * tl.tiles_z + tz : nbins - 1;
                 if (!fits) ++outl;
             }

@@ -23,6 +23,7 @@
 #pragma once
 
 #include "tsp_mlem.cuh"
+#include "tsp_row_bound.h"
 
 namespace tsp {
 
@@ -30,37 +31,14 @@ namespace tsp {
 //   Q(u) = q0 + y (q1 + q2 y) + g1 y u,    aCb = a1 y u + Dy (b1 y + b2),
 //   C0 = log2K - hB Dy^2,   ksu = sqrt(log2(e) iz) of the event,
 // stored as float4 (y~, mid, q0, q1), (q2, g1, a1, b1), (b2, hB, log2K, ksu) and
-// (max, z~, t, c2i): an upper bound of P over the window, and the event's geometry,
-// which the gradient pass needs;
+// (max, z~, t, c2i): an upper bound of P over the window (window_bound, row_p_bound), and the
+// event's geometry, which the gradient pass needs;
 // mid is the middle row of the window (lane rows count outward from it).  P is
 // held times 2^-pshift (see Geo).
 constexpr int kEvcFloat4 = 4;
 
-// An upper bound of P over the event's window.  With C^-1 positive definite
-// (aCb)^2 <= aCa bCb, and aCa = Q - 2 oCb, so
-//   (aCb)^2 / Q - bCb <= bCb |2 oCb| / Q <= cut^2 m / Qmin,
-// m a bound of |2 oCb| over the window's ellipse (Dy / hy)^2 + (u / umax)^2 <= 1 (of
-// l1 Dy/hy + l2 u/umax at most hypot(l1, l2)) and Qmin = min aCa - m.  Infinite where
-// Qmin is not clearly positive.  The bound is some 1.2 times the largest value at
-// the paper's 350 mm radius, up to a few times at 130 mm.
-__device__ __forceinline__ float p_bound(const Geo& g, const EvSig& es, const float4& ev,
-                                         float log2K)
-{
-    const float t = fabsf(ev.z), c2i = ev.w;
-    const float hy = g.hy_coef * rsqrtf(c2i) * 1.001f + g.dy;
-    const float umax = sqrtf(g.cut2) * es.inv_sqrt_2iz + g.dz;
-    const float ymax = fabsf(ev.x) + hy;
-    const float gam = fabsf(g.gR8) * t * c2i * sqrtf(c2i);
-    const float lead = 2.0f * es.iz * g.R * g.R * c2i * c2i;
-    const float l1 = 4.0f * g.il * ymax * fmaf(2.0f * t, t, 1.0f) * hy * c2i + gam * hy;
-    const float l2 = 4.0f * es.iz * ymax * t * c2i * umax;
-    const float m = sqrtf(fmaf(l1, l1, l2 * l2)), q = lead - gam * ymax - m;
-    if (!(q > 1e-3f * lead)) return INFINITY;
-    return 1.001f * exp2f(fmaf(g.half_log2e * g.cut2, m / q, log2K)) * rsqrtf(q);
-}
-
 __device__ __forceinline__ void make_evc(const Geo& g, const EvSig& es, const float4& ev, int mid,
-                                         float4* __restrict__ out)
+                                         bool loose, float4* __restrict__ out)
 {
     const float yt = ev.x, t = ev.z, c2i = ev.w;
     const float il4 = 4.0f * g.il * c2i, iz2 = 2.0f * es.iz * c2i;
@@ -79,7 +57,12 @@ __device__ __forceinline__ void make_evc(const Geo& g, const EvSig& es, const fl
     out[1] = make_float4(q2, -2.0f * iz2 * t, -iz2, il4 * t);
     const float log2K = es.log2K - g.pshift;
     out[2] = make_float4(b2, g.half_log2e * il4, log2K, es.ksu);
-    out[3] = make_float4(p_bound(g, es, ev, log2K), ev.y, t, c2i);
+    const WindowBound b = window_bound(g, es, ev);
+    // (row by row from 0 in k_records, if it is loose)
+    out[3] = make_float4(loose ? 0.0f
+                               : 1.001f * exp2f(fmaf(2.0f * g.half_log2e, b.slack, log2K)) *
+                                     rsqrtf(b.q),
+                         ev.y, t, c2i);
 }
 
 // Lane rows count outward from the middle of the window (see event_rows).
@@ -111,8 +94,9 @@ k_records(Inst p, const int4* __restrict__ items, int n_items, uint2* __restrict
             const float4 ev = p.evs.geo[e];
             const int2 rws = p.evs.rows[e];
             make_evc(g, ev_sig(g, ev), ev, rws.x + (((rws.y & kEvRowsMask) - 1) >> 1),
-                     evc + (size_t)e * kEvcFloat4);
+                     (rws.y & kEvLoose) != 0, evc + (size_t)e * kEvcFloat4);
         }
+        __syncthreads();        // (the bounds below start at the coefficients' 0)
         for (int j0 = blockIdx.y * kRun; j0 < item.z; j0 += kRun * gridDim.y) {
             const int jn = min(kRun, item.z - j0);
             int j = 0, blk = warp;
@@ -153,6 +137,22 @@ k_records(Inst p, const int4* __restrict__ items, int n_items, uint2* __restrict
                     lb = sp.lim_odd >> 1;
                 }
                 const float u0 = sp.has ? fmaf((float)sp.o, g.dz, g.z0) - sp.c.zc : 0.0f;
+                if (evflags & kEvLoose) {
+                    float bound = 0.0f;
+                    if (sp.has) {
+                        float alpha, beta;
+                        row_acb(g, es, ev, sp.c, alpha, beta);
+                        const float ulo = fmaf((float)sp.c.lo, g.dz, g.z0) - sp.c.zc;
+                        bound = row_p_bound(sp.Qc, sp.gam2, alpha, beta, ulo,
+                                            fmaf((float)(sp.c.count - 1), g.dz, ulo),
+                                            es.log2K - g.pshift - g.half_log2e * sp.c.B0, es.iz,
+                                            g.half_log2e);
+                    }
+                    // (positive floats compare as their bits do)
+                    const unsigned most = __reduce_max_sync(0xffffffffu, __float_as_uint(bound));
+                    if (lane == 0)
+                        atomicMax(reinterpret_cast<unsigned*>(evc + (size_t)e * kEvcFloat4 + 3), most);
+                }
                 recs[((size_t)e * G + blk) * 32 + lane] =
                     make_uint2(__float_as_uint(u0), (unsigned)sp.sidx | (unsigned)la << 16 |
                                                         (unsigned)lb << 24);
