@@ -113,13 +113,16 @@ __device__ __forceinline__ void row_idle(RowK<SMEM>& r, RowG& rg)
 // A lane's share of an event's window: the chord of its row inside the frame
 // and the traversal of it.  With has = false the lane has no pixels.  o is the
 // image column the traversal starts at, sidx the stored index of that pixel
-// (an in-bounds index in any case), gidx the flat image index of an idle lane.
+// (an in-bounds index in any case; 32 bits in a staged region), gidx the flat image index
+// of an idle lane (GLD).
+template <bool SMEM>
 struct RowSpan {
     Chord c;
     float Qc, gam2;        // Q(u) = Qc + gam2 u along the chord
     bool has;
     int o, lim_odd, lim_even;
-    long long sidx, gidx;
+    typename std::conditional<SMEM, int, long long>::type sidx;
+    long long gidx;
 };
 
 // Span of lane row iy (valid_row = false for a lane without a row) for the
@@ -131,17 +134,16 @@ struct RowSpan {
 // The event preparation guarantees that every chord lies inside the frame;
 // the clamp keeps every access in bounds regardless (clipped pixels are
 // counted in lclip, pixels with Q <= 0 in qclip).
-template <int TRAV, int LMAX, bool SMEM>
-__device__ __forceinline__ RowSpan row_span(const Geo& g, const EvSig& es, const float4& ev,
+template <int TRAV, int LMAX, bool SMEM, bool GLD>
+__device__ __forceinline__ RowSpan<SMEM> row_span(const Geo& g, const EvSig& es, const float4& ev,
                                             const Ev64* ev64, int iy, bool valid_row, int evflags,
                                             const Frame& f, unsigned long long* qclip,
                                             unsigned long long* lclip)
 {
-    RowSpan r;
+    RowSpan<SMEM> r;
     Chord& c = r.c;
     c.y = c.Dy = c.B0 = c.zc = 0.0f;
     r.o = r.lim_odd = r.lim_even = 0;
-    r.gidx = 0;
     int lo = 0, hi = -1, z0row = 0;
     float Qc = 0.0f, gam2 = 0.0f;
     if (valid_row) {
@@ -206,11 +208,15 @@ __device__ __forceinline__ RowSpan row_span(const Geo& g, const EvSig& es, const
                             f.rw - 1);
         const long long lo_i = LMAX / 2;
         const long long hi_i = (long long)g.ny * g.nz + kPadFloats - LMAX / 2 - 1;
-        r.sidx = (long long)vr * f.stride + col;
-        if constexpr (!SMEM) r.sidx = min(max(r.sidx, lo_i), hi_i);
-        const int iyv = min(max(f.oy + vr, 0), g.ny - 1);
-        const int zv = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(f.oy + vr - f.Y0)));
-        r.gidx = min(max((long long)iyv * g.nz + min(max(zv + col, 0), g.nz - 1), lo_i), hi_i);
+        if constexpr (SMEM)
+            r.sidx = vr * f.stride + col;
+        else
+            r.sidx = min(max((long long)vr * f.stride + col, lo_i), hi_i);
+        if constexpr (GLD) {
+            const int iyv = min(max(f.oy + vr, 0), g.ny - 1);
+            const int zv = f.zbase + (int)rintf(__fmul_rn(f.shear, (float)(f.oy + vr - f.Y0)));
+            r.gidx = min(max((long long)iyv * g.nz + min(max(zv + col, 0), g.nz - 1), lo_i), hi_i);
+        }
         return r;
     }
     // The common origin is used only when it lies within 2 columns of the
@@ -249,8 +255,8 @@ __device__ __forceinline__ void make_row(const Geo& g, const EvSig& es, const fl
 {
     row_idle<GRAD, SMEM>(r, rg);
     const Frame f = *fp;
-    const RowSpan sp = row_span<TRAV, LMAX, SMEM>(g, es, ev, ev64, iy, valid_row, evflags, f,
-                                                  &bs->qclip, &bs->lclip);
+    const RowSpan<SMEM> sp = row_span<TRAV, LMAX, SMEM, GLD>(g, es, ev, ev64, iy, valid_row, evflags,
+                                                             f, &bs->qclip, &bs->lclip);
     const Chord& c = sp.c;
     if constexpr (SMEM)
         r.base = (unsigned)__cvta_generic_to_shared(base) + 4u * (unsigned)sp.sidx;

@@ -118,15 +118,15 @@ k_records(Inst p, const int4* __restrict__ items, int n_items, uint2* __restrict
                 const bool valid = ri >= 0 && ri < rws.y;
                 unsigned long long* qc = &p.accum->rec_qclip;
                 unsigned long long* lc = &p.accum->rec_lclip;
-                RowSpan sp;
+                RowSpan<true> sp;
                 if constexpr (NSEG == 1)
-                    sp = row_span<kAlt, LMAX, true>(g, es, ev, p.evs.geo64 + e, rws.x + ri, valid,
+                    sp = row_span<kAlt, LMAX, true, false>(g, es, ev, p.evs.geo64 + e, rws.x + ri, valid,
                                                     evflags, f, qc, lc);
                 else if ((blk & 1) == 0)
-                    sp = row_span<kPos, LMAX, true>(g, es, ev, p.evs.geo64 + e, rws.x + ri, valid,
+                    sp = row_span<kPos, LMAX, true, false>(g, es, ev, p.evs.geo64 + e, rws.x + ri, valid,
                                                     evflags, f, qc, lc);
                 else
-                    sp = row_span<kNeg, LMAX, true>(g, es, ev, p.evs.geo64 + e, rws.x + ri, valid,
+                    sp = row_span<kNeg, LMAX, true, false>(g, es, ev, p.evs.geo64 + e, rws.x + ri, valid,
                                                     evflags, f, qc, lc);
                 int la, lb;
                 if constexpr (NSEG == 1) {
