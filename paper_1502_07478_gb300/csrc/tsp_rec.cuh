@@ -1071,8 +1071,12 @@ __device__ __forceinline__ void rec2_events(const Inst& I, const Frame* fp, cons
 }
 
 // An item's scale: a lane has the sum and the largest of rho' over its
-// band of rows (Inst::fx_*).  r, the most that an event of the item sees, is the largest
-// mean of rho' over a box of a window's size about the bands that hold window centres.
+// band of rows (Inst::fx_*).  r, what an event of the item sees, is the mean of rho' over
+// a box of a window's size about the bands that hold window centres, averaged with itself
+// for weight, as events are distributed.  (With the largest mean in its place the items
+// at the body's edge had no room for their events from the third update on, and some
+// thousands of float adds in a few items held the whole pass up: 5e6 events at 1 mm
+// 15.1 -> 20 to 24 ms.)
 // (Not the mean over the region: after a few updates most of it, outside
 // the body, is near 0, and the largest terms would lose four to five bits.)
 __device__ __forceinline__ void item_scale(const Inst& I, float2 band, int n, int ngroups, int lane,
@@ -1090,7 +1094,9 @@ __device__ __forceinline__ void item_scale(const Inst& I, float2 band, int n, in
     const float lo = __shfl_sync(0xffffffffu, S, max(lane - I.fx_half - 1, 0));
     float b = lane > I.fx_half ? hi - lo : hi;
     b = b > 0.0f && lane >= I.fx_first && lane <= I.fx_last ? b : 0.0f;
-    float r = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(b))) * I.fx_box;
+    const float m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(b)));
+    const float x = m > 0.0f ? __fdividef(b, m) : 0.0f;
+    float r = m > 0.0f ? __fdividef(m * warp_sum(x * x), warp_sum(x)) * I.fx_box : 0.0f;
     const bool peaked = peak > 0.5f * r;
     if (peaked) r = fmaxf(r, peak);
     const float share = __fdividef(kRoom, (float)ngroups);
@@ -1099,7 +1105,7 @@ __device__ __forceinline__ void item_scale(const Inst& I, float2 band, int n, in
     // (peaked: the bits that leave events with a 2^-7.5th of the pixel's largest P, those at
     // the edge of a window of 3 sigma, within the cap)
     const int t = peaked ? min(18, (int)(__float_as_uint(cap) >> 23) - 127 - 8)
-                         : min(I.fx_bits, 30 - (32 - __clz(n - 1)));
+                         : min(I.fx_bits, 29 - (32 - __clz(n - 1)));
     const float v = __fdividef(r, I.fx_peak) * (float)(1 << t);
     // a power of two, so that neither scaling by it nor the flush rounds (peaked: not above v,
     // for the cap's sake); infinite for an image of no usable scale, whose events all
@@ -1123,9 +1129,9 @@ __device__ __forceinline__ void item_scale(const Inst& I, float2 band, int n, in
 //
 // The scatter sums P / D in fixed point, one word a pixel, with native integer adds
 // (a float add to shared memory is a compare-and-swap loop).  The quantum is the item's:
-// the largest term of an event that sees a mean rho' of r, the most that one of the item's
-// does (item_scale), is fx_peak / r, and takes t = fx_bits (17 to 20) bits, or fewer to
-// leave the word room for four times the item's events (18 at 4000).  What an event
+// the largest term of an event that sees a mean rho' of r, as the item's events do on the
+// average (item_scale), is fx_peak / r, and takes t = fx_bits (17 to 20) bits, or fewer to
+// leave the word room for eight times the item's events (17 at 4000).  What an event
 // really adds at most, its bound of P over D, is known before it is added, so that no sum
 // can overflow: one above 2^24 quanta takes a slower loop (2% of the events at most, in
 // 50 updates of phantoms), and one that the group's share of the word has no room left for,
