@@ -330,6 +330,18 @@ PassArgs pass_args(tsp_ctx* c)
     return a;
 }
 
+// Whether the gradient pass of a list goes without its records: with fewer than two events
+// an item for each event group a pass is a few single events' latency, which is shorter
+// in the general pass (2e4 events at 5 mm 131 us, 154 over records; 6e4 215 and 217; with
+// two warps an event, at 2 mm, items always have more).  The tiles are the general passes'
+// (not wide).
+static bool grad_without_records(const tsp_ctx* c)
+{
+    return c->rec && !c->wide && !c->gld &&
+           item_events(c->outlier_first, c->sched.items_per_sm, c->num_sms) <
+               2 * group_count(kMaxWarps, c->G);
+}
+
 // Prepare the uploaded raw events: Eq. 2, windows, binning, work items.
 // Event preparation in three steps, so that an upload can be streamed in
 // chunks: clear the bin histogram and counters; per chunk, Eq. 2, windows and
@@ -903,7 +915,8 @@ int tsp_loglik_grad(tsp_ctx* c, double* L_out, float* g_rho, int g_on_device, do
     int rc = refresh_rhop(c, st);   // clears the accumulators, sums s rho
     if (rc) return rc;
     const bool grad = g_rho || g_sigma;
-    const PassArgs a = pass_args(c);
+    PassArgs a = pass_args(c);
+    if (grad && grad_without_records(c)) a.evs.recs = nullptr;
     TSP_CUDA(c, launch_pass(c->lmax, grad ? kGrad : kLoglik, a, st));
     c->launches += pass_launches(c);
     if (grad) {

@@ -120,3 +120,26 @@ def test_small_radius_and_wide_cut(cut):
     m = ref > 0.01 * ref.max()
     assert st["n_used"] == rs.n_used
     assert np.max(np.abs(img[m] - ref[m]) / ref[m]) <= 1e-4
+
+
+@pytest.mark.parametrize("ny,nz", [(140, 100), (350, 250)])
+@pytest.mark.parametrize("n", [20_000, 100_000])
+def test_gradient_of_short_and_longer_items(ny, nz, n):
+    """At 5 mm a list of 2e4 has fewer than two events an item and group: its gradient goes
+    without the records, that of 1e5 over them; at 2 mm both do."""
+    from paper_1502_07478_gb300 import Recon
+    w = replace(make_workload("small_5mm"), ny=ny, nz=nz, n_events=n)
+    ev = w.events()
+    r = Recon.from_workload(w)
+    r.upload_events(*ev)
+    r.iterate(2)
+    rho = r.read_image().cpu().numpy().astype(np.float64)
+    L, g, gs = r.loglik_grad()
+    st = r.stats()
+    r.close()
+    Lref, gref, gsref = oracle.loglik_grad(Setup.from_workload(w), ev, rho)
+    gref = np.asarray(gref).reshape(ny, nz)
+    assert st["n_clipped"] == 0
+    assert L == pytest.approx(Lref, rel=1e-6)
+    assert np.linalg.norm(g.cpu().numpy() - gref) <= 1e-4 * np.linalg.norm(gref)
+    np.testing.assert_allclose(gs, gsref, rtol=1e-3)
