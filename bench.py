@@ -60,16 +60,16 @@ SFU_RSQRT_PER_SM_CLK = 15.9
 SFU_EX2_PER_SM_CLK = 31.7
 FMA_PER_SM_CLK = 128
 FMA_OPS_PER_PIXEL = 17
-# DRAM bytes per event of one MLEM tile pass (dram__bytes_read.sum +
+# DRAM bytes per event of one MLEM tile pass over window records (dram__bytes_read.sum +
 # dram__bytes_write.sum of one ncu-captured launch over 1e6 events of the
-# 1 mm workload); the traffic grows with the events.
-TILE_PASS_DRAM_B_PER_EVENT = 47.6
+# 1 mm workload: 1.09 KB of records an event); the traffic grows with the events.
+TILE_PASS_DRAM_B_PER_EVENT = 1096.6
 # The same for the accumulator-only tile pass of the 0.5 mm stress workload
 # (one launch over its first 1e6 events; rho' re-read through L1/L2).
 GLD_PASS_DRAM_B_PER_EVENT = 66.0
 # Warp instructions issued per in-window pixel evaluation (smsp__inst_executed.sum
 # / W of the same captures): the pass is issue-bound, so this is its tracked cost.
-TILE_PASS_WARP_INST_PER_EVAL = 1.06
+TILE_PASS_WARP_INST_PER_EVAL = 0.660
 GLD_PASS_WARP_INST_PER_EVAL = 1.16
 
 
@@ -722,13 +722,15 @@ def main():
     # evaluations per launch (exact count from the event preparation)
     W = st1["n_window"]
     t_pass = float(np.mean(pass_ms)) / 1e3 if pass_ms else None
+    # (the passes over window records run on lists of 64 events over a pixel and more)
+    dense = W >= 64 * workload.ny * workload.nz
+    measured = workload.name == "paper_1mm" and args.variant == "tiles" and dense
     roofline = roofline_dict(
         W, t_pass, roofline_basis(local),
-        ("k_tiles" if args.variant == "tiles" else "k_thread_events") + " (MLEM pass, per launch)",
-        traffic=(TILE_PASS_DRAM_B_PER_EVENT * n
-                 if workload.name == "paper_1mm" and args.variant == "tiles" else None),
-        inst_per_eval=(TILE_PASS_WARP_INST_PER_EVAL
-                       if workload.name == "paper_1mm" and args.variant == "tiles" else None))
+        ("k_thread_events" if args.variant != "tiles" else "k_tiles_rec" if dense else "k_tiles") +
+        " (MLEM pass, per launch)",
+        traffic=TILE_PASS_DRAM_B_PER_EVENT * n if measured else None,
+        inst_per_eval=TILE_PASS_WARP_INST_PER_EVAL if measured else None)
 
     e2e = None
     if not args.no_e2e:

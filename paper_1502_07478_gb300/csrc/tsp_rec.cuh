@@ -1133,9 +1133,9 @@ __device__ __forceinline__ void item_scale(const Inst& I, float2 band, int n, in
 // average (item_scale), is fx_peak / r, and takes t = fx_bits (17 to 20) bits, or fewer to
 // leave the word room for eight times the item's events (17 at 4000).  What an event
 // really adds at most, its bound of P over D, is known before it is added, so that no sum
-// can overflow: one above 2^24 quanta takes a slower loop (2% of the events at most, in
+// can overflow: one above 2^24 quanta takes a slower loop (up to 2.4% of the events in
 // 50 updates of phantoms), and one that the group's share of the word has no room left for,
-// or an eighth of it, float adds to global memory (0.3%).
+// or an eighth of it, float adds to global memory (up to 0.8%).
 //   A term is rounded to 2^-(t + 1) of the event's largest one, and over the cov events
 // of a pixel the rounding of A is 0.3 x 2^(2.2 - t) / sqrt(cov) of it (fx_bits), within
 // the 2^-22 of a term that its exponential and square root carry.  Two words of the
