@@ -89,7 +89,7 @@ def test_first_upload_does_not_wait_for_other_streams():
     from paper_1502_07478_gb300 import Recon
     w = make_workload("small_5mm", n_events=20_000)
     ev = [torch.from_numpy(x).cuda() for x in w.events()]
-    for _ in range(2):                      # (the first round loads the kernels)
+    for _ in range(2):                      # (the first time loads the kernels)
         r = Recon.from_workload(w)
         side, mine = torch.cuda.Stream(), torch.cuda.Stream()
         torch.cuda.synchronize()
